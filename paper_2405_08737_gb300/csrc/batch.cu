@@ -135,7 +135,7 @@ __global__ void batch_plan(BatchDev b) {
     int nchunk = (n + 1 + len - 1) / len;
     if (nchunk > kMaxSplit) nchunk = kMaxSplit;
     // the prep rows and the partials must fit the system's workspace
-    while (nchunk > 1 && (3 + 2 * (int64_t)nchunk) * row * 2 > s.part_doubles) --nchunk;
+    while (nchunk > 1 && (2 + 2 * (int64_t)nchunk) * row * 2 > s.part_doubles) --nchunk;
     len = (n + 1 + nchunk - 1) / nchunk;
     nchunk = (n + 1 + len - 1) / len;
     s.n = n;
@@ -199,12 +199,12 @@ __global__ void __launch_bounds__(256) batch_rows(BatchDev b) {
     } else if (OP == kOpPrep) {
       const int64_t row = (int64_t)(n + 1) * MM;
       const WeightsView w{s.wbar, s.band, s.band_w};
-      rk::history_prep_entry(MM, n, lin, s.Sl, s.Sg, w, s.part, s.part + 2 * row, s.part + 4 * row);
+      rk::history_prep_entry(MM, n, lin, s.Sl, s.Sg, w, s.part, s.part + 2 * row);
     } else {  // kOpReduce: both s of entry lin
       const int64_t row = (int64_t)(n + 1) * MM;
       double2* out = reinterpret_cast<double2*>(s.I);
       if (s.nchunk > 1) {
-        const double2* part = reinterpret_cast<const double2*>(s.part + 6 * row);
+        const double2* part = reinterpret_cast<const double2*>(s.part + 4 * row);
         ok &= rk::history_reduce_entry(2 * row, s.nchunk, lin, part, out);
         ok &= rk::history_reduce_entry(2 * row, s.nchunk, lin + row, part, out);
       } else {
@@ -246,8 +246,7 @@ __global__ void __launch_bounds__(BS) batch_history(BatchDev b) {
     const int64_t lin = (int64_t)xb * BS + threadIdx.x;
     if (lin < row) {
       rk::PartialArgs p{s.M, MM, n, s.chunk_len, s.L, s.R, s.Sl, s.Sg, s.part, s.part + 2 * row,
-                        s.part + 4 * row, WeightsView{s.wbar, s.band, s.band_w},
-                        s.nchunk == 1 ? s.I : s.part + 6 * row};
+                        WeightsView{s.wbar, s.band, s.band_w}, s.nchunk == 1 ? s.I : s.part + 4 * row};
       rk::history_partial_entry(p, lin, chunk);
     }
   }

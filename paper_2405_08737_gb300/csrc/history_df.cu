@@ -5,8 +5,15 @@
 //   I^<(n,c) = sum_m A1[m] G^<(m,c) + sum_{m<=c} B^<[m] G^A(m,c),
 //   I^>(n,c) = sum_m A1[m] G^>(m,c) + sum_{m<=c} B^>[m] G^A(m,c),
 // with A1[m] = w_{n,m} (S^> - S^<)[m], B^s[m] = wbar_m S^s[m] (w_{c,m} S^s[m]
-// in the band m > c - K - 1), G^> = G^< + R below and on the diagonal, and
-// the symmetries G^s(m,c) = -G^s(c,m)^+ (m < c), G^A(m,c) = R(c,m)^+.
+// in the band m > c - K - 1).  With the planes PL(m,c) = L(m,c), Q(m,c) =
+// R(m,c) below and on the diagonal and PL = -L(c,m)^+, Q = -R(c,m)^+ above it
+// (G^< = PL, G^> = PL + Q, G^A = -Q for m < c), and with the part of the
+// settled points that cancels between the terms left out (w_{n,m} = wbar_m
+// there; see history_partial_entry), two products per point are summed:
+//   I^<       = sum_m A1[m] PL(m,c) - sum_{m<c, settled} B^<[m] Q(m,c) + band^<,
+//   I^> - I^< = sum_{m > c - K - 1} A1[m] Q(m,c) + band^> - band^<.
+// (The slice n = 511, M = 16 took 6.57 ms with all the products, 4.63 ms with
+// these.)
 //
 // GB300 issues 64 FP32 operations per FP64 operation, so a complex
 // multiply-add done as four double-float products (each hi*hi, its FMA
@@ -49,8 +56,7 @@ struct DfArgs {
   const double* Sl;             // raw row n (band points of term 2)
   const double* Sg;
   const float4* A1;             // double-float rows [n+1][M][M]
-  const float4* Bl;
-  const float4* Bg;
+  const float4* NB;             // -wbar S^<
   WeightsView w;
   double* dst;                  // partials [chunk][2][n+1][MM] or the output
 };
@@ -60,12 +66,10 @@ using df::c2f;
 using df::cconj;
 using df::cmac;
 using df::cneg;
-__device__ __forceinline__ float4 cadd(float4 a, float4 b) { return df::cadd4(a, b); }
 
 __global__ void __launch_bounds__(256) history_df_prep(int MM, int n, const double* __restrict__ Sl,
                                                        const double* __restrict__ Sg, WeightsView w,
-                                                       float4* __restrict__ A1, float4* __restrict__ Bl,
-                                                       float4* __restrict__ Bg) {
+                                                       float4* __restrict__ A1, float4* __restrict__ NB) {
   const int64_t total = (int64_t)(n + 1) * MM;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -74,8 +78,73 @@ __global__ void __launch_bounds__(256) history_df_prep(int MM, int n, const doub
     const double2 l = reinterpret_cast<const double2*>(Sl)[e];
     const double2 g = reinterpret_cast<const double2*>(Sg)[e];
     A1[e] = c2f(make_double2(wn * (g.x - l.x), wn * (g.y - l.y)));
-    Bl[e] = c2f(make_double2(wb * l.x, wb * l.y));
-    Bg[e] = c2f(make_double2(wb * g.x, wb * g.y));
+    NB[e] = c2f(make_double2(-wb * l.x, -wb * l.y));
+  }
+}
+
+// One thread's sums for its values of a: I^< and D = I^> - I^< (re, im).
+struct Sums {
+  Acc lr[kNA], li[kNA], dr[kNA], di[kNA];
+  __device__ __forceinline__ Sums() {
+#pragma unroll
+    for (int k = 0; k < kNA; ++k) lr[k] = li[k] = dr[k] = di[k] = Acc{0.f, 0.f};
+  }
+};
+
+// History point m, orbital x of column c's entry b: pl, q are the planes'
+// values, s1 and nb the operand rows of the thread's first a at stride `as`.
+__device__ __forceinline__ void point(const DfArgs& p, Sums& t, int m, int c, int a0, int na, int x, int b, float4 pl,
+                                      float4 q, const float4* s1, const float4* nb, int as) {
+  if (m <= c - p.w.band_w) {  // settled: the same for I^< and I^>
+#pragma unroll
+    for (int k = 0; k < kNA; ++k) {
+      if (k < na) {
+        cmac(t.lr[k], t.li[k], s1[(int64_t)k * as], pl);
+        cmac(t.lr[k], t.li[k], nb[(int64_t)k * as], q);
+      }
+    }
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < kNA; ++k) {
+    if (k < na) {
+      const float4 v = s1[(int64_t)k * as];
+      cmac(t.lr[k], t.li[k], v, pl);
+      cmac(t.dr[k], t.di[k], v, q);
+    }
+  }
+  if (m > c) return;
+  // term 2 in the band, with the exact weight: w_{c,m} S^s G^A
+  const int M = p.M;
+  const double wcm = p.w.at(c, m);
+  float4 ga = cneg(q);
+  if (m == c)  // G^A(c,c)_xb = conj(R(c,c)_bx)
+    ga = cconj(c2f(reinterpret_cast<const double2*>(p.R)[tri(c, c) * p.MM + b * M + x]));
+  const double2* sl = reinterpret_cast<const double2*>(p.Sl) + ((int64_t)m * M + a0) * M + x;
+  const double2* sg = reinterpret_cast<const double2*>(p.Sg) + ((int64_t)m * M + a0) * M + x;
+#pragma unroll
+  for (int k = 0; k < kNA; ++k) {
+    if (k < na) {
+      const double2 vl = sl[(int64_t)k * M], vg = sg[(int64_t)k * M];
+      cmac(t.lr[k], t.li[k], c2f(make_double2(wcm * vl.x, wcm * vl.y)), ga);
+      cmac(t.dr[k], t.di[k], c2f(make_double2(wcm * (vg.x - vl.x), wcm * (vg.y - vl.y))), ga);
+    }
+  }
+}
+
+__device__ __forceinline__ void store_sums(const DfArgs& p, const Sums& t, int chunk, int c, int a0, int na, int b) {
+  double2* d = reinterpret_cast<double2*>(p.dst);
+  const int64_t stride_s = (int64_t)(p.n + 1) * p.MM;
+  const int64_t base = (int64_t)chunk * 2 * stride_s + (int64_t)c * p.MM + b;
+#pragma unroll
+  for (int k = 0; k < kNA; ++k) {
+    if (k < na) {
+      const int64_t e = base + (int64_t)(a0 + k) * p.M;
+      const double2 l = make_double2((double)t.lr[k].s + (double)t.lr[k].c, (double)t.li[k].s + (double)t.li[k].c);
+      d[e] = l;
+      d[e + stride_s] = make_double2(l.x + ((double)t.dr[k].s + (double)t.dr[k].c),
+                                     l.y + ((double)t.di[k].s + (double)t.di[k].c));
+    }
   }
 }
 
@@ -93,79 +162,31 @@ __global__ void __launch_bounds__(kDfBlock) history_df_partial(DfArgs p) {
   const int chunk = blockIdx.y;
   const int m0 = chunk * p.chunk_len;
   const int m1 = min(n + 1, m0 + p.chunk_len);
-  const int band_lo = c - p.w.band_w + 1;  // m >= band_lo: w_{c,m} from the band
 
-  Acc lr[kNA], li[kNA], gr[kNA], gi[kNA];  // I^< and I^> (re, im)
-#pragma unroll
-  for (int k = 0; k < kNA; ++k) lr[k] = li[k] = gr[k] = gi[k] = Acc{0.f, 0.f};
+  Sums sum;
   const double2* L = reinterpret_cast<const double2*>(p.L);
   const double2* R = reinterpret_cast<const double2*>(p.R);
 
   for (int m = m0; m < m1; ++m) {
-    const bool below = m > c, diag = m == c;
-    const bool band = !below && m >= band_lo;
-    const double wcm = band ? p.w.at(c, m) : 0.0;
-    // this thread's column b of G(m,c): block (m,c) row x for m >= c; block
-    // (c,m) row b, transposed and conjugated, for m < c
-    const int64_t blk = below || diag ? tri(m, c) * MM : tri(c, m) * MM;
+    // this thread's column b of the planes at (m,c): block (m,c) row x for
+    // m >= c; block (c,m) row b, transposed, conjugated and negated, for m < c
+    const bool direct = m >= c;
+    const int64_t blk = direct ? tri(m, c) * MM : tri(c, m) * MM;
+    const float4* a1 = p.A1 + ((int64_t)m * M + a0) * M;
+    const float4* nb = p.NB + ((int64_t)m * M + a0) * M;
     for (int x = 0; x < M; ++x) {
-      float4 gl, gs, ga;
-      if (below || diag) {
-        gl = c2f(L[blk + x * M + b]);
-        const float4 rr = c2f(R[blk + x * M + b]);
-        gs = cadd(gl, rr);                                 // G^>(m,c) = L + R
-        ga = diag ? cconj(c2f(R[blk + b * M + x])) : rr;   // G^A(c,c)_xb = conj(R(c,c)_bx)
+      float4 pl, q;
+      if (direct) {
+        pl = c2f(L[blk + x * M + b]);
+        q = c2f(R[blk + x * M + b]);
       } else {
-        const float4 l = c2f(L[blk + b * M + x]), rr = c2f(R[blk + b * M + x]);
-        gl = cneg(cconj(l));                               // G^<(m,c)_xb = -conj(L(c,m)_bx)
-        gs = cneg(cconj(cadd(l, rr)));                     // G^>(m,c)_xb = -conj((L+R)(c,m)_bx)
-        ga = cconj(rr);                                    // G^A(m,c)_xb = conj(R(c,m)_bx)
+        pl = cneg(cconj(c2f(L[blk + b * M + x])));
+        q = cneg(cconj(c2f(R[blk + b * M + x])));
       }
-      const float4* a1 = p.A1 + ((int64_t)m * M + a0) * M + x;
-#pragma unroll
-      for (int k = 0; k < kNA; ++k) {
-        if (k < na) {
-          const float4 s1 = a1[(int64_t)k * M];
-          cmac(lr[k], li[k], s1, gl);
-          cmac(gr[k], gi[k], s1, gs);
-        }
-      }
-      if (below) continue;
-      if (!band) {
-        const float4* bl = p.Bl + ((int64_t)m * M + a0) * M + x;
-        const float4* bg = p.Bg + ((int64_t)m * M + a0) * M + x;
-#pragma unroll
-        for (int k = 0; k < kNA; ++k) {
-          if (k < na) {
-            cmac(lr[k], li[k], bl[(int64_t)k * M], ga);
-            cmac(gr[k], gi[k], bg[(int64_t)k * M], ga);
-          }
-        }
-      } else {
-        const double2* sl = reinterpret_cast<const double2*>(p.Sl) + ((int64_t)m * M + a0) * M + x;
-        const double2* sg = reinterpret_cast<const double2*>(p.Sg) + ((int64_t)m * M + a0) * M + x;
-#pragma unroll
-        for (int k = 0; k < kNA; ++k) {
-          if (k < na) {
-            const double2 vl = sl[(int64_t)k * M], vg = sg[(int64_t)k * M];
-            cmac(lr[k], li[k], c2f(make_double2(wcm * vl.x, wcm * vl.y)), ga);
-            cmac(gr[k], gi[k], c2f(make_double2(wcm * vg.x, wcm * vg.y)), ga);
-          }
-        }
-      }
+      point(p, sum, m, c, a0, na, x, b, pl, q, a1 + x, nb + x, M);
     }
   }
-  double2* d = reinterpret_cast<double2*>(p.dst);
-  const int64_t stride_s = (int64_t)(n + 1) * MM;
-  const int64_t base = (int64_t)chunk * 2 * stride_s + (int64_t)c * MM + b;
-#pragma unroll
-  for (int k = 0; k < kNA; ++k) {
-    if (k < na) {
-      const int64_t e = base + (int64_t)(a0 + k) * M;
-      d[e] = make_double2((double)lr[k].s + (double)lr[k].c, (double)li[k].s + (double)li[k].c);
-      d[e + stride_s] = make_double2((double)gr[k].s + (double)gr[k].c, (double)gi[k].s + (double)gi[k].c);
-    }
-  }
+  store_sums(p, sum, chunk, c, a0, na, b);
 }
 
 // Shared-memory form for M <= 32: a block owns CB output columns and AGB
@@ -183,8 +204,8 @@ __global__ void __launch_bounds__(kDfBlock) history_df_tiled(DfArgs p, TileGeom 
   extern __shared__ float4 sm[];
   const int M = p.M, MM = p.MM, n = p.n, AG = p.AG;
   const int CB = tg.CB, AGB = tg.AGB, TM = tg.TM, NAB = AGB * kNA;
-  float4* sG = sm;                                  // [TM][CB][3][MM]: G^<, G^>, G^A as [x][b]
-  float4* sS = sm + (size_t)TM * CB * 3 * MM;       // [TM][3][NAB][M]: A1, B^<, B^> rows
+  float4* sG = sm;                                  // [TM][CB][2][MM]: PL, Q as [x][b]
+  float4* sS = sm + (size_t)TM * CB * 2 * MM;       // [TM][2][NAB][M]: A1, -B^< rows
   // column tiles from the last one down (heavier tiles of each chunk first)
   const int bx = (int)(gridDim.x - 1 - blockIdx.x);
   const int ct = bx / tg.ag_tiles, at = bx - ct * tg.ag_tiles;
@@ -200,14 +221,11 @@ __global__ void __launch_bounds__(kDfBlock) history_df_tiled(DfArgs p, TileGeom 
   const int chunk = blockIdx.y;
   const int m0 = chunk * p.chunk_len;
   const int m1 = min(n + 1, m0 + p.chunk_len);
-  const int band_lo = c - p.w.band_w + 1;
   const double2* L = reinterpret_cast<const double2*>(p.L);
   const double2* R = reinterpret_cast<const double2*>(p.R);
   const int nab = min(NAB, M - a_base);  // values of a of this block
 
-  Acc lr[kNA], li[kNA], gr[kNA], gi[kNA];
-#pragma unroll
-  for (int k = 0; k < kNA; ++k) lr[k] = li[k] = gr[k] = gi[k] = Acc{0.f, 0.f};
+  Sums sum;
 
   for (int mt = m0; mt < m1; mt += TM) {
     const int tm = min(TM, m1 - mt);
@@ -220,92 +238,38 @@ __global__ void __launch_bounds__(kDfBlock) history_df_tiled(DfArgs p, TileGeom 
       const int cc = r / MM, e = r - cc * MM;
       const int m = mt + mi, col = c_base + cc;
       if (col > n) continue;
-      float4* dst = sG + ((size_t)(mi * CB + cc) * 3) * MM;
+      float4* dst = sG + ((size_t)(mi * CB + cc) * 2) * MM;
       if (m >= col) {
         const int64_t blk = tri(m, col) * MM;
-        const float4 l = c2f(L[blk + e]), rv = c2f(R[blk + e]);
-        dst[e] = l;
-        dst[MM + e] = cadd(l, rv);
-        if (m == col) {  // G^A(c,c)_xb = conj(R(c,c)_bx)
-          const int x = e / M, bb = e - x * M;
-          dst[2 * MM + e] = cconj(c2f(R[blk + bb * M + x]));
-        }
+        dst[e] = c2f(L[blk + e]);
+        dst[MM + e] = c2f(R[blk + e]);
       } else {
         const int64_t blk = tri(col, m) * MM;   // stored entry (b, x) at e = b M + x
         const int bb = e / M, x = e - bb * M;
-        const float4 l = c2f(L[blk + e]), rv = c2f(R[blk + e]);
         const int et = x * M + bb;
-        dst[et] = cneg(cconj(l));
-        dst[MM + et] = cneg(cconj(cadd(l, rv)));
-        dst[2 * MM + et] = cconj(rv);
+        dst[et] = cneg(cconj(c2f(L[blk + e])));
+        dst[MM + et] = cneg(cconj(c2f(R[blk + e])));
       }
     }
     // operand rows of the block's values of a
-    const int s_items = tm * 3 * nab * M;
+    const int s_items = tm * 2 * nab * M;
     for (int i = tid; i < s_items; i += kDfBlock) {
-      const int mi = i / (3 * nab * M), r = i - mi * 3 * nab * M;
+      const int mi = i / (2 * nab * M), r = i - mi * 2 * nab * M;
       const int v = r / (nab * M), e = r - v * nab * M;   // e = (a - a_base) M + x
-      const float4* src = v == 0 ? p.A1 : (v == 1 ? p.Bl : p.Bg);
-      sS[((size_t)(mi * 3 + v) * NAB) * M + e] = src[((int64_t)(mt + mi) * M + a_base) * M + e];
+      const float4* src = v == 0 ? p.A1 : p.NB;
+      sS[((size_t)(mi * 2 + v) * NAB) * M + e] = src[((int64_t)(mt + mi) * M + a_base) * M + e];
     }
     __syncthreads();
     if (!live) continue;
     for (int mi = 0; mi < tm; ++mi) {
       const int m = mt + mi;
-      const bool below = m > c;
-      const bool band = !below && m >= band_lo;
-      const double wcm = band ? p.w.at(c, m) : 0.0;
-      const float4* g = sG + ((size_t)(mi * CB + cl) * 3) * MM + b;
-      const float4* s1p = sS + ((size_t)(mi * 3 + 0) * NAB + (a0 - a_base)) * M;
-      const float4* blp = sS + ((size_t)(mi * 3 + 1) * NAB + (a0 - a_base)) * M;
-      const float4* bgp = sS + ((size_t)(mi * 3 + 2) * NAB + (a0 - a_base)) * M;
-      for (int x = 0; x < M; ++x) {
-        const float4 gl = g[x * M], gs = g[MM + x * M];
-#pragma unroll
-        for (int k = 0; k < kNA; ++k) {
-          if (k < na) {
-            const float4 s1 = s1p[k * M + x];
-            cmac(lr[k], li[k], s1, gl);
-            cmac(gr[k], gi[k], s1, gs);
-          }
-        }
-        if (below) continue;
-        const float4 ga = g[2 * MM + x * M];
-        if (!band) {
-#pragma unroll
-          for (int k = 0; k < kNA; ++k) {
-            if (k < na) {
-              cmac(lr[k], li[k], blp[k * M + x], ga);
-              cmac(gr[k], gi[k], bgp[k * M + x], ga);
-            }
-          }
-        } else {
-          const double2* sl = reinterpret_cast<const double2*>(p.Sl) + ((int64_t)m * M + a0) * M + x;
-          const double2* sg = reinterpret_cast<const double2*>(p.Sg) + ((int64_t)m * M + a0) * M + x;
-#pragma unroll
-          for (int k = 0; k < kNA; ++k) {
-            if (k < na) {
-              const double2 vl = sl[(int64_t)k * M], vg = sg[(int64_t)k * M];
-              cmac(lr[k], li[k], c2f(make_double2(wcm * vl.x, wcm * vl.y)), ga);
-              cmac(gr[k], gi[k], c2f(make_double2(wcm * vg.x, wcm * vg.y)), ga);
-            }
-          }
-        }
-      }
+      const float4* g = sG + ((size_t)(mi * CB + cl) * 2) * MM + b;
+      const float4* s1 = sS + ((size_t)(mi * 2 + 0) * NAB + (a0 - a_base)) * M;
+      const float4* nb = sS + ((size_t)(mi * 2 + 1) * NAB + (a0 - a_base)) * M;
+      for (int x = 0; x < M; ++x) point(p, sum, m, c, a0, na, x, b, g[x * M], g[MM + x * M], s1 + x, nb + x, M);
     }
   }
-  if (!live) return;
-  double2* d = reinterpret_cast<double2*>(p.dst);
-  const int64_t stride_s = (int64_t)(n + 1) * MM;
-  const int64_t base = (int64_t)chunk * 2 * stride_s + (int64_t)c * MM + b;
-#pragma unroll
-  for (int k = 0; k < kNA; ++k) {
-    if (k < na) {
-      const int64_t e = base + (int64_t)(a0 + k) * M;
-      d[e] = make_double2((double)lr[k].s + (double)lr[k].c, (double)li[k].s + (double)li[k].c);
-      d[e + stride_s] = make_double2((double)gr[k].s + (double)gr[k].c, (double)gi[k].s + (double)gi[k].c);
-    }
-  }
+  if (live) store_sums(p, sum, chunk, c, a0, na, b);
 }
 
 // Block tiling of history_df_tiled for M orbitals and n + 1 columns, within
@@ -320,7 +284,7 @@ bool tile_geom(int M, int n, size_t smem_max, TileGeom* tg, size_t* smem) {
     tg->CB = 1;
     tg->AGB = kDfBlock / M;
   }
-  const size_t per_m = ((size_t)tg->CB * 3 * M * M + (size_t)3 * tg->AGB * kNA * M) * sizeof(float4);
+  const size_t per_m = ((size_t)tg->CB * 2 * M * M + (size_t)2 * tg->AGB * kNA * M) * sizeof(float4);
   tg->TM = (int)std::max<size_t>(1, std::min<size_t>(8, smem_max / per_m));
   if (per_m > smem_max) return false;
   *smem = per_m * tg->TM;
@@ -336,8 +300,8 @@ inline unsigned grid_for(int64_t n, int64_t cap) {
 
 }  // namespace
 
-// Workspace as launch_history_f64: the three double-float operand rows take
-// the places of A1, Bl, Bg (16 bytes per complex either way), then the
+// Workspace as launch_history_f64: the two double-float operand rows take
+// the places of A1, Bl (16 bytes per complex either way), then the
 // per-chunk partials.
 cudaError_t launch_history_df(const HistoryArgs& a, cudaStream_t s, int* launches) {
   const int M = a.M, MM = M * M, n = a.n;
@@ -349,22 +313,21 @@ cudaError_t launch_history_df(const HistoryArgs& a, cudaStream_t s, int* launche
   int64_t want = std::max<int64_t>(((int64_t)sm_count() * 2048 + threads - 1) / threads, (n + 1 + 31) / 32);
   int nchunk = (int)std::min<int64_t>(std::max<int64_t>(want, 1), kMaxSplit);
   if (nchunk > n + 1) nchunk = n + 1;
-  const size_t prep_bytes = (size_t)3 * row * 16;
+  const size_t prep_bytes = (size_t)2 * row * 16;
   while (nchunk > 1 && prep_bytes + (size_t)nchunk * 2 * row * 16 > a.part_bytes) --nchunk;
   if (prep_bytes + (nchunk > 1 ? (size_t)nchunk * 2 * row * 16 : 0) > a.part_bytes) return cudaErrorInvalidValue;
   const int chunk_len = (n + 1 + nchunk - 1) / nchunk;
   nchunk = (n + 1 + chunk_len - 1) / chunk_len;
 
   float4* A1 = reinterpret_cast<float4*>(a.part);
-  float4* Bl = A1 + row;
-  float4* Bg = Bl + row;
-  double* partials = a.part + 6 * row;
+  float4* NB = A1 + row;
+  double* partials = a.part + 4 * row;
   int nl = 0;
-  history_df_prep<<<grid_for(row, sm_count() * 8), 256, 0, s>>>(MM, n, a.Sl, a.Sg, a.w, A1, Bl, Bg);
+  history_df_prep<<<grid_for(row, sm_count() * 8), 256, 0, s>>>(MM, n, a.Sl, a.Sg, a.w, A1, NB);
   ++nl;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { *launches = nl; return e; }
-  DfArgs p{M, MM, n, AG, chunk_len, a.L, a.R, a.Sl, a.Sg, A1, Bl, Bg, a.w, nchunk == 1 ? a.out : partials};
+  DfArgs p{M, MM, n, AG, chunk_len, a.L, a.R, a.Sl, a.Sg, A1, NB, a.w, nchunk == 1 ? a.out : partials};
   TileGeom tg;
   size_t smem = 0;
   const bool tiled = tile_geom(M, n, kTileSmem, &tg, &smem);

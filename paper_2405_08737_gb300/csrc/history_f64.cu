@@ -9,18 +9,20 @@
 // GB300 design notes.  FP64 on this part runs at about 2 DFMA per clock per
 // SM (1.2 TFLOP/s measured for the whole GPU; FP64 mma.sync measured lower,
 // 1.05 TFLOP/s), so the contraction is bound by the FP64 pipe at every
-// orbital count: 48 M^3 flops per 32 M^2 bytes of history is 1.5 M flop/B,
+// orbital count: 32 M^3 flops per 32 M^2 bytes of history is M flop/B,
 // far above the 0.18 flop/B balance point of 1.2 TFLOP/s over 6.8 TB/s.
 // The kernel therefore spends its FP64 issue slots on complex multiply-adds
 // only:
 //   * a prep pass folds the weights into the self-energy row once:
 //       A1[m] = w_{n,m} (S^> - S^<)[m]          (term 1, all m)
-//       B^s[m] = wbar_m S^s[m]                    (term 2, settled weights)
+//       B^<[m] = wbar_m S^<[m]                    (term 2, settled weights)
 //     so the main loop holds no weight products except in the K+1 band
 //     points next to the diagonal, where w_{c,m} still differs from wbar_m;
-//   * term 1 is split as A1 G^> = A1 G^< + A1 G^R (no G^< + G^R sums);
-//   * one thread owns one output entry (c, a, b) for both s, with four
-//     independent complex accumulators (8 FMA chains);
+//   * term 1 is split as A1 G^> = A1 G^< + A1 G^R (no G^< + G^R sums), and
+//     where the weights are settled its second part cancels against term 2
+//     (history_partial_entry): two products per point instead of four;
+//   * one thread owns one output entry (c, a, b) for both s, with two
+//     or more independent complex accumulators (4 FMA chains);
 //   * the history index m is split into chunks across grid.y; partial sums
 //     go to a workspace and a second kernel adds them in a fixed order, so
 //     results are bitwise reproducible.
@@ -41,12 +43,11 @@ constexpr int kHistBlock = 128;  // threads per block of the contraction
 
 __global__ void __launch_bounds__(256) history_prep(int MM, int n, const double* __restrict__ Sl,
                                                     const double* __restrict__ Sg, WeightsView w,
-                                                    double* __restrict__ A1, double* __restrict__ Bl,
-                                                    double* __restrict__ Bg) {
+                                                    double* __restrict__ A1, double* __restrict__ Bl) {
   const int64_t total = (int64_t)(n + 1) * MM;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x)
-    rk::history_prep_entry(MM, n, e, Sl, Sg, w, A1, Bl, Bg);
+    rk::history_prep_entry(MM, n, e, Sl, Sg, w, A1, Bl);
 }
 
 // Output entries lin in [lin0, lin_end) (whole columns: lin = c M^2 + a M + b).
@@ -89,7 +90,7 @@ inline unsigned grid_for(int64_t n, int64_t cap) {
 // Split of the history index m of the FP64 slice of row n: at least enough
 // threads for full occupancy (every SM x 2048 threads), and chunks short
 // enough that one 128-thread block does about 2^16 complex multiply-adds
-// (3M per point and output), which keeps the tail of the launch short; the
+// (2M per point and output; counted as 3M here), which keeps the tail of the launch short; the
 // partials must fit the workspace.  A band of stored rows below n
 // contributes only history points m < band_hi: the chunks beyond them have
 // no work.  False when even one chunk does not fit.
@@ -117,7 +118,7 @@ bool history_f64_split(int M, int n, size_t part_bytes, int band_hi, int* nchunk
     nchunk = (int)std::min<int64_t>(std::min<int64_t>((n + 1 + len - 1) / len, cap), kMaxSplitSmall);
   }
   if (nchunk > n + 1) nchunk = n + 1;
-  const size_t prep_bytes = (size_t)3 * row * 16;
+  const size_t prep_bytes = (size_t)2 * row * 16;
   while (nchunk > 1 && prep_bytes + (size_t)nchunk * 2 * row * 16 > part_bytes) --nchunk;
   if (prep_bytes + (nchunk > 1 ? (size_t)nchunk * 2 * row * 16 : 0) > part_bytes) return false;
   const int chunk_len = (n + 1 + nchunk - 1) / nchunk;
@@ -128,7 +129,7 @@ bool history_f64_split(int M, int n, size_t part_bytes, int band_hi, int* nchunk
   return true;
 }
 
-// Workspace layout (doubles): A1, Bl, Bg: 3 x (n+1) MM complex; then the
+// Workspace layout (doubles): A1, Bl: 2 x (n+1) MM complex; then the
 // split partials nchunk x 2 x (n+1) MM complex.  The output columns may be
 // contracted in several launches (column ranges, each after an optional
 // event, e.g. the arrival of the history rows it reads); every entry is
@@ -143,14 +144,13 @@ cudaError_t launch_history_f64_ranges(const HistoryArgs& a, int nranges, const i
 
   double* A1 = a.part;
   double* Bl = A1 + 2 * row;
-  double* Bg = Bl + 2 * row;
-  double* partials = Bg + 2 * row;
+  double* partials = Bl + 2 * row;
   int nl = 0;
-  history_prep<<<grid_for(row, sm_count() * 8), 256, 0, s>>>(MM, n, a.Sl, a.Sg, a.w, A1, Bl, Bg);
+  history_prep<<<grid_for(row, sm_count() * 8), 256, 0, s>>>(MM, n, a.Sl, a.Sg, a.w, A1, Bl);
   ++nl;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { *launches = nl; return e; }
-  PartialArgs p{M, MM, n, chunk_len, a.L, a.R, a.Sl, a.Sg, A1, Bl, Bg, a.w,
+  PartialArgs p{M, MM, n, chunk_len, a.L, a.R, a.Sl, a.Sg, A1, Bl, a.w,
                 nchunk == 1 ? a.out : partials};
   p.band_lo = a.band_lo;
   p.band_hi = a.band_hi;

@@ -47,7 +47,7 @@ struct RunSmallArgs {
   double* Sg_w;
   double* I;             // history slice [2][n+1][M][M]
   WeightsView w;
-  double* part;          // workspace: A1 | Bl | Bg | chunk partials
+  double* part;          // workspace: A1 | Bl | chunk partials
   const double* corr0;   // stepper weight tables of row 0 ([n_max][kMaxOrder][kWTab])
   const double* pred0;
   unsigned* bar;         // barrier counter, zero at launch
@@ -160,9 +160,8 @@ __global__ void __launch_bounds__(kRunThreads, 2) run_small_kernel(const __grid_
     const double2* Rr = reinterpret_cast<const double2*>(a.base.R) + off;
     double* A1 = a.part;
     double* Bl = A1 + 2 * row;
-    double* Bg = Bl + 2 * row;
-    double* partials = Bg + 2 * row;
-    rk::PartialArgs p{M, MM, n, r.chunk_len, a.base.L, a.base.R, a.Sl, a.Sg, A1, Bl, Bg, a.w,
+    double* partials = Bl + 2 * row;
+    rk::PartialArgs p{M, MM, n, r.chunk_len, a.base.L, a.base.R, a.Sl, a.Sg, A1, Bl, a.w,
                       r.nchunk == 1 ? a.I : partials};
     const bool next = st + 1 < a.nsteps;
     const Span sr = span_units(row, MM);
@@ -174,7 +173,7 @@ __global__ void __launch_bounds__(kRunThreads, 2) run_small_kernel(const __grid_
         const int blk = rk::div_idx(e, MM), ab = (int)(e - (int64_t)blk * MM);
         ok &= rk::sigma_entry(M, e, ab, blk == n, rk::sigma_uu(M, ab, a.base.U), Lr, Rr,
                               reinterpret_cast<double2*>(a.Sl_w), reinterpret_cast<double2*>(a.Sg_w));
-        rk::history_prep_entry(MM, n, e, a.Sl, a.Sg, a.w, A1, Bl, Bg);
+        rk::history_prep_entry(MM, n, e, a.Sl, a.Sg, a.w, A1, Bl);
       }
       if (sr.base <= row - MM && row - MM < sr.hi) {
         // threads from the top of the block: those past the span's entries

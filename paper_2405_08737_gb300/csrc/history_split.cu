@@ -19,6 +19,11 @@
 //   D[c] = (I^> - I^<)[c] = sum_m A1[m] Q(m,c) + sum_{m<=c} NBD[m] Q(m,c)
 // (G^> - G^< = G^R gives the difference without a second PL product), and
 // the reduction adds I^> = I^< + D.
+// Where the weights are settled (m <= c - band_w: w_{n,m} = wbar_m) NBD = -A1,
+// so the two products of D cancel; D is formed from the other chunks alone
+// (chunk_class 0 and 2).  Leaving the cancelling products out took the split
+// KBE step n = 1023, M = 8 from 0.894 to 0.859 ms and the slice n = 511,
+// M = 32 from 10.45 to 10.26 ms (half the MMAs of half the chunks).
 // For one output tile (128 rows j = (c,b)) and one chunk of 16 complex K
 // entries (m,x), the big operands are the plane tiles PL, Q and the masked
 // QU = Q [m <= c]; the small operands A1, NB^<, NBD (prepared once per
@@ -516,6 +521,7 @@ __global__ void __launch_bounds__(kThreads2, 1) split_main2(Split2Args a) {
         const uint64_t dSU = dS0 + (uint64_t)(((1 + mgrp) * kSmallVar) >> 4);
 #pragma unroll
         for (int i = 0; i < kSlices; ++i) {
+          if (cls == 1 && mgrp == 1) break;  // settled: the two products of D cancel
           const uint32_t idesc = umma_idesc_f16(kNS * (kLevels - i < kSlices ? kLevels - i : kSlices));
 #pragma unroll
           for (int kk = 0; kk < 2; ++kk) {
@@ -577,24 +583,27 @@ __global__ void __launch_bounds__(kThreads2, 1) split_main2(Split2Args a) {
       tc_fence_after();
       const float sc = pow2f(scale_from_field(ec) + es - 14);
       const uint32_t buf = lane_addr + b * kAccCols + my_cols;
+      const bool none = grp == 1 && chunk_class(cu.m_lo, cu.m_hi, cu.c0, cu.c0 + CT - 1, g.band_w) == 1;
+      if (!none) {
 #pragma unroll
-      for (int q4 = 0; q4 < kQ; q4 += 4) {
-        float v[kLevels][4];
-        tmem_ld4xL(buf + q4, kNS, v);
+        for (int q4 = 0; q4 < kQ; q4 += 4) {
+          float v[kLevels][4];
+          tmem_ld4xL(buf + q4, kNS, v);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float lv[kLevels] = {v[0][q], v[1][q], v[2][q], v[3][q], v[4][q]};
-          float hi, lo;
-          combine_levels(lv, hi, lo);
-          float& rh = run[q4 + q][0];
-          float& rl = run[q4 + q][1];
-          df_add(rh, rl, hi * sc);
-          rl += lo * sc;
+          for (int q = 0; q < 4; ++q) {
+            const float lv[kLevels] = {v[0][q], v[1][q], v[2][q], v[3][q], v[4][q]};
+            float hi, lo;
+            combine_levels(lv, hi, lo);
+            float& rh = run[q4 + q][0];
+            float& rl = run[q4 + q][1];
+            df_add(rh, rl, hi * sc);
+            rl += lo * sc;
+          }
         }
-      }
 #pragma unroll
-      for (int d = 0; d < kLevels; ++d) tmem_zero8(buf + d * kNS);
-      tmem_wait_st();
+        for (int d = 0; d < kLevels; ++d) tmem_zero8(buf + d * kNS);
+        tmem_wait_st();
+      }
       tc_fence_before();
       mbar_arrive(&sm.accempty[b]);
       if (u + 1 == u1 || cu.kc + 1 == g.cpt) {
@@ -1059,6 +1068,7 @@ __global__ void __launch_bounds__(kFThreads, 1) split_fused(FusedArgs a) {
           const uint32_t dacc = tmem + b * kAccCols + mgrp * kGroupCols;
 #pragma unroll
           for (int i = 0; i < kSlices; ++i) {
+            if (cls == 1 && mgrp == 1) break;  // settled: the two products of D cancel
             const uint32_t idesc = umma_idesc_f16(kNS * (kLevels - i < kSlices ? kLevels - i : kSlices));
             const uint64_t oa = (uint64_t)((i * kHSlice) >> 4);
             umma_f16(dacc + i * kNS, dA + oa, dS0, idesc, 1);
@@ -1123,27 +1133,31 @@ __global__ void __launch_bounds__(kFThreads, 1) split_fused(FusedArgs a) {
         const float sc = pow2f(scale_from_field(ec) + es - 14);
         const uint32_t buf = lane_addr + b * kAccCols + grp * kGroupCols;
         const uint32_t run = lane_addr + kFRunCol + p * kFRunPart + grp * 2 * kNS;
-        float rh[kNS], rl[kNS];
-        tmem_ld16(run, rh);
-        tmem_ld16(run + kNS, rl);
+        const bool none = grp == 1 && chunk_class(fused_div(P.kap0, M, S.magic), fused_div(P.kap0 + kHK - 1, M, S.magic),
+                                                  P.ctile * CT, P.ctile * CT + CT - 1, S.w.band_w) == 1;
+        if (!none) {
+          float rh[kNS], rl[kNS];
+          tmem_ld16(run, rh);
+          tmem_ld16(run + kNS, rl);
 #pragma unroll
-        for (int q4 = 0; q4 < kNS; q4 += 4) {
-          float v[kLevels][4];
-          tmem_ld4xL(buf + q4, kNS, v);
+          for (int q4 = 0; q4 < kNS; q4 += 4) {
+            float v[kLevels][4];
+            tmem_ld4xL(buf + q4, kNS, v);
 #pragma unroll
-          for (int qq = 0; qq < 4; ++qq) {
-            const float lv[kLevels] = {v[0][qq], v[1][qq], v[2][qq], v[3][qq], v[4][qq]};
-            float hi, lo;
-            combine_levels(lv, hi, lo);
-            df_add(rh[q4 + qq], rl[q4 + qq], hi * sc);
-            rl[q4 + qq] += lo * sc;
+            for (int qq = 0; qq < 4; ++qq) {
+              const float lv[kLevels] = {v[0][qq], v[1][qq], v[2][qq], v[3][qq], v[4][qq]};
+              float hi, lo;
+              combine_levels(lv, hi, lo);
+              df_add(rh[q4 + qq], rl[q4 + qq], hi * sc);
+              rl[q4 + qq] += lo * sc;
+            }
           }
-        }
-        tmem_st16(run, rh);
-        tmem_st16(run + kNS, rl);
+          tmem_st16(run, rh);
+          tmem_st16(run + kNS, rl);
 #pragma unroll
-        for (int d = 0; d < kLevels; ++d) tmem_zero16(buf + d * kNS);
-        tmem_wait_st();
+          for (int d = 0; d < kLevels; ++d) tmem_zero16(buf + d * kNS);
+          tmem_wait_st();
+        }
         tc_fence_before();
         mbar_arrive(&sm.accempty[b]);
       }

@@ -65,7 +65,12 @@ typedef int kbe_status;
 #define KBE_DENSE_MAX_NORB 32  /* largest norb for a dense interaction      */
 
 /* precision argument of kbe_history_slice / kbe_step */
-#define KBE_FP64 0        /* plain FP64 arithmetic, deterministic            */
+#define KBE_FP64 0        /* FP64 accuracy, deterministic: FP64 arithmetic;  */
+                          /* the larger slices ((n+1)^2 norb^3 >= 8e6) form   */
+                          /* their products on the tensor cores from eight    */
+                          /* error-free 8-bit digits per value (about 2^-57   */
+                          /* of the largest product of 32 history entries)    */
+                          /* and sum them in FP64                             */
 #define KBE_SPLIT_BF16 1  /* the contraction on the 16-bit-float tensor cores */
                           /* with error-free 4-digit fixed-point splitting:   */
                           /* every value becomes round(v 2^(31-e)) in base-256 */
@@ -89,6 +94,9 @@ typedef int kbe_status;
 /* Create a context for norb orbitals and at most n_max time points.
  * Allocates device workspace only (split-reduction partials, weight tables,
  * status word); the two-time arrays belong to the caller.
+ * The workspace of the FP64 slices on the tensor cores (about 1.1 KB times
+ * n_max norb ceil(norb/8)) is optional: without room for it every FP64 slice
+ * runs on the FP64 pipe.
  * KBE_EINVAL: out == NULL, norb < 1, norb > 64, n_max < 1, or sizes that
  * overflow 64-bit block indices.  KBE_ENOMEM / KBE_ECUDA on device errors. */
 kbe_status kbe_create(int norb, int n_max, kbe_ctx** out);

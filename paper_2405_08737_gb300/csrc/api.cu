@@ -48,6 +48,9 @@ void release(kbe_ctx* ctx) {
   cudaFree(ctx->d_wbar); cudaFree(ctx->d_band); cudaFree(ctx->d_corr); cudaFree(ctx->d_pred);
   cudaFree(ctx->d_h0); cudaFree(ctx->d_U); cudaFree(ctx->d_v); cudaFree(ctx->d_eps);
   cudaFree(ctx->d_part); cudaFree(ctx->d_status); cudaFree(ctx->d_split); cudaFree(ctx->d_adj);
+  cudaFree(ctx->d_fx);
+  ctx->d_fx = nullptr;
+  ctx->fx_bytes = 0;
   cudaFree(ctx->d_runbar);
   ctx->d_runbar = nullptr;
   cudaFree(ctx->d_planes);
@@ -108,6 +111,22 @@ bool next_events(kbe_ctx* ctx, cudaEvent_t* b, cudaEvent_t* e) {
 // of the same arrays are reused (the split path re-encodes only units that
 // involve rows >= the cached row count).
 struct Staged;
+// Whether the FP64 slice of row n goes to the tensor cores (history_fx.cu): from
+// (n + 1)^2 M^3 = 8e6 on, and never for the rows that kbe_run_steps takes in its
+// cooperative kernel.  Below that the FP64 pipe is as fast or faster, above it
+// falls behind with the cube of M (slices on the FP64 pipe against the tensor
+// cores, us: M = 8, n = 100 107 / 100, n = 1023 7080 / 970; M = 16, n = 30 100 /
+// 136, n = 100 662 / 219; M = 5, n = 200 119 / 107; M = 24, n = 20 160 / 183; M = 32,
+// n = 50 1383 / 521).
+bool use_fx(const kbe_ctx* ctx, int n) {
+  const double N = n + 1.0, M = ctx->M;
+  return ctx->d_fx && N * M * M > kRunMaxRow && N * N * M * M * M >= 8e6;
+}
+cudaError_t slice_f64(const kbe_ctx* ctx, const HistoryArgs& a, cudaStream_t s, int* launches) {
+  if (use_fx(ctx, a.n) && a.band_lo <= 0 && a.band_hi > a.n)
+    return launch_history_fx(a, ctx->d_fx, ctx->fx_bytes, s, launches);
+  return launch_history_f64(a, s, launches);
+}
 kbe_status history(kbe_ctx* ctx, int n, int precision, const void* L, const void* R, const void* Sl,
                    const void* Sg, void* I_out, cudaStream_t s, int* launches, bool stepping = false,
                    const Staged* staged = nullptr);
@@ -172,12 +191,12 @@ kbe_status history(kbe_ctx* ctx, int n, int precision, const void* L, const void
     e = launch_history_df(a, s, launches);
     return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "history slice launch");
   }
-  if (staged) {  // the column ranges contract as their rows arrive (no timing events: they would hold the waits)
+  if (staged && !use_fx(ctx, n)) {  // the column ranges contract as their rows arrive (no timing events: they would hold the waits)
     e = launch_history_f64_ranges(a, staged->k, staged->c_lo, staged->c_hi, staged->ev, s, launches);
     return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "history slice launch");
   }
   if (!next_events(ctx, &a.ev_begin, &a.ev_end)) return fail(ctx, KBE_ECUDA, "profiling: cudaEventCreate");
-  e = launch_history_f64(a, s, launches);
+  e = slice_f64(ctx, a, s, launches);
   return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "history slice launch");
 }
 
@@ -333,7 +352,7 @@ kbe_status step_impl(kbe_ctx* ctx, int n, int P, int precision, void* L, void* R
   cudaError_t e = cudaSuccess;
   if (staged && (e = cudaStreamWaitEvent(s, staged->ev[0], 0)) != cudaSuccess)
     return cuda_fail(ctx, e, "kbe_step: wait for the uploaded rows");
-  const bool pipelined = staged && precision == KBE_FP64 && ctx->adaptive_K == 0 && !ctx->thermal;
+  const bool pipelined = staged && precision == KBE_FP64 && ctx->adaptive_K == 0 && !ctx->thermal && !use_fx(ctx, n);
   if (staged && !pipelined && (e = cudaStreamWaitEvent(s, staged->ev[staged->k - 1], 0)) != cudaSuccess)
     return cuda_fail(ctx, e, "kbe_step: wait for the uploaded rows");
   e = launch_predictor(a, s);
@@ -645,6 +664,15 @@ kbe_status kbe_create(int norb, int n_max, kbe_ctx** out) {
     return fail(nullptr, e == cudaErrorMemoryAllocation ? KBE_ENOMEM : KBE_ECUDA,
                 std::string("kbe_create: split workspace: ") + cudaGetErrorString(e));
   }
+  if ((int64_t)row > kRunMaxRow) {  // rows that the FP64 slice takes on the tensor cores
+    ctx->fx_bytes = fx_workspace_bytes(norb, n_max);
+    if (cudaMalloc(&ctx->d_fx, ctx->fx_bytes) != cudaSuccess || fx_prepare() != cudaSuccess) {
+      cudaGetLastError();  // no room: the slice stays on the FP64 pipe
+      cudaFree(ctx->d_fx);
+      ctx->d_fx = nullptr;
+      ctx->fx_bytes = 0;
+    }
+  }
   if ((e = cudaMemset(ctx->d_status, 0, sizeof(int))) != cudaSuccess) {
     release(ctx);
     delete ctx;
@@ -912,7 +940,7 @@ kbe_status kbe_history_slice_band(kbe_ctx* ctx, int n, int row_lo, int row_hi, c
   a.band_lo = row_lo;
   a.band_hi = row_hi;
   int nl = 0;
-  cudaError_t e = launch_history_f64(a, (cudaStream_t)stream, &nl);
+  cudaError_t e = slice_f64(ctx, a, (cudaStream_t)stream, &nl);
   ctx->last_launches = nl;
   return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "kbe_history_slice_band: launch");
 }
@@ -962,7 +990,7 @@ kbe_status kbe_step_sweep_band(kbe_ctx* ctx, int n, int row_lo, int row_hi, cons
   a.band_hi = row_hi;
   if (!next_events(ctx, &a.ev_begin, &a.ev_end)) return fail(ctx, KBE_ECUDA, "profiling: cudaEventCreate");
   int nl = 0;
-  e = launch_history_f64(a, s, &nl);
+  e = slice_f64(ctx, a, s, &nl);
   ctx->last_launches = 1 + nl;
   return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "kbe_step_sweep_band: history slice");
 }

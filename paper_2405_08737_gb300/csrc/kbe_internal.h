@@ -104,6 +104,8 @@ struct kbe_ctx {
   double* d_part = nullptr;   // FP64 slice workspace: prep rows, chunk partials [chunks][2][n_max][M][M] complex
   void* d_split = nullptr;    // split-precision workspace (digit planes of the small operands, partials)
   size_t split_bytes = 0;
+  void* d_fx = nullptr;       // workspace of the FP64 slice on the tensor cores (null: it stays on the FP64 pipe)
+  size_t fx_bytes = 0;
   void* d_planes = nullptr;   // digit planes of the history (split path), allocated by the first split slice
   kbe::SplitPlanes planes_layout;
   bool planes_failed = false; // allocation failed once: the in-kernel conversion path is used
@@ -210,6 +212,12 @@ cudaError_t launch_history_finish(int nchunk, int64_t row, const double* partial
 // and wait[k] are set); bitwise the same results as one launch.
 cudaError_t launch_history_f64_ranges(const HistoryArgs& a, int nranges, const int* c_lo, const int* c_hi,
                                       const cudaEvent_t* wait, cudaStream_t s, int* launches);
+
+// FP64 history slice on the tensor cores (history_fx.cu): the sums of
+// launch_history_f64 over all stored rows, in the workspace `work`.
+size_t fx_workspace_bytes(int M, int n_max);
+cudaError_t fx_prepare();  // one-time kernel attributes of the current device
+cudaError_t launch_history_fx(const HistoryArgs& a, void* work, size_t work_bytes, cudaStream_t s, int* launches);
 
 // Split-precision history slice (history_split.cu).
 struct SplitGeomHost {

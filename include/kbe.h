@@ -66,7 +66,7 @@ typedef int kbe_status;
 
 /* precision argument of kbe_history_slice / kbe_step */
 #define KBE_FP64 0        /* FP64 accuracy, deterministic: FP64 arithmetic;  */
-                          /* the larger slices ((n+1)^2 norb^3 >= 8e6) form   */
+                          /* the larger slices ((n+1)^2 norb^3 >= 5e6) form   */
                           /* their products on the tensor cores from eight    */
                           /* error-free 8-bit digits per value (about 2^-57   */
                           /* of the largest product of 32 history entries)    */
@@ -94,7 +94,7 @@ typedef int kbe_status;
 /* Create a context for norb orbitals and at most n_max time points.
  * Allocates device workspace only (split-reduction partials, weight tables,
  * status word); the two-time arrays belong to the caller.
- * The workspace of the FP64 slices on the tensor cores (about 1.1 KB times
+ * The workspace of the FP64 slices on the tensor cores (about 2.1 KB times
  * n_max norb ceil(norb/8)) is optional: without room for it every FP64 slice
  * runs on the FP64 pipe.
  * KBE_EINVAL: out == NULL, norb < 1, norb > 64, n_max < 1, or sizes that

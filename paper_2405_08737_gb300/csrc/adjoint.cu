@@ -17,6 +17,7 @@
 // (R(r,r) = -i*1 is a constant of the method and carries no cotangent.)
 
 #include "dfloat.cuh"
+#include "history_fx.h"
 #include "kbe_internal.h"
 
 namespace kbe {
@@ -533,7 +534,12 @@ cudaError_t launch_adjoint_history(const AdjHistArgs& h, cudaStream_t s, int* la
   double* A1 = Js + srow * 2;
   adj_prep<<<blocks_for(srow), 256, 0, s>>>(M, n, h.Ib, h.Sl, h.Sg, h.w, Js, A1);
   int nl = 3;
-  if (h.df) {
+  if (h.fx_work) {  // the Sigma-row cotangents on the tensor cores
+    int k = 0;
+    const cudaError_t ef = launch_adjoint_fx(h, h.fx_work, h.fx_bytes, h.status, s, &k);
+    if (ef != cudaSuccess) return ef;
+    nl += k - 2;
+  } else if (h.df) {
     float4* Ibf = reinterpret_cast<float4*>(A1 + srow * 2);
     float4* Jsf = Ibf + 2 * srow;
     adj_prep_df<<<blocks_for(2 * srow), 256, 0, s>>>(2 * srow, h.Ib, Js, Ibf, Jsf, srow);
@@ -546,7 +552,7 @@ cudaError_t launch_adjoint_history(const AdjHistArgs& h, cudaStream_t s, int* la
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  adj_hist_small_reduce<<<blocks_for(srow), 256, 0, s>>>(M, n, nchunk, h.work, h.w, h.dSl, h.dSg);
+  if (!h.fx_work) adj_hist_small_reduce<<<blocks_for(srow), 256, 0, s>>>(M, n, nchunk, h.work, h.w, h.dSl, h.dSg);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int64_t rows_total = (tri(n + 1, 0) - tri(h.row_lo, 0)) * MM;
   adj_hist_rows<<<blocks_for(rows_total), 256, 0, s>>>(M, n, h.row_lo, Js, A1, h.Sl, h.Sg, h.Ib, h.w, h.dL, h.dR,

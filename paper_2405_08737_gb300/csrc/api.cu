@@ -7,6 +7,7 @@
 #include <cstring>
 #include <new>
 
+#include "history_fx.h"
 #include "kbe_internal.h"
 
 using namespace kbe;
@@ -112,15 +113,15 @@ bool next_events(kbe_ctx* ctx, cudaEvent_t* b, cudaEvent_t* e) {
 // involve rows >= the cached row count).
 struct Staged;
 // Whether the FP64 slice of row n goes to the tensor cores (history_fx.cu): from
-// (n + 1)^2 M^3 = 8e6 on, and never for the rows that kbe_run_steps takes in its
+// (n + 1)^2 M^3 = 5e6 on, and never for the rows that kbe_run_steps takes in its
 // cooperative kernel.  Below that the FP64 pipe is as fast or faster, above it
 // falls behind with the cube of M (slices on the FP64 pipe against the tensor
-// cores, us: M = 8, n = 100 107 / 100, n = 1023 7080 / 970; M = 16, n = 30 100 /
-// 136, n = 100 662 / 219; M = 5, n = 200 119 / 107; M = 24, n = 20 160 / 183; M = 32,
-// n = 50 1383 / 521).
+// cores, us: M = 5, n = 163 95 / 87; M = 8, n = 64 89 / 66, n = 1023 7080 / 905; M = 12,
+// n = 29 63 / 91, n = 50 107 / 130; M = 16, n = 16 55 / 84, n = 30 102 / 89; M = 24,
+// n = 10 68 / 100, n = 20 159 / 138; M = 32, n = 16 249 / 140).
 bool use_fx(const kbe_ctx* ctx, int n) {
   const double N = n + 1.0, M = ctx->M;
-  return ctx->d_fx && N * M * M > kRunMaxRow && N * N * M * M * M >= 8e6;
+  return ctx->d_fx && N * M * M > kRunMaxRow && N * N * M * M * M >= 5e6;
 }
 cudaError_t slice_f64(const kbe_ctx* ctx, const HistoryArgs& a, cudaStream_t s, int* launches) {
   if (use_fx(ctx, a.n) && a.band_lo <= 0 && a.band_hi > a.n)
@@ -198,6 +199,14 @@ kbe_status history(kbe_ctx* ctx, int n, int precision, const void* L, const void
   if (!next_events(ctx, &a.ev_begin, &a.ev_end)) return fail(ctx, KBE_ECUDA, "profiling: cudaEventCreate");
   e = slice_f64(ctx, a, s, launches);
   return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "history slice launch");
+}
+
+// The longest sums of the slice's adjoint follow the slice.
+void adjoint_fx(const kbe_ctx* ctx, AdjHistArgs* h) {
+  if (!use_fx(ctx, h->n)) return;
+  h->fx_work = ctx->d_fx;
+  h->fx_bytes = ctx->fx_bytes;
+  h->status = ctx->d_status;
 }
 
 // Self-energy of n_blocks blocks from first_block (launch_sigma geometry),
@@ -1302,6 +1311,7 @@ kbe_status kbe_adjoint_slice(kbe_ctx* ctx, int n, const void* L, const void* R, 
   AdjHistArgs h{ctx->M, n, row_lo, (const double*)L, (const double*)R, (const double*)S_less,
                 (const double*)S_great, (const double*)dI, weights_view(ctx), (double*)dS_less, (double*)dS_great,
                 (double*)dL, (double*)dR, (double*)dL + row_n, (double*)dR + row_n, ctx->d_part, ctx->part_bytes};
+  adjoint_fx(ctx, &h);
   int nl = 0;
   cudaError_t e = launch_adjoint_history(h, (cudaStream_t)stream, &nl);
   ctx->last_launches = nl;
@@ -1431,6 +1441,7 @@ kbe_status kbe_step_adjoint(kbe_ctx* ctx, int n, int P, int precision, void* L, 
     AdjHistArgs h{ctx->M, n, row_lo, (const double*)L, (const double*)R, Sl, Sg, Ib, weights_view(ctx), dSl, dSg,
                   (double*)dL, (double*)dR, gL, gR, ctx->d_part, ctx->part_bytes};
     h.df = precision == KBE_DF64;  // the step's own arithmetic for its longest reverse sum
+    adjoint_fx(ctx, &h);
     e = launch_adjoint_history(h, s, &nl);
     count += nl;
     if ((st = check("kbe_step_adjoint: history slice")) != KBE_OK) return st;

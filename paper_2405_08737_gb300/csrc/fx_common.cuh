@@ -29,20 +29,57 @@ constexpr int kOver = 6;       // chunks that a column tile visits twice, at mos
 constexpr int kHeadroom = 2;   // bits between a row's exponent and its first values
 constexpr int kNonFinite = 8000;  // exponent of a row or column that holds a non-finite value
 
-// One system's slice as a list of column tiles of CT = 128 / M output columns
-// (times parts of the small operand's rows a).
+// One system's contraction as a list of column tiles of CT = 128 / M output
+// columns (times parts of NA rows a of the small operand).  For the slice the
+// output columns are the c of I(n, c) and the contracted points the m; for its
+// adjoint the other way round (the row m of a Sigma cotangent, summed over c).
 struct Sys {
   const double* L;
   const double* R;
-  const uint8_t* small;   // [unit][part][small block]: written by the prep kernel
+  const double* Sl;       // operand rows: Sigma^<, Sigma^> (slice) or Ibar^<, Ibar^> (adjoint), [n+1][M][M]
+  const double* Sg;
+  const double* wbar;     // composite weights (WeightsView)
+  const double* band;
+  double* out0;           // I^< and I^>, or the cotangents of Sigma^< and Sigma^>
+  double* out1;
+  uint8_t* small;         // [unit][part][small block]: written by the prep kernel
+  double* part;           // partial sums, [tile + CTA - cta0][slot]
+  int* status;
   int M, n, CT, cpt;      // chunks per pass over the history: ceil((n + 1) M / 32)
   int parts, tiles;       // parts of a; column tiles x parts
-  int upt;                // chunk slots per tile: cpt + kOver
-  int shift;              // history point m of column c is "near" when m > c + shift, else "far"
+  int upt;                // chunk slots per tile
+  int band_w;
+  int adj;                // 0: slice, 1: adjoint
+  int shift;              // point m of column c is "near" when m > c + shift, else "far"
   uint32_t magic;         // ceil(2^32 / M) (0 for M = 1): x / M without a division
-  long long unit_base;    // first chunk slot and first tile of the system in the launch
-  long long tile_base;
+  int cta0;               // first CTA of the launch that takes slots of this system
+  long long unit_base;    // first chunk slot of the system in the launch
+  long long chunk_base;   // first chunk x part (prep) and first output entry (reduction)
+  long long entry_base;
 };
+struct Head {             // the systems of a launch
+  int n_sys;
+  long long total;        // chunk slots
+  long long chunks, entries;
+};
+
+// Geometry of a system (the pointers and bases are the caller's): NA values of a per part.
+__host__ __device__ __forceinline__ void set_geometry(Sys& s, int M, int n, int band_w, int adj, int NA) {
+  s.M = M;
+  s.n = n;
+  s.CT = kRows / M;
+  s.cpt = (int)(((long long)(n + 1) * M + kChunkK - 1) / kChunkK);
+  s.parts = (M + NA - 1) / NA;
+  s.tiles = (n + s.CT) / s.CT * s.parts;
+  // the far and near passes overlap in at most kOver chunks; the band points of a tile's columns
+  s.upt = s.cpt + kOver + ((s.CT - 1 + band_w) * M + kChunkK - 1) / kChunkK + 1;
+  s.band_w = band_w;
+  s.adj = adj;
+  s.shift = adj ? band_w - 1 : -band_w;
+  s.magic = M == 1 ? 0u : (uint32_t)((0x100000000ull + (unsigned long long)M - 1) / (unsigned long long)M);
+  s.cta0 = 0;
+  s.unit_base = s.chunk_base = s.entry_base = 0;
+}
 
 // x / M for 0 <= x < 2^32 / M
 __host__ __device__ __forceinline__ int div_m(int x, int M, uint32_t magic) {
@@ -54,82 +91,96 @@ __host__ __device__ __forceinline__ int div_m(int x, int M, uint32_t magic) {
 #endif
 }
 
-// A role's walk over the chunk slots of the launch.  A column tile's chunks come
-// in this order: first the far ones (entries with m <= c + shift count, both
-// planes into one sum), then the near ones (m > c + shift, one sum per plane).
-// The at most kOver chunks that straddle the line are taken once each way, with
-// the other side's entries masked; the remaining slots of a tile are empty.
+enum Class { kFar = 0, kNear = 1, kBand = 2 };
+
+// The walk over the chunk slots of a system.  A column tile's chunks come in
+// this order: the far ones (entries with m <= c + shift count, both planes into
+// one sum), the near ones (m > c + shift, one sum per plane), and the band of
+// term 2 (its own weights w_{c,m}).  The at most kOver chunks that straddle the
+// line between far and near are taken once each way, with the other side's
+// entries masked; the remaining slots of a tile are empty.
 struct Walk {
-  // system (copied: every role reads these once per unit)
-  int M, n, shift, parts, cpt, CT, upt, tiles;
-  uint32_t magic;
-  int si;
-  // tile
-  int T, part, c0;      // tile of the system, its part, first column
+  int si, T, part, c0;  // system of the launch, its tile, the tile's part and first column
   int nfar, far_k;      // far chunks and entries
   int first, near_k;    // first near chunk and entry
-  // chunk slot
-  int idx;
-  int near;             // 0: far, 1: near
+  int band0, band1;     // entries of the band
+  int idx;              // chunk slot of the tile
+  int cls;
   int kc, j0, j1;       // chunk of the history and its units [j0, j1) (empty slot: j0 = j1)
 
-  __host__ __device__ __forceinline__ void set_sys(const Sys& s, int i) {
-    M = s.M; n = s.n; shift = s.shift; parts = s.parts; cpt = s.cpt; CT = s.CT; upt = s.upt; tiles = s.tiles;
-    magic = s.magic;
-    si = i;
-  }
-  // position T, c0 and part are set
-  __host__ __device__ __forceinline__ void tile_start() {
-    const int c1 = c0 + CT - 1 < n ? c0 + CT - 1 : n;
-    const int far_m = c1 + shift < n ? c1 + shift : n;                 // last far point of the tile
-    const int near_m = c0 + shift + 1 > 0 ? c0 + shift + 1 : 0;        // its first near point
-    far_k = far_m < 0 ? 0 : (far_m + 1) * M;
+  // T, c0 and part are set
+  __host__ __device__ __forceinline__ void tile_start(const Sys& s) {
+    const int c1 = c0 + s.CT - 1 < s.n ? c0 + s.CT - 1 : s.n;
+    const int far_m = c1 + s.shift < s.n ? c1 + s.shift : s.n;          // last far point of the tile
+    const int near_m = c0 + s.shift + 1 > 0 ? c0 + s.shift + 1 : 0;     // its first near point
+    far_k = far_m < 0 ? 0 : (far_m + 1) * s.M;
     nfar = (far_k + kChunkK - 1) / kChunkK;
-    near_k = near_m * M;
-    first = near_m > n ? cpt : near_k / kChunkK;
+    near_k = near_m * s.M;
+    first = near_m > s.n ? s.cpt : near_k / kChunkK;
+    band0 = s.adj ? c0 * s.M : near_k;
+    band1 = s.adj ? far_k : (c1 + 1) * s.M;
   }
-  __host__ __device__ __forceinline__ void chunk_start() {
-    near = idx >= nfar;
-    kc = near ? first + idx - nfar : idx;
-    const int end = near ? (n + 1) * M : far_k;
-    const int u = (end - kc * kChunkK + kUnitK - 1) / kUnitK;
-    j1 = kc >= cpt ? 0 : (u < kChunkUnits ? u : kChunkUnits);
-    j0 = near && kc == first && kc < cpt ? (near_k - kc * kChunkK) / kUnitK : 0;
+  __host__ __device__ __forceinline__ void chunk_start(const Sys& s) {
+    const int nnear = s.cpt - first;
+    int beg = 0, end = far_k;
+    cls = kFar;
+    kc = idx;
+    if (idx >= nfar) {
+      cls = kNear;
+      kc = first + idx - nfar;
+      beg = near_k;
+      end = (s.n + 1) * s.M;
+    }
+    if (idx >= nfar + nnear) {
+      cls = kBand;
+      kc = band0 / kChunkK + idx - nfar - nnear;
+      beg = band0;
+      end = band1;
+    }
+    const int lo = beg - kc * kChunkK, hi = end - kc * kChunkK;
+    j0 = lo > 0 ? lo / kUnitK : 0;
+    j1 = hi > 0 ? (hi + kUnitK - 1) / kUnitK : 0;
+    if (j1 > kChunkUnits) j1 = kChunkUnits;
+    if (j1 < j0) j1 = j0;
   }
 };
 __host__ __device__ __forceinline__ void walk_to(Walk& w, const Sys& s, int i, long long slot) {
-  w.set_sys(s, i);
+  w.si = i;
   w.T = (int)(slot / s.upt);
   w.idx = (int)(slot - (long long)w.T * s.upt);
   const int ct = w.T / s.parts;
   w.part = w.T - ct * s.parts;
   w.c0 = ct * s.CT;
-  w.tile_start();
-  w.chunk_start();
+  w.tile_start(s);
+  w.chunk_start(s);
 }
-// The next slot of the launch; 1: of another tile, 2: past the system's last
-// tile (the caller moves to the next system, if any).
-__host__ __device__ __forceinline__ int walk_next(Walk& w) {
+// The next slot; 1: of another tile, 2: past the system's last tile (the
+// caller moves to the next system, if any).
+__host__ __device__ __forceinline__ int walk_next(Walk& w, const Sys& s) {
   int moved = 0;
-  if (++w.idx == w.upt) {
+  if (++w.idx == s.upt) {
     w.idx = 0;
-    if (++w.T == w.tiles) return 2;
-    if (++w.part == w.parts) {
+    if (++w.T == s.tiles) return 2;
+    if (++w.part == s.parts) {
       w.part = 0;
-      w.c0 += w.CT;
+      w.c0 += s.CT;
     }
-    w.tile_start();
+    w.tile_start(s);
     moved = 1;
   }
-  w.chunk_start();
+  w.chunk_start(s);
   return moved;
 }
 
-// Chunk slots [lo, hi) of CTA i of G over `total` slots, and the slot of the
-// partial sums of tile `tile` (counted over the launch) in CTA i: unique, since
-// CTAs take contiguous ranges.
+// Chunk slots [range_lo(i), range_lo(i + 1)) of CTA i of G over `total` slots.
 __host__ __device__ __forceinline__ long long range_lo(long long total, int G, int i) { return total * i / G; }
-__host__ __device__ __forceinline__ long long partial_slot(long long tile, int i) { return tile + i; }
+// First CTA whose range ends beyond slot q (0 <= q < total).
+__host__ __device__ __forceinline__ int cta_of(long long total, int G, long long q) {
+  int i = (int)(q * G / total);
+  while (i > 0 && range_lo(total, G, i) > q) --i;
+  while (range_lo(total, G, i + 1) <= q) ++i;
+  return i;
+}
 
 // Biased exponent field of the high word of a double.
 __host__ __device__ __forceinline__ int field_of(uint32_t hi) { return (int)((hi >> 20) & 0x7FFu); }

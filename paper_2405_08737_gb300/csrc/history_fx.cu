@@ -7,15 +7,24 @@
 // (G^< = PL, G^> = PL + Q), A1[m] = w_{n,m} (S^> - S^<)[m], NB[m] = -wbar_m S^<[m]:
 //   far  (m <= c - band_w): I^< += A1 PL + NB Q          (both components alike)
 //   near (m >  c - band_w): I^< += A1 PL,  D += A1 Q      (I^> = I^< + D)
-// and the band of term 2, w_{c,m} S^s R(c,m)^+ for c - band_w < m <= c, is added
-// in FP64 by the reduction: two real products of 128-row tiles per history point.
+//   band (c - band_w < m <= c): I^< += S^< w_{c,m} R(c,m)^+,  D += (S^> - S^<) w_{c,m} R(c,m)^+
+// -- two real products of 128-row tiles per history point.
+//
+// The adjoint of the slice (adjoint.cu) has the same form with the roles of c
+// and m exchanged.  With J = Ibar^< + Ibar^> and the planes' adjoints in place of
+// the planes (signs and the diagonal as noted at load_quad and fx_prep):
+//   A1bar[m] = sum_{c < m + band_w} (J PL^+ + Ibar^> Q^+) - sum_{c >= m + band_w} J L(c,m),
+//   C[m]     = sum_{c >= m} w_{c,m} J R(c,m),
+//   S^>bar[m] = w_{n,m} A1bar[m] + sum_{band} w_{c,m} Ibar^> R(c,m),   S^<bar[m] = C[m] - S^>bar[m]
+// (the settled columns as in adj_hist_small): the same far, near and band parts,
+// with the sums of the first two scaled by w_{n,m} and wbar_m before the band.
 //
 // Why: FP64 runs at 1.26 TFLOP/s on this part (152 SMs x 2 FMA), the fp16
 // tensor cores at about 1900, so 36 digit products cost a fiftieth of the FP64
 // ones.  What bounds it then is the conversion: every history entry is read in
 // both orientations and cut into digits with about 30 integer instructions per
-// real.  Measured: the slice n = 1023, M = 8 in 0.87 ms, 0.97 with the kernels around
-// it, where the same sums on the FP64 pipe (history_f64.cu) take 7.08 ms.
+// real.  Measured, in this kernel: the slice n = 1023, M = 8 in 0.89 ms (7.05 on the
+// FP64 pipe, history_f64.cu), n = 511, M = 16 in 1.30 ms (14.4).
 //
 // One persistent CTA per SM takes a contiguous range of chunks (32 history
 // entries of a 128-row column tile).  A unit is 8 entries, one MMA K step:
@@ -27,10 +36,13 @@
 //  * one thread copies the small operand's digits of each unit (bulk copies);
 //  * one thread issues the MMAs: digit i of the history against the stacked
 //    digits 0..7-i of the small operand, so the products of level i + j land in
-//    the columns of that level (N = 2 kNA (8 - i));
+//    the columns of that level (N = 2 NA (8 - i) for a part of NA rows a);
 //  * eight epilogue warps fold a chunk's eight integer levels into one 64-bit
 //    integer, and that, scaled, into FP64 sums in registers: two FP64
 //    operations per 32 entries of an output.
+// Parts of NA = 8 rows a for M <= 8, else 16: a part's conversion of the history
+// serves all its rows (two sums of 16 x 8 levels fill tensor memory, so with NA =
+// 16 a near chunk waits for the epilogue of the one before).
 // A row's exponent holds for the units accumulated together in tensor memory.
 // It starts kHeadroom bits above the larger of the unit's and the previous
 // chunk's largest entry; a unit that exceeds it nevertheless closes the
@@ -44,8 +56,7 @@
 #include <algorithm>
 #include <atomic>
 
-#include "fx_common.cuh"
-#include "kbe_internal.h"
+#include "history_fx.h"
 #include "row_kernels.cuh"
 #include "split_common.cuh"
 
@@ -67,73 +78,93 @@ using split::umma_desc;
 using split::umma_f16;
 using split::umma_idesc_f16;
 
-constexpr int kNA = 8;                                    // a values per part
-constexpr int kN = 2 * kNA;                               // real columns per digit of the small operand
 constexpr int kDigPlane = kRows * 2 * kUnitK * 2;         // one digit of one plane: 4 KB
 constexpr int kPlane = kDig * kDigPlane;                  // 32 KB
-constexpr int kVarBytes = 2 * kDig * (kN / 8) * 128;      // one variant's digits of a unit: 4 KB
-constexpr int kExpBytes = 64;                             // exponents of the part's a values (int16), padded
-constexpr int kSmallBytes = kExpBytes + 2 * kVarBytes;    // small block of a unit: exponents | A1 | NB
-constexpr int kBufCols = kDig * kN;                       // accumulator buffer: 8 levels x kN columns
-constexpr int kBufs = 512 / kBufCols;
+constexpr int kExpBytes = 64;                             // exponents of a part's a values (int16), padded
 constexpr int kStages = 2, kBSlots = 4, kExpRing = 32;
 constexpr int kEpiWarps = 8;
 constexpr int kConvWarps = 16;                            // 8 rows each
 constexpr int kMmaWarp = kEpiWarps + kConvWarps, kProdWarp = kMmaWarp + 1;
-constexpr int kThreads = (kProdWarp + 1) * 32;
-constexpr int kMaxCtas = 160;
+constexpr int kThreads = (kProdWarp + 3) * 32;            // whole warpgroups (setmaxnreg): 896
 constexpr long long kSpinLimit = 1ll << 22;               // polls of the final waits
 constexpr long long kWaitCycles = 1ll << 31;              // a work wait gives up after about a second
-constexpr size_t kSlotDoubles = 2 * 2 * (size_t)kNA * kRows;  // partial sums of one (CTA, tile): [2][kNA][128] complex
-// an epilogue still reading a group's exponents is at most kStages units and
-// kBufs + 1 groups behind the converters
-static_assert(kStages + kChunkUnits * (kBufs + 1) < kExpRing, "exponent ring");
+// registers of the warpgroups with NA = 16 (setmaxnreg; sums of 32 FP64 values a
+// thread): 8 x 32 x 104 + 16 x 32 x 64 + 4 x 32 x 40 = 896 x 72, the launch's own
+constexpr int kRegsEpi = 104, kRegsConv = 64, kRegsMisc = 40;
+
+template <int NA>
+struct Cfg {
+  static constexpr int kN = 2 * NA;                              // real columns per digit of the small operand
+  static constexpr int kVarBytes = 2 * kDig * (kN / 8) * 128;    // one variant's digits of a unit
+  static constexpr int kHalfBytes = kExpBytes + 2 * kVarBytes;   // exponents | variant 0 | variant 1
+  static constexpr int kSmallBytes = 2 * kHalfBytes;             // small block of a unit: main half, band half
+  static constexpr int kBufCols = kDig * kN;                     // accumulator buffer: 8 levels x kN columns
+  static constexpr int kBufs = 512 / kBufCols;
+  static constexpr size_t kSlot = 2 * (size_t)NA * kRows;        // partial sums of one (CTA, tile): [2][NA][128] complex
+  // an epilogue still reading a group's exponents is at most kStages units and
+  // the open and the buffered groups (4 units a buffer) behind the converters
+  static_assert(kStages + kChunkUnits * (kBufs + 2) < kExpRing, "exponent ring");
+};
 
 // What the producer thread hands to the converters and the MMA thread with each
-// slot of the small operand's ring: a unit, the end of a segment (a CTA's part
-// of a tile: its sums go to `aux`), or the end of the range.
-enum DescKind { kUnit = 0, kFlush = 1, kEnd = 2 };
-enum DescFlags { kNear = 1, kFirst = 2, kLast = 4, kFresh = 8, kNewTile = 16 };
+// slot of the small operand's ring: a unit, the scaling of an adjoint's sums
+// before the band, the end of a segment (a CTA's part of a tile: its sums go to
+// partial slot `aux`), or the end of the range.
+enum DescKind { kUnit = 0, kScale = 1, kFlush = 2, kEnd = 3 };
+enum DescFlags { kFlagNear = 1, kFlagBand = 2, kFirst = 4, kLast = 8, kFresh = 16, kNewTile = 32 };
 struct alignas(16) Desc {
   int kap;    // first history entry
   int c0;     // first column of the tile
   int flags;  // kind << 8 | DescFlags (first, last unit of its chunk; no chunk to follow; new tile)
-  int aux;    // system of the launch, or the partial slot (flush)
+  int aux;    // system of the launch; partial slot (flush)
 };
 
-enum PostType { kPostSum = 0, kPostFlush = 1, kPostExit = 2 };
 struct alignas(16) Post {  // what the MMA thread hands to the epilogue with a buffer
-  int type, grp, eidx; // sum group (0: I^<, 1: D), exponent ring index
-  int slot;            // partial slot (flush)
-  int16_t es[kNA];     // small operand's exponents
+  int type;                // kUnit (sums), kScale, kFlush, kEnd
+  int grp, eidx, plane;    // sum group (0: I^<, 1: D), exponent ring index and plane
+  int si, c0, slot, pad;   // system; first column (scale); partial slot (flush)
+  int16_t es[16];          // small operand's exponents
 };
 
+template <int NA>
 struct Smem {
   uint8_t stage[kStages][2 * kPlane];
-  uint8_t small[kBSlots][kSmallBytes];
+  uint8_t small[kBSlots][Cfg<NA>::kHalfBytes];
   int16_t erow[kExpRing][2][kRows];   // row exponents of a unit, per plane
-  Post post[kBufs];
+  Post post[Cfg<NA>::kBufs];
   Desc desc[kBSlots];
-  uint64_t full[kStages], empty[kStages], bfull[kBSlots], bempty[kBSlots], accfull[kBufs], accempty[kBufs], mmadone;
+  uint64_t full[kStages], empty[kStages], bfull[kBSlots], bempty[kBSlots];
+  uint64_t accfull[Cfg<NA>::kBufs], accempty[Cfg<NA>::kBufs], mmadone;
   unsigned raise[kStages];            // 1 + the unit whose exponents start a new accumulation
   uint32_t tmem;
   int abort;
 };
 
+// The systems of a launch: one, by value, or a table and its head in device memory.
 struct Args {
-  Sys one;               // the system of a single-system launch
-  const Sys* table;      // or the systems of the launch, in order (device memory)
-  int n_sys, G;
-  long long total;       // chunk slots of the launch
-  double* part;
-  int* status;
-  long long spin;
+  Sys one;
+  Head one_head;
+  const Sys* table;
+  const Head* head;
+  int G;
 };
+__device__ __forceinline__ const Sys& sys_at(const Args& a, int i) { return a.table ? a.table[i] : a.one; }
+__device__ __forceinline__ const Head& head_of(const Args& a) { return a.table ? *a.head : a.one_head; }
+// last system whose base (one of the Sys members) is at most x
+template <class F>
+__device__ __forceinline__ int find_sys(const Args& a, long long x, F base) {
+  int lo = 0, hi = head_of(a).n_sys;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (base(sys_at(a, mid)) <= x) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+__device__ __forceinline__ WeightsView weights_of(const Sys& s) { return WeightsView{s.wbar, s.band, s.band_w}; }
 
-// Waits for a phase of a barrier, suspended by the hardware between polls (most
-// warps of this kernel wait most of the time: polling without suspension took
-// a large part of the issue slots).  Gives up after `limit` clock cycles.
-__device__ __forceinline__ bool mbar_try_suspend(uint64_t* bar, uint32_t parity) {
+// Waits for a phase of a barrier, suspended by the hardware between polls.
+// Gives up after kWaitCycles, or when another role has.
+__device__ __forceinline__ bool try_suspend(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}"
@@ -142,50 +173,27 @@ __device__ __forceinline__ bool mbar_try_suspend(uint64_t* bar, uint32_t parity)
       : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ bool wait_bar(Smem& sm, uint64_t* bar, uint32_t parity, int* status, long long limit) {
-  if (mbar_try_suspend(bar, parity)) return true;
+__device__ __forceinline__ bool wait_bar(int* abort, uint64_t* bar, uint32_t parity, int* status) {
+  if (try_suspend(bar, parity)) return true;
   const long long t0 = clock64();
-  while (!mbar_try_suspend(bar, parity)) {
-    const bool late = clock64() - t0 > limit;
-    if (late || *(volatile int*)&sm.abort) {
-      if (late) { atomicOr(status, kStatusTimeout); sm.abort = 1; }
+  while (!try_suspend(bar, parity)) {
+    const bool late = clock64() - t0 > kWaitCycles;
+    if (late || *(volatile int*)abort) {
+      if (late) { atomicOr(status, kStatusTimeout); *(volatile int*)abort = 1; }
       return false;
     }
   }
   return true;
 }
 
-// A role's position: chunk slot q of the launch and where it lies.
-struct Cursor {
-  long long q;
-  Walk w;
-};
-__device__ __forceinline__ const Sys& sys_at(const Args& a, int i) { return a.table ? a.table[i] : a.one; }
-__device__ __forceinline__ Cursor cursor_at(const Args& a, long long q) {
-  Cursor c;
-  int lo = 0, hi = a.n_sys;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (sys_at(a, mid).unit_base <= q) lo = mid; else hi = mid;
-  }
-  c.q = q;
-  walk_to(c.w, sys_at(a, lo), lo, q - sys_at(a, lo).unit_base);
-  return c;
-}
-// The next chunk slot (before `end`, or its place is not evaluated); true when
-// it is in another tile or at the end.
-__device__ __forceinline__ bool cursor_next(const Args& a, Cursor& c, long long end) {
-  if (++c.q >= end) return true;
-  const int moved = walk_next(c.w);
-  if (moved == 2) walk_to(c.w, sys_at(a, c.w.si + 1), c.w.si + 1, 0);
-  return moved != 0;
-}
-
 // ---------------------------------------------------------------- prep ---
-// fp16 pair (digit of x, digit of y): byte `B` of two digit words, minus 1152
+// fp16 pair (digit of x, digit of y): byte `B` of two digit words, each put into
+// the low mantissa bits of 1024, minus 1152
 template <int B>
 __device__ __forceinline__ uint32_t digit_pair(uint32_t x, uint32_t y) {
-  const uint32_t w = (__byte_perm(x, y, B | ((B + 4) << 8)) & 0x00FF00FFu) | 0x64006400u;
+  // bytes (x, y) of B and B ^ 1 side by side: shared by the two digits
+  const uint32_t xy = __byte_perm(x, y, (B & 2) | ((B & 2) + 4) << 4 | ((B & 2) + 1) << 8 | ((B & 2) + 5) << 12);
+  const uint32_t w = __byte_perm(xy, 0x64646464u, (B & 1) ? 0x4342 : 0x4140);
   uint32_t r;
   asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(w), "r"(0x64806480u));
   return r;
@@ -209,56 +217,88 @@ __device__ __forceinline__ uint64_t bytes_of(double v, int E) {
 }
 __device__ __forceinline__ int field64(double v) { return field_of((uint32_t)__double2hiint(v)); }
 
-// Small operands of chunk kc, part p (grid: chunk x part; warp = a, lane =
-// entry of the chunk): A1 and NB with one exponent per a and chunk, in the real
-// form of a complex product, columns (a, re): (P.re, -P.im), (a, im): (P.im, P.re)
-// over the entry's (re, im).  Layout of a variant of a unit: [K group 2][digit
-// 8][column group 2][8 columns][8 reals].
-__global__ void __launch_bounds__(32 * kNA) fx_prep(Sys s, const double* __restrict__ Sl,
-                                                    const double* __restrict__ Sg, WeightsView w,
-                                                    uint8_t* __restrict__ small) {
-  const int M = s.M, MM = M * M, n = s.n;
-  const int kc = blockIdx.x, p = blockIdx.y, al = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int kap = kc * kChunkK + lane, a = p * kNA + al;
-  const int m = div_m(kap, M, s.magic), x = kap - m * M;
-  double v[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-  if (m <= n && a < M) {
-    const double2 l = reinterpret_cast<const double2*>(Sl)[(size_t)m * MM + a * M + x];
-    const double2 g = reinterpret_cast<const double2*>(Sg)[(size_t)m * MM + a * M + x];
-    const double wn = w.at(n, m), wb = -w.wbar[m];
-    v[0][0] = wn * (g.x - l.x); v[0][1] = wn * (g.y - l.y);
-    v[1][0] = wb * l.x; v[1][1] = wb * l.y;
-  }
-  int E = max(max(field64(v[0][0]), field64(v[0][1])), max(field64(v[1][0]), field64(v[1][1])));
-  E = __reduce_max_sync(0xffffffffu, E);
-  E = E == 0x7FF ? kNonFinite : max(E, 64);
-  const int unit = kc * kChunkUnits + lane / kUnitK, kl = lane % kUnitK;
-  uint8_t* blk = small + ((size_t)unit * s.parts + p) * kSmallBytes;
-  if (kl == 0) reinterpret_cast<int16_t*>(blk)[al] = (int16_t)E;
-  const int kg = kl >> 2, kin = 2 * (kl & 3);
-  const int cre = 2 * al, cim = 2 * al + 1;
+// Small operands of a pair of chunks and a part (grid-stride over them; warp = a,
+// a lane has one entry of each chunk), with one exponent per a, pair and half
+// (near sums accumulate over the pair), in the real form
+// of a complex product: columns (a, re): (P.re, -P.im), (a, im): (P.im, P.re) over
+// the entry's (re, im).  Layout of a variant of a unit: [K group 2][digit 8]
+// [column group][8 columns][8 reals].  With (l, g) = (S^<, S^>), resp. (Ibar^<, Ibar^>):
+//   slice    main w_{n,m} (g - l), -wbar_m l    band l, g - l
+//   adjoint  main -(l + g), -g                  band g, l + g
+template <int NA>
+__global__ void __launch_bounds__(32 * NA) fx_prep(const __grid_constant__ Args a) {
+  using C = Cfg<NA>;
+  const int al = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long long chunks = head_of(a).chunks;
+  for (long long ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
+    const Sys& s = sys_at(a, find_sys(a, ch, [](const Sys& y) { return y.chunk_base; }));
+    const int M = s.M, MM = M * M, n = s.n, parts = s.parts;
+    const int pair = (int)((ch - s.chunk_base) / parts), p = (int)(ch - s.chunk_base - (long long)pair * parts);
+    const int row = p * NA + al;
+    double2 l[2], g[2];
+    double w0[2] = {1.0, 1.0}, w1[2] = {1.0, 1.0};
 #pragma unroll
-  for (int var = 0; var < 2; ++var) {
-    const uint64_t br = bytes_of(v[var][0], E), bi = bytes_of(v[var][1], E);
+    for (int k = 0; k < 2; ++k) {
+      const int kap = (2 * pair + k) * kChunkK + lane;
+      const int m = div_m(kap, M, s.magic), x = kap - m * M;
+      l[k] = g[k] = make_double2(0.0, 0.0);
+      if (m <= n && row < M) {
+        l[k] = reinterpret_cast<const double2*>(s.Sl)[(size_t)m * MM + row * M + x];
+        g[k] = reinterpret_cast<const double2*>(s.Sg)[(size_t)m * MM + row * M + x];
+        if (!s.adj) {
+          w0[k] = weights_of(s).at(n, m);
+          w1[k] = s.wbar[m];
+        }
+      }
+    }
+    const int kl = lane % kUnitK, kg = kl >> 2, kin = 2 * (kl & 3), cre = 2 * al, cim = 2 * al + 1;
 #pragma unroll
-    for (int d = 0; d < kDig; ++d) {
-      const uint32_t ri = digit_of(d, br, bi);              // (re, im)
-      const uint32_t re = ri & 0xFFFFu, im = ri >> 16;
-      uint8_t* base = blk + kExpBytes + var * kVarBytes + (kg * kDig + d) * (kN / 8) * 128 + kin * 2;
-      *reinterpret_cast<uint32_t*>(base + (cre >> 3) * 128 + (cre & 7) * 16) = re | ((im ^ 0x8000u) << 16);
-      *reinterpret_cast<uint32_t*>(base + (cim >> 3) * 128 + (cim & 7) * 16) = im | (re << 16);
+    for (int half = 0; half < 2; ++half) {
+      double v[2][2][2];  // [chunk][variant][re, im]
+      int E = 0;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const double dx = g[k].x - l[k].x, dy = g[k].y - l[k].y, sx = l[k].x + g[k].x, sy = l[k].y + g[k].y;
+        v[k][0][0] = s.adj ? (half ? g[k].x : -sx) : (half ? l[k].x : w0[k] * dx);
+        v[k][0][1] = s.adj ? (half ? g[k].y : -sy) : (half ? l[k].y : w0[k] * dy);
+        v[k][1][0] = s.adj ? (half ? sx : -g[k].x) : (half ? dx : -w1[k] * l[k].x);
+        v[k][1][1] = s.adj ? (half ? sy : -g[k].y) : (half ? dy : -w1[k] * l[k].y);
+        E = max(E, max(max(field64(v[k][0][0]), field64(v[k][0][1])), max(field64(v[k][1][0]), field64(v[k][1][1]))));
+      }
+      E = __reduce_max_sync(0xffffffffu, E);
+      E = E == 0x7FF ? kNonFinite : max(E, 64);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        if (2 * pair + k >= s.cpt) break;
+        const int unit = (2 * pair + k) * kChunkUnits + lane / kUnitK;
+        uint8_t* out = s.small + ((size_t)unit * parts + p) * C::kSmallBytes + half * C::kHalfBytes;
+        if (kl == 0) reinterpret_cast<int16_t*>(out)[al] = (int16_t)E;
+#pragma unroll
+        for (int var = 0; var < 2; ++var) {
+          const uint64_t br = bytes_of(v[k][var][0], E), bi = bytes_of(v[k][var][1], E);
+#pragma unroll
+          for (int d = 0; d < kDig; ++d) {
+            const uint32_t ri = digit_of(d, br, bi);              // (re, im)
+            const uint32_t re = ri & 0xFFFFu, im = ri >> 16;
+            uint8_t* base = out + kExpBytes + var * C::kVarBytes + (kg * kDig + d) * (C::kN / 8) * 128 + kin * 2;
+            *reinterpret_cast<uint32_t*>(base + (cre >> 3) * 128 + (cre & 7) * 16) = re | ((im ^ 0x8000u) << 16);
+            *reinterpret_cast<uint32_t*>(base + (cim >> 3) * 128 + (cim & 7) * 16) = im | (re << 16);
+          }
+        }
+      }
     }
   }
 }
 
 // ---------------------------------------------------------- converters ---
 // A lane's place in a column tile: its row (c, b) of one plane, and where the
-// row's entries lie: `tr` + m M^2 + x for m < c (block (c, m), transposed), and
-// `dr` + m (m + 1) / 2 M^2 + x M for m >= c (block (m, c)).
+// row's entries lie: `tr` + m M^2 + x above the diagonal (m < diag: block (c, m),
+// transposed), and `dr` + m (m + 1) / 2 M^2 + x M below it (block (m, c)).
 struct Row {
   const double2* tr;
   const double2* dr;
-  int c, n, edge;   // column, last history point (-1: no such row), c + shift
+  int n, edge;      // last point (-1: no such row), c + shift
+  int diag;         // first point that is read directly: c, in the adjoint c + 1
   int M;
   uint32_t magic;
 };
@@ -268,17 +308,18 @@ __device__ __forceinline__ Row row_of(const Sys& s, int c0, int j, int plane) {
   r.M = s.M;
   r.magic = s.magic;
   const int cl = div_m(j, r.M, r.magic), b = j - cl * r.M, MM = r.M * r.M;
-  r.c = c0 + cl;
-  const bool live = cl < s.CT && r.c <= s.n;
+  const int c = c0 + cl;
+  const bool live = cl < s.CT && c <= s.n;
   r.n = live ? s.n : -1;
-  r.edge = r.c + s.shift;
-  r.tr = base + (live ? tri(r.c, 0) * MM + b * r.M : 0);
-  r.dr = base + (live ? (int64_t)r.c * MM + b : 0);
+  r.edge = c + s.shift;
+  r.diag = c + s.adj;
+  r.tr = base + (live ? tri(c, 0) * MM + b * r.M : 0);
+  r.dr = base + (live ? (int64_t)c * MM + b : 0);
   return r;
 }
 // Four consecutive entries from kap of a row; `mask` has bit i set where entry
-// i counts, bit 4 + i where it lies above the diagonal (the entry is then -conj
-// of the stored one).  kQuad (M a multiple of 4): the four share their history
+// i counts, bit 4 + i where it lies above the diagonal (the entry of the plane is
+// then -conj of the stored one).  kQuad (M a multiple of 4): the four share their
 // point m; masked entries load something valid instead of branching.
 template <bool kQuad>
 __device__ __forceinline__ void load_quad(const Row& r, int kap, bool near, double2 z[4], unsigned& mask) {
@@ -286,7 +327,7 @@ __device__ __forceinline__ void load_quad(const Row& r, int kap, bool near, doub
   int m = div_m(kap, M, r.magic), x = kap - m * M;
   if (kQuad) {
     const bool in = m <= r.n && (near ? m > r.edge : m <= r.edge);
-    const bool above = m < r.c;
+    const bool above = m < r.diag;
     const double2* p = above ? r.tr + (m * MM + x) : r.dr + (tri(m, 0) * MM + x * M);
     int st = above ? 1 : M;
     if (!in) { p = r.tr; st = 1; }
@@ -299,21 +340,45 @@ __device__ __forceinline__ void load_quad(const Row& r, int kap, bool near, doub
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const bool in = m <= r.n && (near ? m > r.edge : m <= r.edge);
-    const bool above = m < r.c;
+    const bool above = m < r.diag;
     z[i] = make_double2(0.0, 0.0);
     if (in) z[i] = __ldg(above ? r.tr + (m * MM + x) : r.dr + (tri(m, 0) * MM + x * M));
     mask |= ((unsigned)in | ((unsigned)above << 4)) << i;
     if (++x == M) { x = 0; ++m; }
   }
 }
+// Four entries of the band of term 2 (plane R): w_{c,m} R(c,m)^+ for c - band_w < m
+// <= c, in the adjoint w_{m,c} R(m,c) for c <= m < c + band_w.
+__device__ __noinline__ unsigned load_band(const Sys& s, const Row& r, int c, int kap, double2 z[4]) {
+  const int M = r.M, MM = M * M, bw = s.band_w;
+  int m = div_m(kap, M, r.magic), x = kap - m * M;
+  unsigned mask = 0;
+  for (int i = 0; i < 4; ++i) {
+    const int hi = s.adj ? m : c, lo = s.adj ? c : m;
+    const bool in = m <= r.n && lo <= hi && hi - lo < bw;
+    z[i] = make_double2(0.0, 0.0);
+    if (in) {
+      const double w = s.band[(int64_t)hi * bw + (hi - lo)];
+      const double2 v = __ldg(s.adj ? r.dr + (tri(m, 0) * MM + x * M) : r.tr + (m * MM + x));
+      z[i] = make_double2(w * v.x, s.adj ? w * v.y : -w * v.y);
+    }
+    mask |= (unsigned)in << i;
+    if (++x == M) { x = 0; ++m; }
+  }
+  return mask;
+}
 
 // ---------------------------------------------------------------- main ---
-template <bool kQuad>
+template <int NA, bool kQuad>
 __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ Args a) {
+  using C = Cfg<NA>;
+  constexpr int kN = C::kN, kBufs = C::kBufs, kBufCols = C::kBufCols;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+  Smem<NA>& sm = *reinterpret_cast<Smem<NA>*>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long q0 = range_lo(a.total, a.G, blockIdx.x), q1 = range_lo(a.total, a.G, blockIdx.x + 1);
+  const long long total = head_of(a).total;
+  const long long q0 = range_lo(total, a.G, blockIdx.x), q1 = range_lo(total, a.G, blockIdx.x + 1);
+  int* const status = sys_at(a, 0).status;
 
   if (tid == 0) {
     for (int i = 0; i < kStages; ++i) { mbar_init(&sm.full[i], kConvWarps); mbar_init(&sm.empty[i], 1); sm.raise[i] = 0; }
@@ -339,7 +404,8 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
     // --------------------------------------------------------- epilogue --
     // warp = 4 half + quadrant: 32 output rows (tensor-memory lanes), half of
     // the part's a values (kN / 2 columns)
-    constexpr int kC = kN / 2;
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
+    constexpr int kC = kN / 2, kCols = NA == 8 ? 2 : 1;  // columns in registers at a time
     const int quad = warp & 3, half = warp >> 2;
     const int j = quad * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16) + half * kC;
@@ -348,63 +414,84 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
     for (int i = 0; i < kC; ++i) acc[0][i] = acc[1][i] = 0.0;
     for (unsigned p = 0;; ++p) {
       const int buf = p % kBufs;
-      if (!__all_sync(0xffffffffu, wait_bar(sm, &sm.accfull[buf], (p / kBufs) & 1, a.status, a.spin))) break;
+      if (!__all_sync(0xffffffffu, wait_bar(&sm.abort, &sm.accfull[buf], (p / kBufs) & 1, status))) break;
       tc_fence_after();
       const Post& ps = sm.post[buf];
       const int type = ps.type;
-      if (type == kPostExit) break;
-      if (type == kPostFlush) {
-        double2* out = reinterpret_cast<double2*>(a.part + (size_t)ps.slot * kSlotDoubles);
+      if (type == kEnd) break;
+      if (type != kUnit) {
+        const Sys& s = sys_at(a, ps.si);
+        if (type == kFlush) {
+          double2* out = reinterpret_cast<double2*>(s.part) + (size_t)ps.slot * C::kSlot;
 #pragma unroll
-        for (int g = 0; g < 2; ++g)
+          for (int g = 0; g < 2; ++g)
 #pragma unroll
-          for (int i = 0; i < kC / 2; ++i) {
-            out[(g * kNA + half * (kNA / 2) + i) * kRows + j] = make_double2(acc[g][2 * i], acc[g][2 * i + 1]);
-            acc[g][2 * i] = acc[g][2 * i + 1] = 0.0;
+            for (int i = 0; i < kC / 2; ++i) {
+              out[(g * NA + half * (NA / 2) + i) * kRows + j] = make_double2(acc[g][2 * i], acc[g][2 * i + 1]);
+              acc[g][2 * i] = acc[g][2 * i + 1] = 0.0;
+            }
+        } else {  // the adjoint's sums, before its band
+          const int m = min(ps.c0 + div_m(j, s.M, s.magic), s.n);
+          const double wn = weights_of(s).at(s.n, m), wb = -s.wbar[m];
+#pragma unroll
+          for (int i = 0; i < kC; ++i) {
+            acc[0][i] *= wn;
+            acc[1][i] *= wb;
           }
+        }
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.accempty[buf]);
         continue;
       }
       const int g = ps.grp;
-      const int E = sm.erow[ps.eidx][g][j];
-      int es[kC / 2];
+      const int E = sm.erow[ps.eidx][ps.plane][j];
+      // the levels of kCols columns from column c2 of the buffer
+      uint32_t r[kDig][kCols];
+      auto read = [&](int c2) {
 #pragma unroll
-      for (int i = 0; i < kC / 2; ++i) es[i] = ps.es[half * (kNA / 2) + i];
+        for (int d = 0; d < kDig; ++d) {
+          const uint32_t at = lane_addr + buf * kBufCols + d * kN + c2;
+          if constexpr (kCols == 2)
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(r[d][0]), "=r"(r[d][kCols - 1]) : "r"(at));
+          else
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[d][0]) : "r"(at));
+        }
+      };
       auto fold = [&](double(&s)[kC]) {
+        read(0);
 #pragma unroll
-        for (int c4 = 0; c4 < kC; c4 += 2) {
-          uint32_t r[kDig][2];
-#pragma unroll
-          for (int d = 0; d < kDig; ++d)
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];"
-                         : "=r"(r[d][0]), "=r"(r[d][1])
-                         : "r"(lane_addr + buf * kBufCols + d * kN + c4));
+        for (int c2 = 0; c2 < kC; c2 += kCols) {
+          const int es = ps.es[half * (NA / 2) + c2 / 2];
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          if (c4 + 2 == kC) {  // every level of this buffer is in registers
+          int v[kDig][kCols];
+#pragma unroll
+          for (int i = 0; i < kCols; ++i)
+#pragma unroll
+            for (int d = 0; d < kDig; ++d) v[d][i] = __float2int_rn(__uint_as_float(r[d][i]));
+          if (c2 + kCols < kC) {
+            read(c2 + kCols);  // in flight while these are folded
+          } else {             // every level of this buffer is in registers
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.accempty[buf]);
           }
+          // scale 2^(ev + eu - 68 + 12), ev = E - 1022, eu = es - 1022
+          const int ex = E + es - 2 * 1022 - 56;
 #pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            int v[kDig];
-#pragma unroll
-            for (int d = 0; d < kDig; ++d) v[d] = __float2int_rn(__uint_as_float(r[d][i]));
+          for (int i = 0; i < kCols; ++i) {
             // the 64-bit integer sum_l S_l 256^(7-l) / 2^12: |S_0| <= 2^19, |S_1| <= 2^21, |S_2| <= 2^22 and
             // |S_l| <= l 2^21 fit the 32-bit steps, and 2^10 products of 62-bit values stay below 2^(124+7-56-12)
-            const uint64_t p01 = (uint64_t)(int64_t)(v[0] * 256 + v[1]), p23 = (uint64_t)(int64_t)(v[2] * 256 + v[3]);
-            const int low = v[5] * 16 + ((v[6] + (v[7] >> 8) + 8) >> 4);
-            const int64_t t = (int64_t)((p01 << 36) + (p23 << 20) + ((uint64_t)(int64_t)v[4] << 12) + (uint64_t)(int64_t)low);
-            // scale 2^(ev + eu - 68 + 12), ev = E - 1022, eu = es - 1022
-            const int ex = E + es[(c4 + i) / 2] - 2 * 1022 - 56;
+            const uint64_t p01 = (uint64_t)(int64_t)(v[0][i] * 256 + v[1][i]), p23 = (uint64_t)(int64_t)(v[2][i] * 256 + v[3][i]);
+            const int low = v[5][i] * 16 + ((v[6][i] + (v[7][i] >> 8) + 8) >> 4);
+            const int64_t t =
+                (int64_t)((p01 << 36) + (p23 << 20) + ((uint64_t)(int64_t)v[4][i] << 12) + (uint64_t)(int64_t)low);
             if (ex >= -1022 && ex <= 1023) {
-              s[c4 + i] = fma((double)t, __hiloint2double((ex + 1023) << 20, 0), s[c4 + i]);
+              s[c2 + i] = fma((double)t, __hiloint2double((ex + 1023) << 20, 0), s[c2 + i]);
             } else if (ex >= kNonFinite - 4096) {
-              s[c4 + i] = __longlong_as_double(0x7FF8000000000000ll);
+              s[c2 + i] = __longlong_as_double(0x7FF8000000000000ll);
             } else {  // the scale alone leaves the range of FP64
               const int h = ex / 2;
-              s[c4 + i] += (double)t * __hiloint2double((h + 1023) << 20, 0) * __hiloint2double((ex - h + 1023) << 20, 0);
+              s[c2 + i] += (double)t * __hiloint2double((h + 1023) << 20, 0) * __hiloint2double((ex - h + 1023) << 20, 0);
             }
           }
         }
@@ -415,6 +502,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
     // ------------------------------------------------------- converters --
     // lane = row (3 bits) | K half q << 3 | plane << 4: a quarter warp writes
     // 128 consecutive bytes of a digit plane
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsConv));
     const int wq = warp - kEpiWarps;
     const int q = (lane >> 3) & 1, plane = lane >> 4;
     const uint32_t dst0 = plane * kPlane + (q * 16 + wq) * 128 + (lane & 7) * 16;
@@ -427,14 +515,24 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       Desc ds;
       do {
         const int b = d % kBSlots;
-        if (!__all_sync(0xffffffffu, wait_bar(sm, &sm.bfull[b], (d / kBSlots) & 1, a.status, a.spin))) return false;
+        if (!__all_sync(0xffffffffu, wait_bar(&sm.abort, &sm.bfull[b], (d / kBSlots) & 1, status))) return false;
         ds = sm.desc[b];
         ++d;
-      } while (ds.flags >> 8 == kFlush);
+      } while (ds.flags >> 8 == kFlush || ds.flags >> 8 == kScale);
       flags = ds.flags;
       if (flags >> 8 == kEnd) return false;
       if (flags & kNewTile) row = row_of(sys_at(a, ds.aux), ds.c0, 8 * wq + (lane & 7), plane);
-      load_quad<kQuad>(row, ds.kap + 4 * q, flags & kNear, z, mask);
+      const int kap = ds.kap + 4 * q;
+      if (flags & kFlagBand) {
+        double2 v[4];
+        const int c = ds.c0 + div_m(8 * wq + (lane & 7), row.M, row.magic);
+        mask = plane ? load_band(sys_at(a, ds.aux), row, c, kap, v) : 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) z[i] = plane ? v[i] : make_double2(0.0, 0.0);
+        if (mask) mask = 15u;  // the others are zero
+      } else {
+        load_quad<kQuad>(row, kap, flags & kFlagNear, z, mask);
+      }
       return true;
     };
     bool more = load();
@@ -451,7 +549,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       mx >>= 20;
       mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
       const int other = __shfl_xor_sync(0xffffffffu, mx, 16);
-      if (!(flags & kNear)) mx = max(mx, other);
+      if (!(flags & (kFlagNear | kFlagBand))) mx = max(mx, other);
       bool raised = false;
       if (flags & kFirst) {
         const int prev = (flags & kFresh) || seen == 0x7FF ? 0 : seen;
@@ -472,7 +570,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
         bi[i] = digit_bytes((uint32_t)__double2hiint(z[i].y), (uint32_t)__double2loint(z[i].y), Ez);
       }
       more = load();  // in flight while this unit's digits are written
-      if (!__all_sync(0xffffffffu, wait_bar(sm, &sm.empty[s], ((u / kStages) & 1) ^ 1, a.status, a.spin))) break;
+      if (!__all_sync(0xffffffffu, wait_bar(&sm.abort, &sm.empty[s], ((u / kStages) & 1) ^ 1, status))) break;
       if (__any_sync(0xffffffffu, raised) && lane == 0) *(volatile unsigned*)&sm.raise[s] = u + 1;
       if (q == 0) sm.erow[u % kExpRing][plane][8 * wq + (lane & 7)] = (int16_t)E;
       uint8_t* dst = sm.stage[s] + dst0;
@@ -485,62 +583,91 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.full[s]);
     }
-  } else if (warp == kProdWarp) {
-    // --------------------------------------------------------- producer --
-    if (lane == 0) {
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsMisc));
+    if (warp == kProdWarp && lane == 0) {
+      // ------------------------------------------------------- producer --
       unsigned d = 0;
       // the next slot, its descriptor written; false when the wait ran out
       auto put = [&](int kap, int c0, int flags, int aux) -> bool {
         const int b = d % kBSlots;
-        if (!wait_bar(sm, &sm.bempty[b], ((d / kBSlots) & 1) ^ 1, a.status, a.spin)) return false;
+        if (!wait_bar(&sm.abort, &sm.bempty[b], ((d / kBSlots) & 1) ^ 1, status)) return false;
         sm.desc[b] = Desc{kap, c0, flags, aux};
         return true;
       };
+      auto message = [&](int kind, int kap, int c0, int aux) -> bool {
+        if (!put(kap, c0, kind << 8, aux)) return false;
+        mbar_arrive(&sm.bfull[d++ % kBSlots]);
+        return true;
+      };
       bool stop = false;
-      Cursor c = cursor_at(a, q0);
-      int fresh = kFresh | kNewTile, near = -1;
-      while (c.q < q1 && !stop) {
-        const Sys& S = sys_at(a, c.w.si);
-        if (c.w.near != near) fresh |= kFresh;
-        const uint32_t bytes = kExpBytes + (c.w.near ? 1 : 2) * kVarBytes;
-        for (int unit = c.w.j0; unit < c.w.j1; ++unit) {
-          const int flags = (c.w.near ? kNear : 0) | (unit == c.w.j0 ? kFirst : 0) | (unit + 1 == c.w.j1 ? kLast : 0);
-          if (!put(c.w.kc * kChunkK + unit * kUnitK, c.w.c0, kUnit << 8 | flags | fresh, c.w.si)) { stop = true; break; }
-          const int b = d % kBSlots;
-          mbar_arrive_expect_tx(&sm.bfull[b], bytes);
-          bulk_g2s(sm.small[b], S.small + ((size_t)(c.w.kc * kChunkUnits + unit) * c.w.parts + c.w.part) * kSmallBytes,
-                   bytes, &sm.bfull[b]);
-          ++d;
-          fresh = 0;
-          near = c.w.near;
-        }
-        if (stop) break;
-        const long long tile = S.tile_base + c.w.T;
-        if (cursor_next(a, c, q1)) {
-          if (!put(0, 0, kFlush << 8, (int)partial_slot(tile, blockIdx.x))) { stop = true; break; }
-          mbar_arrive(&sm.bfull[d++ % kBSlots]);
-          fresh = kFresh | kNewTile;
+      if (q0 < q1) {
+        long long q = q0;
+        int si = find_sys(a, q0, [](const Sys& y) { return y.unit_base; });
+        const Sys* S = &sys_at(a, si);
+        Walk w;
+        walk_to(w, *S, si, q0 - S->unit_base);
+        int fresh = kFresh | kNewTile, cls = -1;
+        bool scaled = false, joined = false;
+        while (q < q1 && !stop) {
+          if (w.cls != cls) fresh |= kFresh;
+          if (S->adj && !scaled && w.cls == kBand && w.j0 < w.j1) {
+            if (!message(kScale, 0, w.c0, si)) break;
+            scaled = true;
+          }
+          // a near sum takes one plane, so two chunks (an even one and the next)
+          // stay within 2^10 products and are accumulated together
+          const bool join = w.cls == kNear && !(w.kc & 1) && q + 1 < q1 && w.idx + 1 < w.nfar + S->cpt - w.first;
+          const uint32_t bytes = kExpBytes + (w.cls == kNear ? 1 : 2) * C::kVarBytes;
+          const uint8_t* src = S->small + (w.cls == kBand ? C::kHalfBytes : 0) +
+                               ((size_t)w.kc * kChunkUnits * S->parts + w.part) * C::kSmallBytes;
+          for (int unit = w.j0; unit < w.j1; ++unit) {
+            const int flags = (w.cls == kNear ? kFlagNear : 0) | (w.cls == kBand ? kFlagBand : 0) |
+                              (unit == w.j0 && !joined ? kFirst : 0) | (unit + 1 == w.j1 && !join ? kLast : 0);
+            if (!put(w.kc * kChunkK + unit * kUnitK, w.c0, kUnit << 8 | flags | fresh, si)) { stop = true; break; }
+            const int b = d % kBSlots;
+            mbar_arrive_expect_tx(&sm.bfull[b], bytes);
+            bulk_g2s(sm.small[b], src + (size_t)unit * S->parts * C::kSmallBytes, bytes, &sm.bfull[b]);
+            ++d;
+            fresh = 0;
+            cls = w.cls;
+          }
+          if (stop) break;
+          joined = join;
+          const int T = w.T, c0 = w.c0, slot = T + (int)blockIdx.x - S->cta0, sys = si;
+          const bool adj = S->adj;
+          int moved = 1;
+          if (++q < q1) {
+            moved = walk_next(w, *S);
+            if (moved == 2) {
+              S = &sys_at(a, ++si);
+              walk_to(w, *S, si, 0);
+            }
+          }
+          if (moved) {
+            if (adj && !scaled && !message(kScale, 0, c0, sys)) { stop = true; break; }
+            if (!message(kFlush, sys, 0, slot)) { stop = true; break; }
+            fresh = kFresh | kNewTile;
+            scaled = false;
+          }
         }
       }
-      if (!stop && put(0, 0, kEnd << 8, 0)) mbar_arrive(&sm.bfull[d++ % kBSlots]);
+      if (!stop) message(kEnd, 0, 0, 0);
       // the copies already issued must land before the CTA can exit (each slot's last phase)
       for (unsigned k = d > kBSlots ? d - kBSlots : 0; k < d; ++k) {
         long long spins = 0;
         while (!mbar_try(&sm.bfull[k % kBSlots], (k / kBSlots) & 1) && ++spins < kSpinLimit) __nanosleep(64);
-        if (spins >= kSpinLimit) atomicOr(a.status, kStatusTimeout);
+        if (spins >= kSpinLimit) atomicOr(status, kStatusTimeout);
       }
-    }
-    __syncwarp();
-  } else {
-    // -------------------------------------------------------------- MMA --
-    if (lane == 0) {
-      // A: [digit 8][K group 2][row group 16][8 rows][16 B]; B: [K group 2][digit 8][column group 2][8][16 B]
+    } else if (warp == kMmaWarp && lane == 0) {
+      // ------------------------------------------------------------ MMA --
+      // A: [digit 8][K group 2][row group 16][8 rows][16 B]; B: [K group 2][digit 8][column group][8][16 B]
       const uint64_t a0 = umma_desc(smem_u32(sm.stage[0]), kRows * 16, 128);
       const uint64_t b0 = umma_desc(smem_u32(sm.small[0] + kExpBytes), kDig * (kN / 8) * 128, 128);
       unsigned u = 0, p = 0;
       bool any = false, stop = false, open = false;
-      int nb = 0;     // buffers of the open group
-      int held = -1;  // slot of a flush descriptor not released yet (every tile has units: one at most)
+      int nb = 0;  // buffers of the open group
+      unsigned held = 0;  // slots (bits) of messages not released yet
       auto close = [&]() {
         for (int k = 0; k < nb; ++k) {
           mbar_arrive(&sm.accfull[(p + k) % kBufs]);
@@ -550,11 +677,14 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
         open = false;
       };
       // hands a message without sums to the epilogue
-      auto message = [&](int type, int slot) -> bool {
+      auto message = [&](int type, int si, int c0, int slot) -> bool {
         const int buf = p % kBufs;
-        if (!wait_bar(sm, &sm.accempty[buf], ((p / kBufs) & 1) ^ 1, a.status, a.spin)) return false;
-        sm.post[buf].type = type;
-        sm.post[buf].slot = slot;
+        if (!wait_bar(&sm.abort, &sm.accempty[buf], ((p / kBufs) & 1) ^ 1, status)) return false;
+        Post& ps = sm.post[buf];
+        ps.type = type;
+        ps.si = si;
+        ps.c0 = c0;
+        ps.slot = slot;
         mbar_arrive(&sm.accfull[buf]);
         mbar_arrive(&sm.accfull[buf]);
         ++p;
@@ -562,63 +692,78 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       };
       for (unsigned d = 0; !stop; ++d) {
         const int b = d % kBSlots;
-        if (!wait_bar(sm, &sm.bfull[b], (d / kBSlots) & 1, a.status, a.spin)) { stop = true; break; }
+        if (!wait_bar(&sm.abort, &sm.bfull[b], (d / kBSlots) & 1, status)) { stop = true; break; }
         const Desc ds = sm.desc[b];
         const int kind = ds.flags >> 8;
         if (kind == kEnd) break;
-        if (kind == kFlush) {
-          held = b;  // until the next unit is full: then every converter has read past this descriptor
-          if (!message(kPostFlush, ds.aux)) stop = true;
+        if (kind != kUnit) {
+          // released when the next unit is full: then every converter has read
+          // past this descriptor (at most a scaling and a flush come in a row,
+          // since every tile starts with a unit)
+          held |= 1u << b;
+          if (!message(kind, kind == kFlush ? ds.kap : ds.aux, ds.c0, ds.aux)) stop = true;
           continue;
         }
         const int s = u % kStages;
-        const bool near = ds.flags & kNear;
-        if (!wait_bar(sm, &sm.full[s], (u / kStages) & 1, a.status, a.spin)) { stop = true; break; }
-        if (held >= 0) {
-          mbar_arrive(&sm.bempty[held]);
-          held = -1;
-        }
+        const bool two = ds.flags & (kFlagNear | kFlagBand), band = ds.flags & kFlagBand;
+        if (!wait_bar(&sm.abort, &sm.full[s], (u / kStages) & 1, status)) { stop = true; break; }
+        for (int k = 0; k < kBSlots && held; ++k)
+          if (held >> k & 1u) {
+            mbar_arrive(&sm.bempty[k]);
+            held &= ~(1u << k);
+          }
         const bool begin = (ds.flags & kFirst) || *(volatile unsigned*)&sm.raise[s] == u + 1;
         if (begin) {
           if (open) close();
-          nb = near ? 2 : 1;
-          const int4 ex = *reinterpret_cast<const int4*>(sm.small[b]);
-          for (int g = 0; g < nb && !stop; ++g) {
-            const int buf = (p + g) % kBufs;
-            if (!wait_bar(sm, &sm.accempty[buf], (((p + g) / kBufs) & 1) ^ 1, a.status, a.spin)) { stop = true; break; }
-            Post& ps = sm.post[buf];
-            ps.type = kPostSum;
-            ps.grp = g;
-            ps.eidx = u % kExpRing;
-            *reinterpret_cast<int4*>(ps.es) = ex;
-          }
-          if (stop) break;
+          nb = two ? 2 : 1;
           open = true;
         }
+        // the buffer of sum g of a new accumulation
+        auto begin_sum = [&](int g) -> bool {
+          const int buf = (p + g) % kBufs;
+          if (!wait_bar(&sm.abort, &sm.accempty[buf], (((p + g) / kBufs) & 1) ^ 1, status)) return false;
+          Post& ps = sm.post[buf];
+          ps.type = kUnit;
+          ps.grp = g;
+          ps.eidx = u % kExpRing;
+          ps.plane = band ? 1 : g;
+#pragma unroll
+          for (int i = 0; i < NA / 8; ++i)
+            reinterpret_cast<int4*>(ps.es)[i] = reinterpret_cast<const int4*>(sm.small[b])[i];
+          return true;
+        };
+        if (begin && !begin_sum(0)) { stop = true; break; }
         tc_fence_after();
-        const uint64_t dPL = a0 + ((uint64_t)(s * 2 * kPlane) >> 4), dQ = dPL + (kPlane >> 4);
-        const uint64_t dA = b0 + ((uint64_t)(b * kSmallBytes) >> 4), dB = near ? dA : dA + (kVarBytes >> 4);
-        const uint32_t t0 = tmem + (p % kBufs) * kBufCols, t1 = near ? tmem + ((p + 1) % kBufs) * kBufCols : t0;
+        // far: PL x variant 0 and Q x variant 1 into one sum; near: PL and Q x
+        // variant 0 into two; band: Q x variant 0 and 1 into two
+        const uint64_t dP = a0 + ((uint64_t)(s * 2 * kPlane) >> 4), dQ = dP + (kPlane >> 4);
+        const uint64_t dA = b0 + ((uint64_t)(b * C::kHalfBytes) >> 4);
+        const uint64_t x0 = band ? dQ : dP, v1 = two && !band ? dA : dA + (C::kVarBytes >> 4);
+        const uint32_t t0 = tmem + (p % kBufs) * kBufCols, t1 = two ? tmem + ((p + 1) % kBufs) * kBufCols : t0;
 #pragma unroll
         for (int i = 0; i < kDig; ++i)
-          umma_f16(t0 + i * kN, dPL + ((i * kDigPlane) >> 4), dA, umma_idesc_f16(kN * (kDig - i)), !(begin && i == 0));
+          umma_f16(t0 + i * kN, x0 + ((i * kDigPlane) >> 4), dA, umma_idesc_f16(kN * (kDig - i)), !(begin && i == 0));
+        any = true;
+        if (begin && two) {
+          if (!begin_sum(1)) { stop = true; break; }
+          tc_fence_after();
+        }
 #pragma unroll
         for (int i = 0; i < kDig; ++i)
-          umma_f16(t1 + i * kN, dQ + ((i * kDigPlane) >> 4), dB, umma_idesc_f16(kN * (kDig - i)),
-                   !(begin && near && i == 0));
+          umma_f16(t1 + i * kN, dQ + ((i * kDigPlane) >> 4), v1, umma_idesc_f16(kN * (kDig - i)),
+                   !(begin && two && i == 0));
         umma_commit(&sm.empty[s]);
         umma_commit(&sm.bempty[b]);
-        any = true;
         ++u;
         if (ds.flags & kLast) close();
       }
-      if (!stop) message(kPostExit, 0);
+      if (!stop) message(kEnd, 0, 0, 0);
       // every MMA must complete before tensor memory is freed
       if (any) {
         umma_commit(&sm.mmadone);
         long long spins = 0;
         while (!mbar_try(&sm.mmadone, 0) && ++spins < kSpinLimit) __nanosleep(64);
-        if (spins >= kSpinLimit) atomicOr(a.status, kStatusTimeout);
+        if (spins >= kSpinLimit) atomicOr(status, kStatusTimeout);
       }
     }
     __syncwarp();
@@ -632,78 +777,101 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
 }
 
 // -------------------------------------------------------------- reduce ---
-// Output entry lin = (c, a, b): the partial sums of its tile in CTA order, then
-// the band of term 2 in FP64 with its exact weights.
-__global__ void __launch_bounds__(256) fx_reduce(Sys s, long long total, int G, const double* __restrict__ part,
-                                                 const double* __restrict__ Sl, const double* __restrict__ Sg,
-                                                 WeightsView w, double* __restrict__ out, int* status) {
-  const int M = s.M, MM = M * M, n = s.n;
-  const int64_t lin = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t row = (int64_t)(n + 1) * MM;
-  if (lin >= row) return;
-  const int c = (int)(lin / MM), ab = (int)(lin - (int64_t)c * MM), a = ab / M, b = ab - a * M;
-  const int ct = c / s.CT, T = ct * s.parts + a / kNA;
-  const int64_t at = (int64_t)(a % kNA) * kRows + (c - ct * s.CT) * M + b;
-  const long long lo = s.unit_base + (long long)T * s.upt, hi = lo + s.upt;
-  int i = (int)(lo * G / total);
-  while (i > 0 && range_lo(total, G, i) > lo) --i;
-  while (range_lo(total, G, i + 1) <= lo) ++i;
-  rk::Cd p{0, 0}, d{0, 0}, tl{0, 0}, tg{0, 0};
-  for (; i < G && range_lo(total, G, i) < hi; ++i) {
-    const double2* q = reinterpret_cast<const double2*>(part + (size_t)partial_slot(s.tile_base + T, i) * kSlotDoubles);
-    const double2 x = q[at], y = q[at + kNA * kRows];
-    p.re += x.x; p.im += x.y;
-    d.re += y.x; d.im += y.y;
-  }
-  for (int m = max(0, c - w.band_w + 1); m <= c; ++m) {
-    const double wcm = w.at(c, m);
-    const double* r = s.R + (tri(c, m) * MM + b * M) * 2;
-    const double* sl = Sl + ((int64_t)m * MM + a * M) * 2;
-    const double* sg = Sg + ((int64_t)m * MM + a * M) * 2;
-#pragma unroll 4
-    for (int x = 0; x < M; ++x) {
-      const rk::Cd rr = rk::ld(r + 2 * x);
-      rk::Cd vl = rk::ld(sl + 2 * x), vg = rk::ld(sg + 2 * x);
-      vl.re *= wcm; vl.im *= wcm; vg.re *= wcm; vg.im *= wcm;
-      rk::mac_cj(tl, vl, rr);
-      rk::mac_cj(tg, vg, rr);
+// Output entries (c, a, b): the partial sums of their tile in CTA order.
+template <int NA>
+__global__ void __launch_bounds__(256) fx_reduce(const __grid_constant__ Args a) {
+  const Head& h = head_of(a);
+  const long long entries = h.entries, total = h.total;
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < entries;
+       e += (long long)gridDim.x * blockDim.x) {
+    const Sys& s = sys_at(a, find_sys(a, e, [](const Sys& y) { return y.entry_base; }));
+    const long long lin = e - s.entry_base;
+    const int M = s.M, MM = M * M;
+    const int c = rk::div_idx(lin, MM), ab = (int)(lin - (long long)c * MM), row = ab / M, b = ab - row * M;
+    const int ct = c / s.CT, T = ct * s.parts + row / NA;
+    const int64_t at = (int64_t)(row % NA) * kRows + (c - ct * s.CT) * M + b;
+    const long long lo = s.unit_base + (long long)T * s.upt, hi = lo + s.upt;
+    double2 p = make_double2(0.0, 0.0), d = p;
+    for (int i = cta_of(total, a.G, lo); i < a.G && range_lo(total, a.G, i) < hi; ++i) {
+      if (range_lo(total, a.G, i + 1) <= range_lo(total, a.G, i)) continue;
+      const double2* q = reinterpret_cast<const double2*>(s.part) + (size_t)(T + i - s.cta0) * Cfg<NA>::kSlot;
+      const double2 x = q[at], y = q[at + NA * kRows];
+      p.x += x.x; p.y += x.y;
+      d.x += y.x; d.y += y.y;
     }
+    // slice: I^<, I^> = I^< + D; adjoint: S^>bar, S^<bar = C - S^>bar
+    const double2 q = s.adj ? make_double2(d.x - p.x, d.y - p.y) : make_double2(p.x + d.x, p.y + d.y);
+    reinterpret_cast<double2*>(s.adj ? s.out1 : s.out0)[lin] = p;
+    reinterpret_cast<double2*>(s.adj ? s.out0 : s.out1)[lin] = q;
+    if (!s.adj && !(isfinite(p.x) && isfinite(p.y) && isfinite(q.x) && isfinite(q.y))) atomicOr(s.status, kStatusNumeric);
   }
-  const double2 x = make_double2(p.re + tl.re, p.im + tl.im);
-  const double2 y = make_double2(p.re + d.re + tg.re, p.im + d.im + tg.im);
-  reinterpret_cast<double2*>(out)[lin] = x;
-  reinterpret_cast<double2*>(out)[row + lin] = y;
-  if (!(isfinite(x.x) && isfinite(x.y) && isfinite(y.x) && isfinite(y.y))) atomicOr(status, kStatusNumeric);
 }
 
-bool make_sys(int M, int n, int band_w, Sys* s) {
-  if (M < 1 || M > kMaxNorb || n < 0) return false;
-  s->M = M;
-  s->n = n;
-  s->CT = kRows / M;
-  s->cpt = (int)(((long long)(n + 1) * M + kChunkK - 1) / kChunkK);
-  s->parts = (M + kNA - 1) / kNA;
-  s->tiles = (n + s->CT) / s->CT * s->parts;
-  s->upt = s->cpt + kOver;
-  s->shift = -band_w;
-  s->magic = M == 1 ? 0u : (uint32_t)((0x100000000ull + (unsigned long long)M - 1) / (unsigned long long)M);
-  s->unit_base = s->tile_base = 0;
-  return true;
+int parts_of(int M) { return M <= 8 ? 8 : 16; }  // NA
+
+size_t small_bytes(const Sys& s, int NA) {
+  const size_t blk = NA == 8 ? Cfg<8>::kSmallBytes : Cfg<16>::kSmallBytes;
+  return ((size_t)s.cpt * kChunkUnits * s.parts * blk + 255) / 256 * 256;
+}
+size_t slot_bytes(int NA) { return 16 * (NA == 8 ? Cfg<8>::kSlot : Cfg<16>::kSlot); }
+
+// prep, contraction and reduction of the systems of `a`
+template <int NA>
+cudaError_t enqueue(const Args& a, bool quad, unsigned prep_blocks, unsigned red_blocks, cudaStream_t st, int* launches,
+                    cudaEvent_t ev_begin, cudaEvent_t ev_end) {
+  fx_prep<NA><<<prep_blocks, 32 * NA, 0, st>>>(a);
+  ++*launches;
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  if (ev_begin) cudaEventRecord(ev_begin, st);
+  if (quad)
+    fx_main<NA, true><<<a.G, kThreads, sizeof(Smem<NA>), st>>>(a);
+  else
+    fx_main<NA, false><<<a.G, kThreads, sizeof(Smem<NA>), st>>>(a);
+  if (ev_end) cudaEventRecord(ev_end, st);
+  ++*launches;
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  fx_reduce<NA><<<red_blocks, 256, 0, st>>>(a);
+  ++*launches;
+  return cudaGetLastError();
 }
 
-size_t small_bytes(const Sys& s) { return ((size_t)s.cpt * kChunkUnits * s.parts * kSmallBytes + 255) / 256 * 256; }
-
-int grid_ctas(long long total) { return (int)std::min<long long>(total, std::min(sm_count(), kMaxCtas)); }
+// One system's contraction in its workspace.
+cudaError_t launch_one(Sys s, int M, int n, int band_w, int adj, void* work, size_t work_bytes, cudaStream_t st,
+                       int* launches, cudaEvent_t ev_begin, cudaEvent_t ev_end) {
+  *launches = 0;
+  if (M < 1 || M > kMaxNorb || n < 0) return cudaErrorInvalidValue;
+  const int NA = parts_of(M);
+  set_geometry(s, M, n, band_w, adj, NA);
+  s.small = reinterpret_cast<uint8_t*>(work);
+  s.part = reinterpret_cast<double*>(s.small + small_bytes(s, NA));
+  Args a{};
+  a.one_head.n_sys = 1;
+  a.one_head.total = (long long)s.tiles * s.upt;
+  a.one_head.chunks = (long long)(s.cpt + 1) / 2 * s.parts;
+  a.one_head.entries = (long long)(n + 1) * M * M;
+  a.G = (int)std::min<long long>(a.one_head.total, sm_count());
+  if (small_bytes(s, NA) + ((size_t)s.tiles + a.G) * slot_bytes(NA) > work_bytes) return cudaErrorInvalidValue;
+  a.one = s;
+  cudaError_t e = fx_prepare();
+  if (e != cudaSuccess) return e;
+  const unsigned prep = (unsigned)std::min<long long>(a.one_head.chunks, 1 << 30);
+  const unsigned red = (unsigned)std::min<long long>((a.one_head.entries + 255) / 256, 1 << 30);
+  return NA == 8 ? enqueue<8>(a, M % 4 == 0, prep, red, st, launches, ev_begin, ev_end)
+                 : enqueue<16>(a, M % 4 == 0, prep, red, st, launches, ev_begin, ev_end);
+}
 
 }  // namespace
 
 size_t fx_workspace_bytes(int M, int n_max) {
-  Sys s;
-  if (!make_sys(M, n_max - 1, 1, &s)) return 0;
-  return small_bytes(s) + ((size_t)s.tiles + std::min(sm_count(), kMaxCtas)) * kSlotDoubles * sizeof(double);
+  if (M < 1 || M > kMaxNorb || n_max < 1) return 0;
+  Sys s{};
+  const int NA = parts_of(M);
+  set_geometry(s, M, n_max - 1, kMaxOrder + 1, 0, NA);
+  return small_bytes(s, NA) + ((size_t)s.tiles + sm_count()) * slot_bytes(NA);
 }
 
-// The kernel's dynamic shared memory exceeds the default limit (set once per device).
+// The main kernels' dynamic shared memory exceeds the default limit (set once per device).
 cudaError_t fx_prepare() {
   static std::atomic<unsigned long long> done_mask{0};
   int dev = 0;
@@ -711,50 +879,45 @@ cudaError_t fx_prepare() {
   if (e != cudaSuccess) return e;
   const unsigned long long bit = 1ull << (dev & 63);
   if (done_mask.load() & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(fx_main<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fx_main<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
+  const auto set = [](const void* f, size_t bytes) {
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  };
+  e = set((const void*)fx_main<8, true>, sizeof(Smem<8>));
+  if (e == cudaSuccess) e = set((const void*)fx_main<8, false>, sizeof(Smem<8>));
+  if (e == cudaSuccess) e = set((const void*)fx_main<16, true>, sizeof(Smem<16>));
+  if (e == cudaSuccess) e = set((const void*)fx_main<16, false>, sizeof(Smem<16>));
   if (e == cudaSuccess) done_mask.fetch_or(bit);
   return e;
 }
 
 cudaError_t launch_history_fx(const HistoryArgs& h, void* work, size_t work_bytes, cudaStream_t st, int* launches) {
-  *launches = 0;
-  Sys s;
-  if (!make_sys(h.M, h.n, h.w.band_w, &s)) return cudaErrorInvalidValue;
+  Sys s{};
   s.L = h.L;
   s.R = h.R;
-  uint8_t* small = reinterpret_cast<uint8_t*>(work);
-  double* part = reinterpret_cast<double*>(small + small_bytes(s));
-  s.small = small;
-  const long long total = (long long)s.tiles * s.upt;
-  const int G = grid_ctas(total);
-  if (small_bytes(s) + ((size_t)s.tiles + G) * kSlotDoubles * sizeof(double) > work_bytes) return cudaErrorInvalidValue;
-  cudaError_t e = fx_prepare();
-  if (e != cudaSuccess) return e;
-  fx_prep<<<dim3(s.cpt, s.parts), 32 * kNA, 0, st>>>(s, h.Sl, h.Sg, h.w, small);
-  ++*launches;
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  Args a{};
-  a.one = s;
-  a.n_sys = 1;
-  a.G = G;
-  a.total = total;
-  a.part = part;
-  a.status = h.status;
-  a.spin = kWaitCycles;
-  if (h.ev_begin) cudaEventRecord(h.ev_begin, st);
-  if (s.M % 4 == 0)
-    fx_main<true><<<G, kThreads, sizeof(Smem), st>>>(a);
-  else
-    fx_main<false><<<G, kThreads, sizeof(Smem), st>>>(a);
-  if (h.ev_end) cudaEventRecord(h.ev_end, st);
-  ++*launches;
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const int64_t row = (int64_t)(s.n + 1) * s.M * s.M;
-  fx_reduce<<<(unsigned)((row + 255) / 256), 256, 0, st>>>(s, total, G, part, h.Sl, h.Sg, h.w, h.out, h.status);
-  ++*launches;
-  return cudaGetLastError();
+  s.Sl = h.Sl;
+  s.Sg = h.Sg;
+  s.wbar = h.w.wbar;
+  s.band = h.w.band;
+  s.out0 = h.out;
+  s.out1 = h.out + 2 * (size_t)(h.n + 1) * h.M * h.M;
+  s.status = h.status;
+  return launch_one(s, h.M, h.n, h.w.band_w, 0, work, work_bytes, st, launches, h.ev_begin, h.ev_end);
+}
+
+// The Sigma-row cotangents of the slice's adjoint (the sums of adj_hist_small and its reduction).
+cudaError_t launch_adjoint_fx(const AdjHistArgs& h, void* work, size_t work_bytes, int* status, cudaStream_t st,
+                              int* launches) {
+  Sys s{};
+  s.L = h.L;
+  s.R = h.R;
+  s.Sl = h.Ib;
+  s.Sg = h.Ib + 2 * (size_t)(h.n + 1) * h.M * h.M;
+  s.wbar = h.w.wbar;
+  s.band = h.w.band;
+  s.out0 = h.dSl;
+  s.out1 = h.dSg;
+  s.status = status;
+  return launch_one(s, h.M, h.n, h.w.band_w, 1, work, work_bytes, st, launches, nullptr, nullptr);
 }
 
 }  // namespace kbe

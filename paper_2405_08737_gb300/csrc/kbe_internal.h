@@ -213,12 +213,6 @@ cudaError_t launch_history_finish(int nchunk, int64_t row, const double* partial
 cudaError_t launch_history_f64_ranges(const HistoryArgs& a, int nranges, const int* c_lo, const int* c_hi,
                                       const cudaEvent_t* wait, cudaStream_t s, int* launches);
 
-// FP64 history slice on the tensor cores (history_fx.cu): the sums of
-// launch_history_f64 over all stored rows, in the workspace `work`.
-size_t fx_workspace_bytes(int M, int n_max);
-cudaError_t fx_prepare();  // one-time kernel attributes of the current device
-cudaError_t launch_history_fx(const HistoryArgs& a, void* work, size_t work_bytes, cudaStream_t s, int* launches);
-
 // Split-precision history slice (history_split.cu).
 struct SplitGeomHost {
   int M, n, CT, parts, cpt, tiles;
@@ -430,6 +424,9 @@ struct AdjHistArgs {
   double* work;
   size_t work_bytes;
   int df = 0;           // 1: the Sigma-row cotangent sums in double-float (KBE_DF64 steps)
+  void* fx_work = nullptr;  // workspace of history_fx.cu: those sums on the tensor cores
+  size_t fx_bytes = 0;
+  int* status = nullptr;
 };
 cudaError_t launch_adjoint_history(const AdjHistArgs& a, cudaStream_t s, int* launches);
 

@@ -1,5 +1,6 @@
-"""FP64 history slices on the tensor cores (csrc/history_fx.cu): sizes around its
-tiles against the oracle, at the FP64 path's tolerance.
+"""FP64 history slices on the tensor cores (csrc/history_fx.cu) and the sums of
+their adjoint: sizes around its tiles against the oracle, at the FP64 path's
+tolerance.
 
 The error of a slice of n + 1 points is below 2^-56 of the largest products per
 32 history entries plus FP64 rounding of the sums, well under 1e-12 of the
@@ -83,6 +84,29 @@ def test_high_orders_and_zero_history(kbe):
     ctx.history_slice(n, _dev(0 * L), _dev(0 * R), _dev(Sl), _dev(Sg), out)
     ctx.sync_status()
     assert not out.abs().any()
+    ctx.close()
+
+
+@pytest.mark.parametrize("M,n", [(5, 269), (8, 128), (13, 70), (16, 47), (24, 26), (33, 16)])
+def test_adjoint_is_the_transpose(kbe, M, n):
+    """Re<Ibar, I(dS)> = Re<Sbar, dS> for random rows Ibar, dS, which are
+    independent of each other (1e-12 of the products' sizes; I is linear in the
+    self-energy row and checked against the oracle above)."""
+    import torch
+    ctx, t, order, L, R, Sl, Sg = _setup(kbe, M, n, 7 * M + n, "random")
+    rng = np.random.default_rng(M)
+    Ib = _dev(rng.standard_normal((2, n + 1, M, M)) + 1j * rng.standard_normal((2, n + 1, M, M)))
+    Ld, Rd, Sld, Sgd = _dev(L), _dev(R), _dev(Sl), _dev(Sg)
+    out = torch.zeros_like(Ib)
+    ctx.history_slice(n, Ld, Rd, Sld, Sgd, out)
+    dSl, dSg = torch.zeros_like(Sld), torch.zeros_like(Sgd)
+    dL = torch.zeros((n + 1, M, M), dtype=torch.complex128, device="cuda")
+    ctx.adjoint_slice(n, Ld, Rd, Sld, Sgd, Ib, dSl, dSg, dL, torch.zeros_like(dL), n)
+    ctx.sync_status()
+    lhs = (Ib.conj() * out).sum().real
+    rhs = (dSl.conj() * Sld).sum().real + (dSg.conj() * Sgd).sum().real
+    size = (dSl.conj() * Sld).abs().sum() + (dSg.conj() * Sgd).abs().sum()
+    assert abs(lhs - rhs) < TOL * size
     ctx.close()
 
 

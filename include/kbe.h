@@ -87,7 +87,9 @@ typedef int kbe_status;
                           /* the FP32 pipe (hi + lo floats, about 2^-47 per   */
                           /* product, compensated sums): about 1e-14 of the   */
                           /* terms' sizes, several times the FP64 pipe's      */
-                          /* rate on this part.  Deterministic.               */
+                          /* rate on this part.  Slices of (n+1)^2 norb^3 >=  */
+                          /* 8e6 are formed as for KBE_FP64, which is faster  */
+                          /* there.  Deterministic.                           */
 
 /* ---------------------------------------------------------- lifecycle -- */
 
@@ -276,7 +278,10 @@ kbe_status kbe_rhs_row(kbe_ctx* ctx, int j, int precision, const void* L, const 
  * With KBE_SPLIT_BF16 the context keeps the tensor-core digit planes of the
  * history between steps on the same L and R: rows below the row of the
  * previous step are not encoded again.  A caller that rewrites those rows
- * between steps (a restart into the same buffers) calls kbe_reset_cache. */
+ * between steps (a restart into the same buffers) calls kbe_reset_cache.
+ * Rows that kbe_run_steps takes in its cooperative launch take it here too,
+ * one launch per step (not during a stream capture: there, and where the
+ * device refuses it, one launch per kernel). */
 kbe_status kbe_step(kbe_ctx* ctx, int n, int P, int precision, void* L, void* R, void* S_less,
                     void* S_great, void* I_work, void* F_ring, void* stream);
 
@@ -548,7 +553,9 @@ kbe_status kbe_read_profiling(kbe_ctx* ctx, int* count, double* total_ms);
  * model) advanced together: one batched KBE step runs kbe_step's sequence
  * for every active system as ONE CUDA graph launch (batched elementwise
  * kernels, and for KBE_FP64 one persistent history kernel over a work list
- * of (system, tile, history chunk) items).  The paper steps one system;
+ * of (system, tile, history chunk) items for the smaller slices and one
+ * persistent tensor-core kernel each for the larger ones of systems with up
+ * to 8 and with more orbitals).  The paper steps one system;
  * this is a throughput form for ensembles of systems. */
 typedef struct kbe_batch kbe_batch;
 

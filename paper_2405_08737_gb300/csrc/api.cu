@@ -112,17 +112,7 @@ bool next_events(kbe_ctx* ctx, cudaEvent_t* b, cudaEvent_t* e) {
 // of the same arrays are reused (the split path re-encodes only units that
 // involve rows >= the cached row count).
 struct Staged;
-// Whether the FP64 slice of row n goes to the tensor cores (history_fx.cu): from
-// (n + 1)^2 M^3 = 5e6 on, and never for the rows that kbe_run_steps takes in its
-// cooperative kernel.  Below that the FP64 pipe is as fast or faster, above it
-// falls behind with the cube of M (slices on the FP64 pipe against the tensor
-// cores, us: M = 5, n = 163 95 / 87; M = 8, n = 64 89 / 66, n = 1023 7080 / 905; M = 12,
-// n = 29 63 / 91, n = 50 107 / 130; M = 16, n = 16 55 / 84, n = 30 102 / 89; M = 24,
-// n = 10 68 / 100, n = 20 159 / 138; M = 32, n = 16 249 / 140).
-bool use_fx(const kbe_ctx* ctx, int n) {
-  const double N = n + 1.0, M = ctx->M;
-  return ctx->d_fx && N * M * M > kRunMaxRow && N * N * M * M * M >= 5e6;
-}
+bool use_fx(const kbe_ctx* ctx, int n) { return ctx->d_fx && fx_takes(ctx->M, n); }
 cudaError_t slice_f64(const kbe_ctx* ctx, const HistoryArgs& a, cudaStream_t s, int* launches) {
   if (use_fx(ctx, a.n) && a.band_lo <= 0 && a.band_hi > a.n)
     return launch_history_fx(a, ctx->d_fx, ctx->fx_bytes, s, launches);
@@ -189,7 +179,8 @@ kbe_status history(kbe_ctx* ctx, int n, int precision, const void* L, const void
   cudaError_t e;
   if (precision == KBE_DF64) {
     if (!next_events(ctx, &a.ev_begin, &a.ev_end)) return fail(ctx, KBE_ECUDA, "profiling: cudaEventCreate");
-    e = launch_history_df(a, s, launches);
+    e = ctx->d_fx && fx_takes_df(ctx->M, n) ? launch_history_fx(a, ctx->d_fx, ctx->fx_bytes, s, launches)
+                                            : launch_history_df(a, s, launches);
     return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "history slice launch");
   }
   if (staged && !use_fx(ctx, n)) {  // the column ranges contract as their rows arrive (no timing events: they would hold the waits)
@@ -411,6 +402,65 @@ kbe_status step_impl(kbe_ctx* ctx, int n, int P, int precision, void* L, void* R
   }
   if ((e = keep(P)) != cudaSuccess) return cuda_fail(ctx, e, "kbe_step: iterate copy");
   return KBE_OK;
+}
+
+// Whether a call's steps may run in the cooperative kernel (run_small.cu): plain
+// FP64 steps with the local interaction and fixed orders.
+bool coop_steps(const kbe_ctx* ctx, int precision) {
+  return precision == KBE_FP64 && !ctx->dense && ctx->adaptive_K == 0 && !ctx->thermal && !ctx->profiling &&
+         !ctx->run_coop_refused;
+}
+bool small_row(const kbe_ctx* ctx, int n) { return (int64_t)(n + 1) * ctx->M * ctx->M <= kRunMaxRow; }
+
+// The steps of rows *n, *n + 1, ... up to n_last in one cooperative launch, as
+// long as the rows are small and at most kRunMaxSteps; *n becomes the next row.
+// Where the device refuses the launch, the same rows take the per-kernel step.
+kbe_status steps_small(kbe_ctx* ctx, int* n, int n_last, int P, void* L, void* R, void* Sl, void* Sg, void* I_work,
+                       void* F_ring, cudaStream_t s, bool run, int* launches) {
+  RunSmallHost h{};
+  h.base = step_args(ctx, *n, L, R, I_work, F_ring);
+  h.Sl = (double*)Sl;
+  h.Sg = (double*)Sg;
+  h.I = (double*)I_work;
+  h.w = weights_view(ctx);
+  h.part = ctx->d_part;
+  h.corr0 = ctx->d_corr;
+  h.pred0 = ctx->d_pred;
+  h.bar = ctx->d_runbar;
+  h.spin = 1ll << 24;  // polls: about a second or more
+  if (run) {           // the failure-path test of kbe_run_steps: one launch only
+    if (ctx->dbg_run_spin > 0) h.spin = ctx->dbg_run_spin;
+    h.withhold = ctx->dbg_run_withhold;
+    ctx->dbg_run_spin = 0;
+    ctx->dbg_run_withhold = -1;
+  }
+  h.P = P;
+  while (h.nsteps < kRunMaxSteps && *n <= n_last && small_row(ctx, *n)) {
+    const int i = h.nsteps;
+    if (!history_f64_split(ctx->M, *n, ctx->part_bytes, 0x7fffffff, &h.nchunk[i], &h.chunk_len[i]))
+      return fail(ctx, KBE_ENOMEM, "kbe_run_steps: history workspace too small");
+    h.n[i] = *n;
+    h.kn[i] = ctx->grid.order[*n];
+    h.field[i] = ctx->model.field(ctx->grid.t[*n]);
+    ++h.nsteps;
+    ++*n;
+  }
+  kbe_status st = KBE_OK;
+  const cudaError_t e = launch_run_small(h, s, launches);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    // fewer SMs available than the device has (e.g. a partitioned GPU): these rows and all later ones
+    // take the per-kernel step (the launch error is not sticky)
+    cudaGetLastError();
+    ctx->run_coop_refused = true;
+    for (int i = 0; i < h.nsteps && st == KBE_OK; ++i) {
+      int c = 0;
+      st = step_impl(ctx, h.n[i], P, KBE_FP64, L, R, Sl, Sg, I_work, F_ring, 0, kRing, s, nullptr, &c);
+      *launches += c;
+    }
+  } else if (e != cudaSuccess) {
+    st = cuda_fail(ctx, e, "kbe_run_steps: cooperative run launch");
+  }
+  return st;
 }
 
 kbe_status check_step_call(kbe_ctx* ctx, int n, int P, int precision, const void* L, const void* R, const void* Sl,
@@ -1116,7 +1166,16 @@ kbe_status kbe_step(kbe_ctx* ctx, int n, int P, int precision, void* L, void* R,
   kbe_status st = check_step_call(ctx, n, P, precision, L, R, Sl, Sg, I_work, F_ring);
   if (st != KBE_OK) return st;
   int count = 0;
-  st = step_impl(ctx, n, P, precision, L, R, Sl, Sg, I_work, F_ring, 0, kRing, (cudaStream_t)stream, nullptr, &count);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing((cudaStream_t)stream, &capture) != cudaSuccess) cudaGetLastError();
+  if (coop_steps(ctx, precision) && small_row(ctx, n) && capture == cudaStreamCaptureStatusNone) {
+    // one launch instead of a dozen (steps on the stored history, us: M = 2, n = 30 89 -> 46; M = 4, n = 63
+    // 105 -> 61; M = 8, n = 63 197 -> 185)
+    int next = n;
+    st = steps_small(ctx, &next, n, P, L, R, Sl, Sg, I_work, F_ring, (cudaStream_t)stream, false, &count);
+  } else {
+    st = step_impl(ctx, n, P, precision, L, R, Sl, Sg, I_work, F_ring, 0, kRing, (cudaStream_t)stream, nullptr, &count);
+  }
   ctx->last_launches = count;
   return st;
 }
@@ -1139,54 +1198,13 @@ kbe_status kbe_run_steps(kbe_ctx* ctx, int n_first, int n_last, int P, int preci
   int total = 0;
   // Plain FP64 steps with the local interaction and fixed orders: runs of
   // small rows go to the cooperative kernel, up to kRunMaxSteps rows per launch.
-  const bool coop = precision == KBE_FP64 && !ctx->dense && ctx->adaptive_K == 0 && !ctx->thermal &&
-                    !ctx->profiling && !ctx->run_coop_refused;
-  const int64_t MM = (int64_t)ctx->M * ctx->M;
+  const bool coop = coop_steps(ctx, precision);
   int n = n_first;
   while (n <= n_last && st == KBE_OK) {
-    if (coop && (int64_t)(n + 1) * MM <= kRunMaxRow) {
-      RunSmallHost h{};
-      h.base = step_args(ctx, n, L, R, I_work, F_ring);
-      h.Sl = (double*)Sl;
-      h.Sg = (double*)Sg;
-      h.I = (double*)I_work;
-      h.w = weights_view(ctx);
-      h.part = ctx->d_part;
-      h.corr0 = ctx->d_corr;
-      h.pred0 = ctx->d_pred;
-      h.bar = ctx->d_runbar;
-      h.spin = ctx->dbg_run_spin > 0 ? ctx->dbg_run_spin : 1ll << 24;  // polls: about a second or more
-      h.withhold = ctx->dbg_run_withhold;
-      ctx->dbg_run_spin = 0;  // one launch only
-      ctx->dbg_run_withhold = -1;
-      h.P = P;
-      while (h.nsteps < kRunMaxSteps && n <= n_last && (int64_t)(n + 1) * MM <= kRunMaxRow) {
-        const int i = h.nsteps;
-        if (!history_f64_split(ctx->M, n, ctx->part_bytes, 0x7fffffff, &h.nchunk[i], &h.chunk_len[i]))
-          return fail(ctx, KBE_ENOMEM, "kbe_run_steps: history workspace too small");
-        h.n[i] = n;
-        h.kn[i] = ctx->grid.order[n];
-        h.field[i] = ctx->model.field(ctx->grid.t[n]);
-        ++h.nsteps;
-        ++n;
-      }
+    if (coop && small_row(ctx, n) && !ctx->run_coop_refused) {
       int count = 0;
-      const cudaError_t e = launch_run_small(h, (cudaStream_t)stream, &count);
+      st = steps_small(ctx, &n, n_last, P, L, R, Sl, Sg, I_work, F_ring, (cudaStream_t)stream, true, &count);
       total += count;
-      if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
-        // fewer SMs available than the device has (e.g. a partitioned GPU): these rows and all later ones
-        // take the per-kernel step (the launch error is not sticky)
-        cudaGetLastError();
-        ctx->run_coop_refused = true;
-        for (int i = 0; i < h.nsteps && st == KBE_OK; ++i) {
-          int c = 0;
-          st = step_impl(ctx, h.n[i], P, precision, L, R, Sl, Sg, I_work, F_ring, 0, kRing, (cudaStream_t)stream,
-                         nullptr, &c);
-          total += c;
-        }
-      } else if (e != cudaSuccess) {
-        st = cuda_fail(ctx, e, "kbe_run_steps: cooperative run launch");
-      }
       continue;
     }
     int count = 0;

@@ -20,6 +20,13 @@
 // through an atomic counter.  (block, item_work_log2) is the tile policy; the
 // autotuner times candidate policies on the batch itself.
 //
+// Systems whose slice is large enough (fx_takes) run it on the tensor cores
+// instead: batch_fx_plan lists them on the device, and one launch of
+// history_fx.cu's kernels per class (M <= 8, M > 8) contracts all of them, each CTA
+// with an equal share of the chunks.  Ten systems of M = 4..24 and 299..667 points:
+// 221 ms per step on the FP64 pipe, 28.5 ms so.  The graph is captured again only
+// when the set of kernels in use changes.
+//
 // Elementwise kernels run grid-stride over the concatenation of all active
 // systems' rows; a thread finds its system by binary search over the
 // offsets the plan kernel wrote.
@@ -31,6 +38,7 @@
 #include <string>
 #include <vector>
 
+#include "history_fx.h"
 #include "row_kernels.cuh"
 
 namespace kbe {
@@ -56,9 +64,11 @@ struct BatchSys {
   double* eps;
   double* part;
   int64_t part_doubles;
+  void* fx_work;        // the context's workspace of history_fx.cu, or null
   // written by the plan kernel
   int n;                // row of this step, -1 when inactive
   int nchunk, chunk_len, xblk;
+  int fx;               // the FP64 slice of this step runs on the tensor cores
 };
 
 struct BatchDev {
@@ -72,6 +82,10 @@ struct BatchDev {
   int64_t* item_off;    // [n_sys + 1] (rank order)
   unsigned long long* counter;
   int* status;
+  // FP64 slices on the tensor cores: systems of up to 8 and of more orbitals
+  int use_fx, ctas;
+  fx::Sys* fx_table[2];
+  fx::Head* fx_head;    // [2]
 };
 
 __device__ __forceinline__ int find_rank(const int64_t* off, int n, int64_t x) {
@@ -122,6 +136,7 @@ __global__ void batch_plan(BatchDev b) {
     if (n < 1 || n >= s.n_t) {
       s.n = -1;
       s.nchunk = s.chunk_len = s.xblk = 0;
+      s.fx = 0;
       cost[i] = -1.0;
       elems[i] = items[i] = 0;
       continue;
@@ -143,7 +158,8 @@ __global__ void batch_plan(BatchDev b) {
     s.chunk_len = len;
     s.xblk = (int)((outputs + b.block - 1) / b.block);
     elems[i] = outputs;
-    items[i] = (int64_t)s.xblk * nchunk;
+    s.fx = b.use_fx && s.fx_work && fx_takes(s.M, n);
+    items[i] = s.fx ? 0 : (int64_t)s.xblk * nchunk;
     cost[i] = (double)len * (double)s.M;  // work of one item, up to the common factors
   }
   __syncthreads();
@@ -166,6 +182,57 @@ __global__ void batch_plan(BatchDev b) {
     }
     b.elem_off[b.n_sys] = e;
     b.item_off[b.n_sys] = it;
+  }
+}
+
+// The work lists of the tensor-core slices (one block, after batch_plan).
+__global__ void batch_fx_plan(BatchDev b) {
+  extern __shared__ int pos[];  // [n_sys]: the system's place in its list
+  for (int i = threadIdx.x; i < b.n_sys; i += blockDim.x) pos[i] = b.sys[i].fx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int count[2] = {0, 0};
+    for (int i = 0; i < b.n_sys; ++i) pos[i] = pos[i] ? count[b.sys[i].M > 8]++ : -1;
+    b.fx_head[0].n_sys = count[0];
+    b.fx_head[1].n_sys = count[1];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < b.n_sys; i += blockDim.x) {
+    if (pos[i] < 0) continue;
+    const BatchSys& s = b.sys[i];
+    const int NA = fx::part_rows(s.M);
+    fx::Sys y{};
+    fx::set_geometry(y, s.M, s.n, s.band_w, 0, NA);
+    y.L = s.L;
+    y.R = s.R;
+    y.Sl = s.Sl;
+    y.Sg = s.Sg;
+    y.wbar = s.wbar;
+    y.band = s.band;
+    y.out0 = s.I;
+    y.out1 = s.I + 2 * (int64_t)(s.n + 1) * s.M * s.M;
+    y.small = reinterpret_cast<uint8_t*>(s.fx_work);
+    y.part = reinterpret_cast<double*>(y.small + fx::small_bytes(y, NA));
+    y.status = b.status;
+    b.fx_table[s.M > 8][pos[i]] = y;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    fx::Head& h = b.fx_head[threadIdx.x];
+    fx::Sys* t = b.fx_table[threadIdx.x];
+    long long units = 0, chunks = 0, entries = 0;
+    for (int i = 0; i < h.n_sys; ++i) {
+      t[i].unit_base = units;
+      t[i].chunk_base = chunks;
+      t[i].entry_base = entries;
+      units += (long long)t[i].tiles * t[i].upt;
+      chunks += fx::prep_items(t[i]);
+      entries += (long long)(t[i].n + 1) * t[i].M * t[i].M;
+    }
+    h.total = units;
+    h.chunks = chunks;
+    h.entries = entries;
+    for (int i = 0; i < h.n_sys; ++i) t[i].cta0 = fx::cta_of(units, b.ctas, t[i].unit_base);
   }
 }
 
@@ -197,10 +264,12 @@ __global__ void __launch_bounds__(256) batch_rows(BatchDev b) {
                             reinterpret_cast<const double2*>(s.L) + off, reinterpret_cast<const double2*>(s.R) + off,
                             reinterpret_cast<double2*>(s.Sl), reinterpret_cast<double2*>(s.Sg));
     } else if (OP == kOpPrep) {
+      if (s.fx) continue;
       const int64_t row = (int64_t)(n + 1) * MM;
       const WeightsView w{s.wbar, s.band, s.band_w};
       rk::history_prep_entry(MM, n, lin, s.Sl, s.Sg, w, s.part, s.part + 2 * row);
     } else {  // kOpReduce: both s of entry lin
+      if (s.fx) continue;
       const int64_t row = (int64_t)(n + 1) * MM;
       double2* out = reinterpret_cast<double2*>(s.I);
       if (s.nchunk > 1) {
@@ -273,7 +342,8 @@ struct kbe_batch {
   int hist_blocks[2] = {0, 0};   // persistent grid for block = 128, 256
   // graph of one step for (P, precision, policy); split graphs also key on rows
   cudaGraphExec_t graph = nullptr;
-  int g_P = 0, g_prec = -1, g_block = 0, g_work = 0;
+  int g_P = 0, g_prec = -1, g_block = 0, g_work = 0, g_fx = 0;
+  bool quad[2] = {true, true};   // every M of the tensor-core lists a multiple of 4
   std::vector<int> g_rows;
   int g_count = 0;               // kernels in the step graph
   int last_launches = 0;
@@ -307,6 +377,18 @@ void drop_graph(kbe_batch* b) {
 }
 
 
+// Where the FP64 slices of a step run: bit 0 some on the FP64 pipe, bits 1 and 2
+// some on the tensor cores with up to 8 / more orbitals (as batch_plan decides).
+int slice_paths(const kbe_batch* b, const int* rows) {
+  int mask = 0;
+  for (int i = 0; i < b->n_sys; ++i) {
+    if (rows[i] < 1) continue;
+    const BatchSys& y = b->sys[i];
+    mask |= b->dev.use_fx && y.fx_work && fx_takes(y.M, rows[i]) ? (y.M > 8 ? 4 : 2) : 1;
+  }
+  return mask;
+}
+
 // Enqueue one batched step (rows already on the device).  Split precision
 // runs the fused contraction over the work list built from the host rows
 // (its image already uploaded).
@@ -315,20 +397,33 @@ cudaError_t enqueue_step(kbe_batch* b, int P, int precision, const int* rows_hos
   int nl = 0;
   batch_plan<<<1, 256, (size_t)b->n_sys * 24, s>>>(d);
   ++nl;
+  const int paths = precision == KBE_FP64 ? slice_paths(b, rows_host) : 0;
+  if (paths & 6) {
+    batch_fx_plan<<<1, 256, (size_t)b->n_sys * sizeof(int), s>>>(d);
+    ++nl;
+  }
   batch_rows<kOpPredictor><<<sm_count() * 8, 256, 0, s>>>(d);
   ++nl;
   cudaError_t e = cudaGetLastError();
   for (int it = 0; it < P && e == cudaSuccess; ++it) {
     batch_rows<kOpSigma><<<sm_count() * 8, 256, 0, s>>>(d);
     ++nl;
-    if (precision == KBE_FP64) {  // prep also clears the work counter
-      batch_rows<kOpPrep><<<sm_count() * 8, 256, 0, s>>>(d);
-      if (d.block == 128)
-        batch_history<128><<<b->hist_blocks[0], 128, 0, s>>>(d);
-      else
-        batch_history<256><<<b->hist_blocks[1], 256, 0, s>>>(d);
-      batch_rows<kOpReduce><<<sm_count() * 8, 256, 0, s>>>(d);
-      nl += 3;
+    if (precision == KBE_FP64) {
+      if (paths & 1) {  // prep also clears the work counter
+        batch_rows<kOpPrep><<<sm_count() * 8, 256, 0, s>>>(d);
+        if (d.block == 128)
+          batch_history<128><<<b->hist_blocks[0], 128, 0, s>>>(d);
+        else
+          batch_history<256><<<b->hist_blocks[1], 256, 0, s>>>(d);
+        batch_rows<kOpReduce><<<sm_count() * 8, 256, 0, s>>>(d);
+        nl += 3;
+      }
+      for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+        if (!(paths >> (k + 1) & 1)) continue;
+        int c = 0;
+        e = launch_fx_table(k ? 16 : 8, b->quad[k], d.fx_table[k], d.fx_head + k, s, &c);
+        nl += c;
+      }
     } else if (precision == KBE_DF64) {  // each system's double-float slice in its context's workspace
       for (int i = 0; i < b->n_sys && e == cudaSuccess; ++i) {
         const int n = rows_host[i];
@@ -338,7 +433,8 @@ cudaError_t enqueue_step(kbe_batch* b, int P, int precision, const int* rows_hos
         HistoryArgs a{y.M, n, y.L, y.R, y.Sl, y.Sg, WeightsView{y.wbar, y.band, y.band_w}, y.I, c->d_part,
                       c->part_bytes, d.status};
         int k = 0;
-        e = launch_history_df(a, s, &k);
+        e = c->d_fx && fx_takes_df(y.M, n) ? launch_history_fx(a, c->d_fx, c->fx_bytes, s, &k)
+                                           : launch_history_df(a, s, &k);
         nl += k;
       }
     } else if (b->fplan.n_ent > 0) {  // one persistent tensor-core contraction over every active system's units
@@ -404,7 +500,8 @@ kbe_status kbe_batch_create(kbe_ctx* const* ctxs, int n_sys, kbe_batch** out) {
   const size_t o_sys = take(sizeof(BatchSys) * n_sys), o_rows = take(sizeof(int) * n_sys),
                o_rank = take(sizeof(int) * n_sys), o_eoff = take(sizeof(int64_t) * (n_sys + 1)),
                o_ioff = take(sizeof(int64_t) * (n_sys + 1)), o_cnt = take(sizeof(unsigned long long)),
-               o_st = take(sizeof(int));
+               o_st = take(sizeof(int)), o_fx8 = take(sizeof(fx::Sys) * n_sys), o_fx16 = take(sizeof(fx::Sys) * n_sys),
+               o_head = take(2 * sizeof(fx::Head));
   size_t n_order = 0;
   for (int i = 0; i < n_sys; ++i) n_order += ctxs[i]->grid.n_t;
   if (e == cudaSuccess) e = cudaMalloc(&b->d_mem, off);
@@ -429,6 +526,11 @@ kbe_status kbe_batch_create(kbe_ctx* const* ctxs, int n_sys, kbe_batch** out) {
   b->dev.item_off = reinterpret_cast<int64_t*>(base + o_ioff);
   b->dev.counter = reinterpret_cast<unsigned long long*>(base + o_cnt);
   b->dev.status = reinterpret_cast<int*>(base + o_st);
+  b->dev.use_fx = 1;
+  b->dev.ctas = sm_count();
+  b->dev.fx_table[0] = reinterpret_cast<fx::Sys*>(base + o_fx8);
+  b->dev.fx_table[1] = reinterpret_cast<fx::Sys*>(base + o_fx16);
+  b->dev.fx_head = reinterpret_cast<fx::Head*>(base + o_head);
   // per-system tables
   std::vector<int> order(n_order);
   std::vector<double> field(n_order);
@@ -452,6 +554,8 @@ kbe_status kbe_batch_create(kbe_ctx* const* ctxs, int n_sys, kbe_batch** out) {
     y.eps = c->d_eps;
     y.part = c->d_part;
     y.part_doubles = (int64_t)(c->part_bytes / sizeof(double));
+    y.fx_work = c->d_fx;
+    if (c->M % 4) b->quad[c->M > 8] = false;
     y.order = b->d_order + at;
     y.field = b->d_field + at;
     y.n = -1;
@@ -607,7 +711,7 @@ kbe_status kbe_batch_step(kbe_batch* b, const int* rows, int P, int precision, v
     b->fplan_rows.assign(rows, rows + b->n_sys);
   }
   if (!b->graph || b->g_P != P || b->g_prec != precision || b->g_block != b->dev.block ||
-      b->g_work != b->dev.item_work_log2 || !same_rows) {
+      b->g_work != b->dev.item_work_log2 || !same_rows || (precision == KBE_FP64 && b->g_fx != slice_paths(b, rows))) {
     drop_graph(b);
     cudaStream_t cs;
     if ((e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking)) != cudaSuccess) return bcuda(b, e, "kbe_batch_step: capture stream");
@@ -631,6 +735,7 @@ kbe_status kbe_batch_step(kbe_batch* b, const int* rows, int P, int precision, v
     b->g_prec = precision;
     b->g_block = b->dev.block;
     b->g_work = b->dev.item_work_log2;
+    b->g_fx = slice_paths(b, rows);
     b->g_rows.assign(rows, rows + b->n_sys);
     b->g_count = count;
   }
@@ -653,7 +758,9 @@ kbe_status kbe_batch_autotune(kbe_batch* b, const int* rows, int reps, void* str
   if ((e = cudaMemcpyAsync((void*)b->dev.rows, rows, sizeof(int) * b->n_sys, cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return bcuda(b, e, "kbe_batch_autotune: rows upload");
   // the slice of the current state: self-energy rows, then timed history slices
+  // (of every active system: the policy concerns the FP64 pipe's kernel)
   BatchDev d = b->dev;
+  d.use_fx = 0;
   batch_plan<<<1, 256, (size_t)b->n_sys * 24, s>>>(d);
   batch_rows<kOpSigma><<<sm_count() * 8, 256, 0, s>>>(d);
   cudaEvent_t e0, e1;

@@ -29,6 +29,13 @@ constexpr int kOver = 6;       // chunks that a column tile visits twice, at mos
 constexpr int kHeadroom = 2;   // bits between a row's exponent and its first values
 constexpr int kNonFinite = 8000;  // exponent of a row or column that holds a non-finite value
 
+// Values of a per part, bytes of a part's small operand of one unit (two halves
+// of 64 exponent bytes and two variants of 8 digits x 16 reals x 2 NA columns),
+// complex entries of a partial slot.
+__host__ __device__ constexpr int part_rows(int M) { return M <= 8 ? 8 : 16; }
+__host__ __device__ constexpr int small_block_bytes(int NA) { return 2 * (64 + 2 * kDig * 2 * NA * 2 * kUnitK * 2); }
+__host__ __device__ constexpr int slot_complex(int NA) { return 2 * NA * kRows; }
+
 // One system's contraction as a list of column tiles of CT = 128 / M output
 // columns (times parts of NA rows a of the small operand).  For the slice the
 // output columns are the c of I(n, c) and the contracted points the m; for its
@@ -80,6 +87,12 @@ __host__ __device__ __forceinline__ void set_geometry(Sys& s, int M, int n, int 
   s.cta0 = 0;
   s.unit_base = s.chunk_base = s.entry_base = 0;
 }
+// Bytes of the small operands, rounded up to a 256-byte boundary (the partial sums follow).
+__host__ __device__ __forceinline__ size_t small_bytes(const Sys& s, int NA) {
+  return ((size_t)s.cpt * kChunkUnits * s.parts * small_block_bytes(NA) + 255) / 256 * 256;
+}
+// Prep items of a system: pairs of chunks x parts.
+__host__ __device__ __forceinline__ long long prep_items(const Sys& s) { return (long long)((s.cpt + 1) / 2) * s.parts; }
 
 // x / M for 0 <= x < 2^32 / M
 __host__ __device__ __forceinline__ int div_m(int x, int M, uint32_t magic) {

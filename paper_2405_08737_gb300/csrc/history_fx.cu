@@ -100,7 +100,8 @@ struct Cfg {
   static constexpr int kSmallBytes = 2 * kHalfBytes;             // small block of a unit: main half, band half
   static constexpr int kBufCols = kDig * kN;                     // accumulator buffer: 8 levels x kN columns
   static constexpr int kBufs = 512 / kBufCols;
-  static constexpr size_t kSlot = 2 * (size_t)NA * kRows;        // partial sums of one (CTA, tile): [2][NA][128] complex
+  static constexpr size_t kSlot = slot_complex(NA);              // partial sums of one (CTA, tile): [2][NA][128] complex
+  static_assert(kSmallBytes == small_block_bytes(NA), "small operand layout");
   // an epilogue still reading a group's exponents is at most kStages units and
   // the open and the buffered groups (4 units a buffer) behind the converters
   static_assert(kStages + kChunkUnits * (kBufs + 2) < kExpRing, "exponent ring");
@@ -807,14 +808,6 @@ __global__ void __launch_bounds__(256) fx_reduce(const __grid_constant__ Args a)
   }
 }
 
-int parts_of(int M) { return M <= 8 ? 8 : 16; }  // NA
-
-size_t small_bytes(const Sys& s, int NA) {
-  const size_t blk = NA == 8 ? Cfg<8>::kSmallBytes : Cfg<16>::kSmallBytes;
-  return ((size_t)s.cpt * kChunkUnits * s.parts * blk + 255) / 256 * 256;
-}
-size_t slot_bytes(int NA) { return 16 * (NA == 8 ? Cfg<8>::kSlot : Cfg<16>::kSlot); }
-
 // prep, contraction and reduction of the systems of `a`
 template <int NA>
 cudaError_t enqueue(const Args& a, bool quad, unsigned prep_blocks, unsigned red_blocks, cudaStream_t st, int* launches,
@@ -841,17 +834,17 @@ cudaError_t launch_one(Sys s, int M, int n, int band_w, int adj, void* work, siz
                        int* launches, cudaEvent_t ev_begin, cudaEvent_t ev_end) {
   *launches = 0;
   if (M < 1 || M > kMaxNorb || n < 0) return cudaErrorInvalidValue;
-  const int NA = parts_of(M);
+  const int NA = part_rows(M);
   set_geometry(s, M, n, band_w, adj, NA);
   s.small = reinterpret_cast<uint8_t*>(work);
   s.part = reinterpret_cast<double*>(s.small + small_bytes(s, NA));
   Args a{};
   a.one_head.n_sys = 1;
   a.one_head.total = (long long)s.tiles * s.upt;
-  a.one_head.chunks = (long long)(s.cpt + 1) / 2 * s.parts;
+  a.one_head.chunks = prep_items(s);
   a.one_head.entries = (long long)(n + 1) * M * M;
   a.G = (int)std::min<long long>(a.one_head.total, sm_count());
-  if (small_bytes(s, NA) + ((size_t)s.tiles + a.G) * slot_bytes(NA) > work_bytes) return cudaErrorInvalidValue;
+  if (small_bytes(s, NA) + ((size_t)s.tiles + a.G) * slot_complex(NA) * 16 > work_bytes) return cudaErrorInvalidValue;
   a.one = s;
   cudaError_t e = fx_prepare();
   if (e != cudaSuccess) return e;
@@ -866,9 +859,9 @@ cudaError_t launch_one(Sys s, int M, int n, int band_w, int adj, void* work, siz
 size_t fx_workspace_bytes(int M, int n_max) {
   if (M < 1 || M > kMaxNorb || n_max < 1) return 0;
   Sys s{};
-  const int NA = parts_of(M);
+  const int NA = part_rows(M);
   set_geometry(s, M, n_max - 1, kMaxOrder + 1, 0, NA);
-  return small_bytes(s, NA) + ((size_t)s.tiles + sm_count()) * slot_bytes(NA);
+  return small_bytes(s, NA) + ((size_t)s.tiles + sm_count()) * slot_complex(NA) * 16;
 }
 
 // The main kernels' dynamic shared memory exceeds the default limit (set once per device).
@@ -902,6 +895,17 @@ cudaError_t launch_history_fx(const HistoryArgs& h, void* work, size_t work_byte
   s.out1 = h.out + 2 * (size_t)(h.n + 1) * h.M * h.M;
   s.status = h.status;
   return launch_one(s, h.M, h.n, h.w.band_w, 0, work, work_bytes, st, launches, h.ev_begin, h.ev_end);
+}
+
+cudaError_t launch_fx_table(int NA, bool quad, const Sys* table, const Head* head, cudaStream_t st, int* launches) {
+  *launches = 0;
+  Args a{};
+  a.table = table;
+  a.head = head;
+  a.G = sm_count();
+  const unsigned prep = (unsigned)a.G * (NA == 8 ? 8 : 4), red = (unsigned)a.G * 8;
+  return NA == 8 ? enqueue<8>(a, quad, prep, red, st, launches, nullptr, nullptr)
+                 : enqueue<16>(a, quad, prep, red, st, launches, nullptr, nullptr);
 }
 
 // The Sigma-row cotangents of the slice's adjoint (the sums of adj_hist_small and its reduction).

@@ -137,3 +137,44 @@ def test_non_finite_entries(kbe, where, bad):
     ok = np.isfinite(b)
     assert np.abs(a[ok] - b[ok]).max() < TOL * np.abs(b[ok]).max()
     ctx.close()
+
+
+def test_batch_crosses_the_line(kbe):
+    """Batched steps whose rows move from the FP64 pipe to the tensor cores
+    (M = 8 from n = 98 on; M = 12 and M = 3 stay on either side): the rows of
+    kbe_step within 1e-13, whatever set of kernels the graph holds."""
+    import torch
+    sizes = [(8, 102), (12, 90), (3, 60), (8, 140)]
+    first = [95, 84, 54, 134]
+    runs = []
+    for batched in (False, True):
+        rs = []
+        for k, (M, n_t) in enumerate(sizes):
+            t, order = W.grid(n_t, 0.05, 0.4, 40 + k)
+            h = W.goe_h(M, k)
+            L, R, F = W.restart_state(h, W.half_filled_rho(h), t, order, first[k], n_t)
+            ctx = kbe.Context(M, n_t)
+            ctx.set_grid(t, order)
+            ctx.set_model(h, np.linspace(0.5, 1.5, M), W.site_potential(M), None)
+            r = kbe.Run(ctx)
+            r.L.copy_(torch.as_tensor(L, device="cuda"))
+            r.R.copy_(torch.as_tensor(R, device="cuda"))
+            for j, f in F.items():
+                r.F[j % kbe.KBE_RING_ROWS, :, : j + 1] = torch.as_tensor(f, device="cuda")
+            rs.append(r)
+        b = kbe.Batch(rs) if batched else None
+        for q in range(6):
+            if batched:
+                b.step([f + q for f in first], P=2)
+            else:
+                for f, r in zip(first, rs):
+                    r.step(f + q, P=2)
+        if batched:
+            b.sync_status()
+            b.close()
+        runs.append(rs)
+    for a, b in zip(*runs):
+        for x, y in ((a.L, b.L), (a.R, b.R)):
+            assert (x - y).abs().max() < 1e-13 * x.abs().max()
+        a.ctx.close()
+        b.ctx.close()

@@ -23,7 +23,7 @@ namespace fx {
 constexpr int kDig = 8;        // digits per value
 constexpr int kRows = 128;     // output rows (c, b) of a column tile, one tensor-memory lane each
 constexpr int kUnitK = 8;      // complex history entries of a unit (one MMA K step of 16 reals)
-constexpr int kChunkUnits = 4; // units accumulated in tensor memory: 2 planes x 64 reals x 8 digit pairs = 2^10 products
+constexpr int kChunkUnits = 4; // units of a chunk; two chunks of a plane accumulate: 128 reals x 8 digit pairs = 2^10
 constexpr int kChunkK = kUnitK * kChunkUnits;
 constexpr int kOver = 6;       // chunks that a column tile visits twice, at most (see Walk)
 constexpr int kHeadroom = 2;   // bits between a row's exponent and its first values
@@ -107,9 +107,8 @@ __host__ __device__ __forceinline__ int div_m(int x, int M, uint32_t magic) {
 enum Class { kFar = 0, kNear = 1, kBand = 2 };
 
 // The walk over the chunk slots of a system.  A column tile's chunks come in
-// this order: the far ones (entries with m <= c + shift count, both planes into
-// one sum), the near ones (m > c + shift, one sum per plane), and the band of
-// term 2 (its own weights w_{c,m}).  The at most kOver chunks that straddle the
+// this order: the far ones (entries with m <= c + shift count), the near ones
+// (m > c + shift), and the band of term 2 (its own weights w_{c,m}).  The at most kOver chunks that straddle the
 // line between far and near are taken once each way, with the other side's
 // entries masked; the remaining slots of a tile are empty.
 struct Walk {

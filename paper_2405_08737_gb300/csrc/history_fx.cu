@@ -23,8 +23,11 @@
 // tensor cores at about 1900, so 36 digit products cost a fiftieth of the FP64
 // ones.  What bounds it then is the conversion: every history entry is read in
 // both orientations and cut into digits with about 30 integer instructions per
-// real.  Measured, in this kernel: the slice n = 1023, M = 8 in 0.89 ms (7.05 on the
-// FP64 pipe, history_f64.cu), n = 511, M = 16 in 1.30 ms (14.4).
+// real, and the digit stores (64 KB a unit), the MMA operand reads and the history
+// loads share the L1 / shared-memory data pipe, about 70% busy (M = 8, n = 600: issue
+// slots 62%, tensor pipe 37%).  With NA = 16 the epilogue holds the MMAs back as well.
+// Measured, in this kernel: the slice n = 1023, M = 8 in 0.83 ms (7.05 on the FP64
+// pipe, history_f64.cu), n = 511, M = 16 in 1.23 ms (14.4).
 //
 // One persistent CTA per SM takes a contiguous range of chunks (32 history
 // entries of a 128-row column tile).  A unit is 8 entries, one MMA K step:
@@ -34,15 +37,18 @@
 //    the row's exponent with its neighbours and writes the digit planes
 //    (2 x 32 KB per unit) into a ring of two stages;
 //  * one thread copies the small operand's digits of each unit (bulk copies);
-//  * one thread issues the MMAs: digit i of the history against the stacked
-//    digits 0..7-i of the small operand, so the products of level i + j land in
-//    the columns of that level (N = 2 NA (8 - i) for a part of NA rows a);
-//  * eight epilogue warps fold a chunk's eight integer levels into one 64-bit
-//    integer, and that, scaled, into FP64 sums in registers: two FP64
-//    operations per 32 entries of an output.
+//  * two threads issue the MMAs, one per product of the unit: digit i of the
+//    history against the stacked digits 0..7-i of the small operand, so the
+//    products of level i + j land in the columns of that level (N = 2 NA (8 - i)
+//    for a part of NA rows a);
+//  * eight epilogue warps fold the eight integer levels of up to two chunks into
+//    one 64-bit integer, and that, scaled, into FP64 sums in registers: two FP64
+//    operations per 64 entries of an output.
 // Parts of NA = 8 rows a for M <= 8, else 16: a part's conversion of the history
 // serves all its rows (two sums of 16 x 8 levels fill tensor memory, so with NA =
-// 16 a near chunk waits for the epilogue of the one before).
+// 16 an accumulation waits for the epilogue of the one before).
+// One MMA thread instead of two: 0.88 and 1.31 ms for the two slices above.  History
+// loads of far quads as 4 x 16 instead of 2 x 32 bytes pass twice through the data pipe.
 // A row's exponent holds for the units accumulated together in tensor memory.
 // It starts kHeadroom bits above the larger of the unit's and the previous
 // chunk's largest entry; a unit that exceeds it nevertheless closes the
@@ -84,17 +90,17 @@ constexpr int kExpBytes = 64;                             // exponents of a part
 constexpr int kStages = 2, kBSlots = 4, kExpRing = 32;
 constexpr int kEpiWarps = 8;
 constexpr int kConvWarps = 16;                            // 8 rows each
-constexpr int kMmaWarp = kEpiWarps + kConvWarps, kProdWarp = kMmaWarp + 1;
+constexpr int kMmaWarp = kEpiWarps + kConvWarps, kProdWarp = kMmaWarp + 1, kMmaWarp2 = kMmaWarp + 2;
 constexpr int kThreads = (kProdWarp + 3) * 32;            // whole warpgroups (setmaxnreg): 896
 constexpr long long kSpinLimit = 1ll << 22;               // polls of the final waits
 constexpr long long kWaitCycles = 1ll << 31;              // a work wait gives up after about a second
-// registers of the warpgroups with NA = 16 (setmaxnreg; sums of 32 FP64 values a
-// thread): 8 x 32 x 104 + 16 x 32 x 64 + 4 x 32 x 40 = 896 x 72, the launch's own
-constexpr int kRegsEpi = 104, kRegsConv = 64, kRegsMisc = 40;
-
 template <int NA>
 struct Cfg {
   static constexpr int kN = 2 * NA;                              // real columns per digit of the small operand
+  // registers of the epilogue, converter and other warpgroups (setmaxnreg), whose
+  // sum is the launch's 896 x 72: an epilogue thread holds 2 NA FP64 sums
+  static constexpr int kRegsEpi = NA == 8 ? 104 : 112, kRegsConv = NA == 8 ? 64 : 56, kRegsMisc = NA == 8 ? 40 : 56;
+  static_assert(256 * kRegsEpi + 512 * kRegsConv + 128 * kRegsMisc == kThreads * 72, "register split");
   static constexpr int kVarBytes = 2 * kDig * (kN / 8) * 128;    // one variant's digits of a unit
   static constexpr int kHalfBytes = kExpBytes + 2 * kVarBytes;   // exponents | variant 0 | variant 1
   static constexpr int kSmallBytes = 2 * kHalfBytes;             // small block of a unit: main half, band half
@@ -102,8 +108,8 @@ struct Cfg {
   static constexpr int kBufs = 512 / kBufCols;
   static constexpr size_t kSlot = slot_complex(NA);              // partial sums of one (CTA, tile): [2][NA][128] complex
   static_assert(kSmallBytes == small_block_bytes(NA), "small operand layout");
-  // an epilogue still reading a group's exponents is at most kStages units and
-  // the open and the buffered groups (4 units a buffer) behind the converters
+  // an epilogue still reading an accumulation's exponents is at most kStages units
+  // and the open and the buffered ones (8 units per two buffers) behind the converters
   static_assert(kStages + kChunkUnits * (kBufs + 2) < kExpRing, "exponent ring");
 };
 
@@ -112,18 +118,22 @@ struct Cfg {
 // before the band, the end of a segment (a CTA's part of a tile: its sums go to
 // partial slot `aux`), or the end of the range.
 enum DescKind { kUnit = 0, kScale = 1, kFlush = 2, kEnd = 3 };
-enum DescFlags { kFlagNear = 1, kFlagBand = 2, kFirst = 4, kLast = 8, kFresh = 16, kNewTile = 32 };
+enum DescFlags { kFlagNear = 1, kFlagBand = 2, kFirst = 4, kLast = 8, kFresh = 16, kNewTile = 32, kFlagLow = 64 };
 struct alignas(16) Desc {
   int kap;    // first history entry
   int c0;     // first column of the tile
-  int flags;  // kind << 8 | DescFlags (first, last unit of its chunk; no chunk to follow; new tile)
+  int flags;  // a values of the part << 16 | kind << 8 | DescFlags (first, last unit of its chunk; no chunk to follow; new tile; far points
+              // may lie below the diagonal)
   int aux;    // system of the launch; partial slot (flush)
 };
+
+__device__ __forceinline__ int kind_of(int flags) { return flags >> 8 & 0xFF; }
 
 struct alignas(16) Post {  // what the MMA thread hands to the epilogue with a buffer
   int type;                // kUnit (sums), kScale, kFlush, kEnd
   int grp, eidx, plane;    // sum group (0: I^<, 1: D), exponent ring index and plane
-  int si, c0, slot, pad;   // system; first column (scale); partial slot (flush)
+  int si, c0, slot;        // system; first column (scale); partial slot (flush)
+  int cols;                // a values of the part, plus one
   int16_t es[16];          // small operand's exponents
 };
 
@@ -135,7 +145,7 @@ struct Smem {
   Post post[Cfg<NA>::kBufs];
   Desc desc[kBSlots];
   uint64_t full[kStages], empty[kStages], bfull[kBSlots], bempty[kBSlots];
-  uint64_t accfull[Cfg<NA>::kBufs], accempty[Cfg<NA>::kBufs], mmadone;
+  uint64_t accfull[Cfg<NA>::kBufs], accempty[Cfg<NA>::kBufs], mmadone[2];
   unsigned raise[kStages];            // 1 + the unit whose exponents start a new accumulation
   uint32_t tmem;
   int abort;
@@ -300,13 +310,14 @@ struct Row {
   const double2* dr;
   int n, edge;      // last point (-1: no such row), c + shift
   int diag;         // first point that is read directly: c, in the adjoint c + 1
-  int M;
+  int M, wide;      // wide: the plane starts on a 32-byte boundary
   uint32_t magic;
 };
 __device__ __forceinline__ Row row_of(const Sys& s, int c0, int j, int plane) {
   Row r;
   const double2* base = reinterpret_cast<const double2*>(plane ? s.R : s.L);
   r.M = s.M;
+  r.wide = (reinterpret_cast<uintptr_t>(base) & 31u) == 0;
   r.magic = s.magic;
   const int cl = div_m(j, r.M, r.magic), b = j - cl * r.M, MM = r.M * r.M;
   const int c = c0 + cl;
@@ -318,20 +329,45 @@ __device__ __forceinline__ Row row_of(const Sys& s, int c0, int j, int plane) {
   r.dr = base + (live ? (int64_t)c * MM + b : 0);
   return r;
 }
+// m (m + 1) / 2 as one 32 x 32 -> 64 bit product
+__device__ __forceinline__ uint64_t tri0(int m) {
+  const uint32_t h = (uint32_t)m >> 1, odd = (uint32_t)m & 1u;
+  return (uint64_t)(odd ? (uint32_t)m : h) * (odd ? h + 1 : (uint32_t)m + 1);
+}
 // Four consecutive entries from kap of a row; `mask` has bit i set where entry
 // i counts, bit 4 + i where it lies above the diagonal (the entry of the plane is
 // then -conj of the stored one).  kQuad (M a multiple of 4): the four share their
-// point m; masked entries load something valid instead of branching.
+// point m; masked entries load something valid instead of branching.  A slice's
+// far points (far_tr) all lie above the diagonal.
+// Two entries (32 bytes, 32-byte aligned) in one load: a far quad's 64 bytes lie
+// in a row of their own, and 16-byte loads of them took as many passes through
+// the L1 data pipe, which the digit stores and the MMA operands share, as both.
+__device__ __forceinline__ void ldg_pair(const double2* p, double2& x, double2& y) {
+  asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];" : "=d"(x.x), "=d"(x.y), "=d"(y.x), "=d"(y.y) : "l"(p));
+}
 template <bool kQuad>
-__device__ __forceinline__ void load_quad(const Row& r, int kap, bool near, double2 z[4], unsigned& mask) {
+__device__ __forceinline__ void load_quad(const Row& r, int kap, bool near, bool far_tr, double2 z[4], unsigned& mask) {
   const int M = r.M, MM = M * M;
   int m = div_m(kap, M, r.magic), x = kap - m * M;
   if (kQuad) {
+    if (far_tr) {
+      const bool in = m <= r.edge && r.n >= 0;
+      const double2* p = r.tr + (in ? (unsigned)(m * MM + x) : 0u);
+      if (r.wide) {
+        ldg_pair(p, z[0], z[1]);
+        ldg_pair(p + 2, z[2], z[3]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) z[i] = __ldg(p + i);
+      }
+      mask = in ? 0xFFu : 0u;
+      return;
+    }
     const bool in = m <= r.n && (near ? m > r.edge : m <= r.edge);
-    const bool above = m < r.diag;
-    const double2* p = above ? r.tr + (m * MM + x) : r.dr + (tri(m, 0) * MM + x * M);
-    int st = above ? 1 : M;
-    if (!in) { p = r.tr; st = 1; }
+    const bool above = m < r.diag || !in;
+    const double2* p = r.tr + (in ? (unsigned)(m * MM + x) : 0u);
+    if (!above) p = r.dr + (tri0(m) * (unsigned)MM + (unsigned)(x * M));
+    const unsigned st = above ? 1u : (unsigned)M;
 #pragma unroll
     for (int i = 0; i < 4; ++i) z[i] = __ldg(p + i * st);
     mask = (in ? 15u : 0u) | (above ? 0xF0u : 0u);
@@ -343,7 +379,7 @@ __device__ __forceinline__ void load_quad(const Row& r, int kap, bool near, doub
     const bool in = m <= r.n && (near ? m > r.edge : m <= r.edge);
     const bool above = m < r.diag;
     z[i] = make_double2(0.0, 0.0);
-    if (in) z[i] = __ldg(above ? r.tr + (m * MM + x) : r.dr + (tri(m, 0) * MM + x * M));
+    if (in) z[i] = __ldg(above ? r.tr + (m * MM + x) : r.dr + (tri0(m) * (unsigned)MM + (unsigned)(x * M)));
     mask |= ((unsigned)in | ((unsigned)above << 4)) << i;
     if (++x == M) { x = 0; ++m; }
   }
@@ -369,6 +405,65 @@ __device__ __noinline__ unsigned load_band(const Sys& s, const Row& r, int c, in
   return mask;
 }
 
+// ------------------------------------------------------------ epilogue ---
+// Folds the accumulator buffer at `at` into the FP64 sums s of this thread's row
+// and half of the a values, and hands the buffer back (empty) once its levels are
+// in registers.  kWhole: every a value of the part is in use (otherwise the
+// columns past the last one are skipped).
+template <int NA, bool kWhole>
+__device__ __forceinline__ void fold(double (&s)[NA], uint32_t at, int E, int half, const Post& ps, uint64_t* empty) {
+  constexpr int kN = 2 * NA, kC = NA, kCols = NA == 8 ? 2 : 1;  // kCols: columns in registers at a time
+  const int cols = kWhole ? kC : (ps.cols - half) & ~1;
+  uint32_t r[kDig][kCols];
+  auto read = [&](int c2) {  // the levels of columns c2, ... in flight
+#pragma unroll
+    for (int d = 0; d < kDig; ++d) {
+      const uint32_t p = at + d * kN + 2 * c2 - c2 % 2;
+      if constexpr (kCols == 2)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(r[d][0]), "=r"(r[d][kCols - 1]) : "r"(p));
+      else
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[d][0]) : "r"(p));
+    }
+  };
+  read(0);
+#pragma unroll
+  for (int c2 = 0; c2 < kC; c2 += kCols) {
+    if (!kWhole && c2 > 0 && c2 >= cols) continue;
+    const int es = ps.es[2 * (c2 / 2) + half];
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    int v[kDig][kCols];
+#pragma unroll
+    for (int i = 0; i < kCols; ++i)
+#pragma unroll
+      for (int d = 0; d < kDig; ++d) v[d][i] = __float2int_rn(__uint_as_float(r[d][i]));
+    if (c2 + kCols < cols) {
+      read(c2 + kCols);  // while these are folded
+    } else {
+      tc_fence_before();
+      __syncwarp();
+      if ((threadIdx.x & 31) == 0) mbar_arrive(empty);
+    }
+    // scale 2^(ev + eu - 68 + 12), ev = E - 1022, eu = es - 1022
+    const int ex = E + es - 2 * 1022 - 56;
+#pragma unroll
+    for (int i = 0; i < kCols; ++i) {
+      // the 64-bit integer sum_l S_l 256^(7-l) / 2^12: |S_0| <= 2^19, |S_1| <= 2^21, |S_2| <= 2^22 and
+      // |S_l| <= l 2^21 fit the 32-bit steps, and 2^10 products of 62-bit values stay below 2^(124+7-56-12)
+      const uint64_t p01 = (uint64_t)(int64_t)(v[0][i] * 256 + v[1][i]), p23 = (uint64_t)(int64_t)(v[2][i] * 256 + v[3][i]);
+      const int low = v[5][i] * 16 + ((v[6][i] + (v[7][i] >> 8) + 8) >> 4);
+      const int64_t t = (int64_t)((p01 << 36) + (p23 << 20) + ((uint64_t)(int64_t)v[4][i] << 12) + (uint64_t)(int64_t)low);
+      if (ex >= -1022 && ex <= 1023) {
+        s[c2 + i] = fma((double)t, __hiloint2double((ex + 1023) << 20, 0), s[c2 + i]);
+      } else if (ex >= kNonFinite - 4096) {
+        s[c2 + i] = __longlong_as_double(0x7FF8000000000000ll);
+      } else {  // the scale alone leaves the range of FP64
+        const int h = ex / 2;
+        s[c2 + i] += (double)t * __hiloint2double((h + 1023) << 20, 0) * __hiloint2double((ex - h + 1023) << 20, 0);
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------- main ---
 template <int NA, bool kQuad>
 __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ Args a) {
@@ -382,11 +477,13 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
   int* const status = sys_at(a, 0).status;
 
   if (tid == 0) {
-    for (int i = 0; i < kStages; ++i) { mbar_init(&sm.full[i], kConvWarps); mbar_init(&sm.empty[i], 1); sm.raise[i] = 0; }
-    for (int i = 0; i < kBSlots; ++i) { mbar_init(&sm.bfull[i], 1); mbar_init(&sm.bempty[i], 1); }
-    // accfull: the MMA thread's arrival (post written) and its commit; accempty: one lane per epilogue warp
+    // empty, bempty: both MMA threads
+    for (int i = 0; i < kStages; ++i) { mbar_init(&sm.full[i], kConvWarps); mbar_init(&sm.empty[i], 2); sm.raise[i] = 0; }
+    for (int i = 0; i < kBSlots; ++i) { mbar_init(&sm.bfull[i], 1); mbar_init(&sm.bempty[i], 2); }
+    // accfull: an MMA thread's arrival (post written) and its commit; accempty: one lane per epilogue warp
     for (int i = 0; i < kBufs; ++i) { mbar_init(&sm.accfull[i], 2); mbar_init(&sm.accempty[i], kEpiWarps); }
-    mbar_init(&sm.mmadone, 1);
+    mbar_init(&sm.mmadone[0], 1);
+    mbar_init(&sm.mmadone[1], 1);
     sm.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -403,23 +500,26 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
 
   if (warp < kEpiWarps) {
     // --------------------------------------------------------- epilogue --
-    // warp = 4 half + quadrant: 32 output rows (tensor-memory lanes), half of
-    // the part's a values (kN / 2 columns)
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
-    constexpr int kC = kN / 2, kCols = NA == 8 ? 2 : 1;  // columns in registers at a time
+    // warp = 4 half + quadrant: 32 output rows (tensor-memory lanes), the even
+    // or the odd a values of the part (kN / 2 columns)
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::kRegsEpi));
+    constexpr int kC = kN / 2;
     const int quad = warp & 3, half = warp >> 2;
     const int j = quad * 32 + lane;
-    const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16) + half * kC;
+    const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16) + 2 * half;  // + 4 (c / 2) + c % 2
     double acc[2][kC];
 #pragma unroll
     for (int i = 0; i < kC; ++i) acc[0][i] = acc[1][i] = 0.0;
-    for (unsigned p = 0;; ++p) {
-      const int buf = p % kBufs;
-      if (!__all_sync(0xffffffffu, wait_bar(&sm.abort, &sm.accfull[buf], (p / kBufs) & 1, status))) break;
+    unsigned used[2] = {0, 0};  // buffers taken from each MMA thread
+    for (int from = 0;;) {      // thread 0's message, or its sum and then thread 1's
+      const unsigned k = from ? used[1]++ : used[0]++;
+      const int buf = 2 * (k % (kBufs / 2)) + from;
+      if (!__all_sync(0xffffffffu, wait_bar(&sm.abort, &sm.accfull[buf], (k / (kBufs / 2)) & 1, status))) break;
       tc_fence_after();
       const Post& ps = sm.post[buf];
       const int type = ps.type;
       if (type == kEnd) break;
+      if (type == kUnit) from ^= 1;
       if (type != kUnit) {
         const Sys& s = sys_at(a, ps.si);
         if (type == kFlush) {
@@ -428,7 +528,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
           for (int g = 0; g < 2; ++g)
 #pragma unroll
             for (int i = 0; i < kC / 2; ++i) {
-              out[(g * NA + half * (NA / 2) + i) * kRows + j] = make_double2(acc[g][2 * i], acc[g][2 * i + 1]);
+              out[(g * NA + 2 * i + half) * kRows + j] = make_double2(acc[g][2 * i], acc[g][2 * i + 1]);
               acc[g][2 * i] = acc[g][2 * i + 1] = 0.0;
             }
         } else {  // the adjoint's sums, before its band
@@ -446,64 +546,21 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       }
       const int g = ps.grp;
       const int E = sm.erow[ps.eidx][ps.plane][j];
-      // the levels of kCols columns from column c2 of the buffer
-      uint32_t r[kDig][kCols];
-      auto read = [&](int c2) {
-#pragma unroll
-        for (int d = 0; d < kDig; ++d) {
-          const uint32_t at = lane_addr + buf * kBufCols + d * kN + c2;
-          if constexpr (kCols == 2)
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(r[d][0]), "=r"(r[d][kCols - 1]) : "r"(at));
-          else
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[d][0]) : "r"(at));
-        }
-      };
-      auto fold = [&](double(&s)[kC]) {
-        read(0);
-#pragma unroll
-        for (int c2 = 0; c2 < kC; c2 += kCols) {
-          const int es = ps.es[half * (NA / 2) + c2 / 2];
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          int v[kDig][kCols];
-#pragma unroll
-          for (int i = 0; i < kCols; ++i)
-#pragma unroll
-            for (int d = 0; d < kDig; ++d) v[d][i] = __float2int_rn(__uint_as_float(r[d][i]));
-          if (c2 + kCols < kC) {
-            read(c2 + kCols);  // in flight while these are folded
-          } else {             // every level of this buffer is in registers
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.accempty[buf]);
-          }
-          // scale 2^(ev + eu - 68 + 12), ev = E - 1022, eu = es - 1022
-          const int ex = E + es - 2 * 1022 - 56;
-#pragma unroll
-          for (int i = 0; i < kCols; ++i) {
-            // the 64-bit integer sum_l S_l 256^(7-l) / 2^12: |S_0| <= 2^19, |S_1| <= 2^21, |S_2| <= 2^22 and
-            // |S_l| <= l 2^21 fit the 32-bit steps, and 2^10 products of 62-bit values stay below 2^(124+7-56-12)
-            const uint64_t p01 = (uint64_t)(int64_t)(v[0][i] * 256 + v[1][i]), p23 = (uint64_t)(int64_t)(v[2][i] * 256 + v[3][i]);
-            const int low = v[5][i] * 16 + ((v[6][i] + (v[7][i] >> 8) + 8) >> 4);
-            const int64_t t =
-                (int64_t)((p01 << 36) + (p23 << 20) + ((uint64_t)(int64_t)v[4][i] << 12) + (uint64_t)(int64_t)low);
-            if (ex >= -1022 && ex <= 1023) {
-              s[c2 + i] = fma((double)t, __hiloint2double((ex + 1023) << 20, 0), s[c2 + i]);
-            } else if (ex >= kNonFinite - 4096) {
-              s[c2 + i] = __longlong_as_double(0x7FF8000000000000ll);
-            } else {  // the scale alone leaves the range of FP64
-              const int h = ex / 2;
-              s[c2 + i] += (double)t * __hiloint2double((h + 1023) << 20, 0) * __hiloint2double((ex - h + 1023) << 20, 0);
-            }
-          }
-        }
-      };
-      if (g == 0) fold(acc[0]); else fold(acc[1]);
+      uint64_t* const empty = &sm.accempty[buf];
+      const uint32_t at = lane_addr + buf * kBufCols;
+      if (ps.cols > NA) {
+        if (g == 0) fold<NA, true>(acc[0], at, E, half, ps, empty);
+        else fold<NA, true>(acc[1], at, E, half, ps, empty);
+      } else {
+        if (g == 0) fold<NA, false>(acc[0], at, E, half, ps, empty);
+        else fold<NA, false>(acc[1], at, E, half, ps, empty);
+      }
     }
   } else if (warp < kMmaWarp) {
     // ------------------------------------------------------- converters --
     // lane = row (3 bits) | K half q << 3 | plane << 4: a quarter warp writes
     // 128 consecutive bytes of a digit plane
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsConv));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsConv));
     const int wq = warp - kEpiWarps;
     const int q = (lane >> 3) & 1, plane = lane >> 4;
     const uint32_t dst0 = plane * kPlane + (q * 16 + wq) * 128 + (lane & 7) * 16;
@@ -519,9 +576,9 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
         if (!__all_sync(0xffffffffu, wait_bar(&sm.abort, &sm.bfull[b], (d / kBSlots) & 1, status))) return false;
         ds = sm.desc[b];
         ++d;
-      } while (ds.flags >> 8 == kFlush || ds.flags >> 8 == kScale);
+      } while (kind_of(ds.flags) == kFlush || kind_of(ds.flags) == kScale);
       flags = ds.flags;
-      if (flags >> 8 == kEnd) return false;
+      if (kind_of(flags) == kEnd) return false;
       if (flags & kNewTile) row = row_of(sys_at(a, ds.aux), ds.c0, 8 * wq + (lane & 7), plane);
       const int kap = ds.kap + 4 * q;
       if (flags & kFlagBand) {
@@ -532,25 +589,21 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
         for (int i = 0; i < 4; ++i) z[i] = plane ? v[i] : make_double2(0.0, 0.0);
         if (mask) mask = 15u;  // the others are zero
       } else {
-        load_quad<kQuad>(row, kap, flags & kFlagNear, z, mask);
+        load_quad<kQuad>(row, kap, flags & kFlagNear, !(flags & (kFlagNear | kFlagLow)), z, mask);
       }
       return true;
     };
     bool more = load();
     for (unsigned u = 0; more; ++u) {
       const int s = u % kStages;
-      // exponent of the row (far units: of both planes, which go into one sum)
+      // exponent of the row
       int mx = 0;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int h = max(__double2hiint(z[i].x) & 0x7FFFFFFF, __double2hiint(z[i].y) & 0x7FFFFFFF);
-        mx = max(mx, h);  // masked entries are zero without kQuad
-      }
+      for (int i = 0; i < 4; ++i)  // masked entries are zero without kQuad
+        mx = __vimax3_s32(mx, __double2hiint(z[i].x) & 0x7FFFFFFF, __double2hiint(z[i].y) & 0x7FFFFFFF);
       if (kQuad && !(mask & 1u)) mx = 0;
       mx >>= 20;
       mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
-      const int other = __shfl_xor_sync(0xffffffffu, mx, 16);
-      if (!(flags & (kFlagNear | kFlagBand))) mx = max(mx, other);
       bool raised = false;
       if (flags & kFirst) {
         const int prev = (flags & kFresh) || seen == 0x7FF ? 0 : seen;
@@ -566,7 +619,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       uint64_t br[4], bi[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const uint32_t fl = (mask << (27 - i)) & 0x80000000u;
+        const uint32_t fl = (kQuad ? mask << 24 : mask << (27 - i)) & 0x80000000u;
         br[i] = digit_bytes((uint32_t)__double2hiint(z[i].x) ^ fl, (uint32_t)__double2loint(z[i].x), Ez);
         bi[i] = digit_bytes((uint32_t)__double2hiint(z[i].y), (uint32_t)__double2loint(z[i].y), Ez);
       }
@@ -585,7 +638,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       if (lane == 0) mbar_arrive(&sm.full[s]);
     }
   } else {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsMisc));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsMisc));
     if (warp == kProdWarp && lane == 0) {
       // ------------------------------------------------------- producer --
       unsigned d = 0;
@@ -616,15 +669,17 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
             if (!message(kScale, 0, w.c0, si)) break;
             scaled = true;
           }
-          // a near sum takes one plane, so two chunks (an even one and the next)
-          // stay within 2^10 products and are accumulated together
-          const bool join = w.cls == kNear && !(w.kc & 1) && q + 1 < q1 && w.idx + 1 < w.nfar + S->cpt - w.first;
+          // a sum takes one plane, so two chunks (an even one and the next) stay
+          // within 2^10 products of 2^14 and are accumulated together
+          const bool join = w.cls != kBand && !(w.kc & 1) && q + 1 < q1 &&
+                            w.idx + 1 < (w.cls == kFar ? w.nfar : w.nfar + S->cpt - w.first);
           const uint32_t bytes = kExpBytes + (w.cls == kNear ? 1 : 2) * C::kVarBytes;
           const uint8_t* src = S->small + (w.cls == kBand ? C::kHalfBytes : 0) +
                                ((size_t)w.kc * kChunkUnits * S->parts + w.part) * C::kSmallBytes;
           for (int unit = w.j0; unit < w.j1; ++unit) {
             const int flags = (w.cls == kNear ? kFlagNear : 0) | (w.cls == kBand ? kFlagBand : 0) |
-                              (unit == w.j0 && !joined ? kFirst : 0) | (unit + 1 == w.j1 && !join ? kLast : 0);
+                              (unit == w.j0 && !joined ? kFirst : 0) | (unit + 1 == w.j1 && !join ? kLast : 0) |
+                              (S->adj ? kFlagLow : 0) | min(NA, S->M - w.part * NA) << 16;
             if (!put(w.kc * kChunkK + unit * kUnitK, w.c0, kUnit << 8 | flags | fresh, si)) { stop = true; break; }
             const int b = d % kBSlots;
             mbar_arrive_expect_tx(&sm.bfull[b], bytes);
@@ -660,27 +715,37 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
         while (!mbar_try(&sm.bfull[k % kBSlots], (k / kBSlots) & 1) && ++spins < kSpinLimit) __nanosleep(64);
         if (spins >= kSpinLimit) atomicOr(status, kStatusTimeout);
       }
-    } else if (warp == kMmaWarp && lane == 0) {
-      // ------------------------------------------------------------ MMA --
+    } else if ((warp == kMmaWarp || warp == kMmaWarp2) && lane == 0) {
+      // ----------------------------------------------------- MMA threads --
+      // Thread 0 issues the first of a unit's two products, thread 1 the second,
+      // each into accumulator buffers of its own: one alone leaves the tensor
+      // cores idle between its units.  Both walk the same descriptors; thread
+      // `me` takes the buffers me, me + 2, ... in turn.
       // A: [digit 8][K group 2][row group 16][8 rows][16 B]; B: [K group 2][digit 8][column group][8][16 B]
+      const int me = warp == kMmaWarp ? 0 : 1;
       const uint64_t a0 = umma_desc(smem_u32(sm.stage[0]), kRows * 16, 128);
       const uint64_t b0 = umma_desc(smem_u32(sm.small[0] + kExpBytes), kDig * (kN / 8) * 128, 128);
-      unsigned u = 0, p = 0;
+      unsigned u = 0, k = 0;  // units; this thread's buffers taken
       bool any = false, stop = false, open = false;
-      int nb = 0;  // buffers of the open group
       unsigned held = 0;  // slots (bits) of messages not released yet
+      int buf = me;
+      auto next_buffer = [&]() {
+        ++k;
+        buf = 2 * (k % (kBufs / 2)) + me;
+      };
+      auto wait_buffer = [&]() {
+        return wait_bar(&sm.abort, &sm.accempty[buf], ((k / (kBufs / 2)) & 1) ^ 1, status);
+      };
       auto close = [&]() {
-        for (int k = 0; k < nb; ++k) {
-          mbar_arrive(&sm.accfull[(p + k) % kBufs]);
-          umma_commit(&sm.accfull[(p + k) % kBufs]);
-        }
-        p += nb;
+        mbar_arrive(&sm.accfull[buf]);
+        umma_commit(&sm.accfull[buf]);
+        next_buffer();
         open = false;
       };
-      // hands a message without sums to the epilogue
+      // hands a message without sums to the epilogue (thread 0)
       auto message = [&](int type, int si, int c0, int slot) -> bool {
-        const int buf = p % kBufs;
-        if (!wait_bar(&sm.abort, &sm.accempty[buf], ((p / kBufs) & 1) ^ 1, status)) return false;
+        if (me) return true;
+        if (!wait_buffer()) return false;
         Post& ps = sm.post[buf];
         ps.type = type;
         ps.si = si;
@@ -688,14 +753,14 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
         ps.slot = slot;
         mbar_arrive(&sm.accfull[buf]);
         mbar_arrive(&sm.accfull[buf]);
-        ++p;
+        next_buffer();
         return true;
       };
       for (unsigned d = 0; !stop; ++d) {
         const int b = d % kBSlots;
         if (!wait_bar(&sm.abort, &sm.bfull[b], (d / kBSlots) & 1, status)) { stop = true; break; }
         const Desc ds = sm.desc[b];
-        const int kind = ds.flags >> 8;
+        const int kind = kind_of(ds.flags);
         if (kind == kEnd) break;
         if (kind != kUnit) {
           // released when the next unit is full: then every converter has read
@@ -706,64 +771,49 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
           continue;
         }
         const int s = u % kStages;
-        const bool two = ds.flags & (kFlagNear | kFlagBand), band = ds.flags & kFlagBand;
+        const bool near = ds.flags & kFlagNear, band = ds.flags & kFlagBand;
         if (!wait_bar(&sm.abort, &sm.full[s], (u / kStages) & 1, status)) { stop = true; break; }
-        for (int k = 0; k < kBSlots && held; ++k)
-          if (held >> k & 1u) {
-            mbar_arrive(&sm.bempty[k]);
-            held &= ~(1u << k);
+        for (int i = 0; i < kBSlots && held; ++i)
+          if (held >> i & 1u) {
+            mbar_arrive(&sm.bempty[i]);
+            held &= ~(1u << i);
           }
         const bool begin = (ds.flags & kFirst) || *(volatile unsigned*)&sm.raise[s] == u + 1;
         if (begin) {
           if (open) close();
-          nb = two ? 2 : 1;
           open = true;
-        }
-        // the buffer of sum g of a new accumulation
-        auto begin_sum = [&](int g) -> bool {
-          const int buf = (p + g) % kBufs;
-          if (!wait_bar(&sm.abort, &sm.accempty[buf], (((p + g) / kBufs) & 1) ^ 1, status)) return false;
+          if (!wait_buffer()) { stop = true; break; }
           Post& ps = sm.post[buf];
           ps.type = kUnit;
-          ps.grp = g;
+          ps.grp = me && (near || band);
           ps.eidx = u % kExpRing;
-          ps.plane = band ? 1 : g;
+          ps.plane = band ? 1 : me;
+          ps.cols = (ds.flags >> 16) + 1;
 #pragma unroll
           for (int i = 0; i < NA / 8; ++i)
             reinterpret_cast<int4*>(ps.es)[i] = reinterpret_cast<const int4*>(sm.small[b])[i];
-          return true;
-        };
-        if (begin && !begin_sum(0)) { stop = true; break; }
-        tc_fence_after();
-        // far: PL x variant 0 and Q x variant 1 into one sum; near: PL and Q x
-        // variant 0 into two; band: Q x variant 0 and 1 into two
-        const uint64_t dP = a0 + ((uint64_t)(s * 2 * kPlane) >> 4), dQ = dP + (kPlane >> 4);
-        const uint64_t dA = b0 + ((uint64_t)(b * C::kHalfBytes) >> 4);
-        const uint64_t x0 = band ? dQ : dP, v1 = two && !band ? dA : dA + (C::kVarBytes >> 4);
-        const uint32_t t0 = tmem + (p % kBufs) * kBufCols, t1 = two ? tmem + ((p + 1) % kBufs) * kBufCols : t0;
-#pragma unroll
-        for (int i = 0; i < kDig; ++i)
-          umma_f16(t0 + i * kN, x0 + ((i * kDigPlane) >> 4), dA, umma_idesc_f16(kN * (kDig - i)), !(begin && i == 0));
-        any = true;
-        if (begin && two) {
-          if (!begin_sum(1)) { stop = true; break; }
-          tc_fence_after();
         }
+        tc_fence_after();
+        // far: PL x variant 0 and Q x variant 1, both to I^<; near: PL and Q x
+        // variant 0 to I^< and D; band: Q x variants 0 and 1 to I^< and D
+        const uint64_t x = a0 + ((uint64_t)(s * 2 * kPlane + (me || band ? kPlane : 0)) >> 4);
+        const uint64_t v = b0 + ((uint64_t)(b * C::kHalfBytes + (me && !near ? C::kVarBytes : 0)) >> 4);
+        const uint32_t t = tmem + buf * kBufCols;
 #pragma unroll
         for (int i = 0; i < kDig; ++i)
-          umma_f16(t1 + i * kN, dQ + ((i * kDigPlane) >> 4), v1, umma_idesc_f16(kN * (kDig - i)),
-                   !(begin && two && i == 0));
+          umma_f16(t + i * kN, x + ((i * kDigPlane) >> 4), v, umma_idesc_f16(kN * (kDig - i)), !(begin && i == 0));
         umma_commit(&sm.empty[s]);
         umma_commit(&sm.bempty[b]);
+        any = true;
         ++u;
         if (ds.flags & kLast) close();
       }
       if (!stop) message(kEnd, 0, 0, 0);
       // every MMA must complete before tensor memory is freed
       if (any) {
-        umma_commit(&sm.mmadone);
+        umma_commit(&sm.mmadone[me]);
         long long spins = 0;
-        while (!mbar_try(&sm.mmadone, 0) && ++spins < kSpinLimit) __nanosleep(64);
+        while (!mbar_try(&sm.mmadone[me], 0) && ++spins < kSpinLimit) __nanosleep(64);
         if (spins >= kSpinLimit) atomicOr(status, kStatusTimeout);
       }
     }

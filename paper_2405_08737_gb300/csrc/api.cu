@@ -203,10 +203,16 @@ void adjoint_fx(const kbe_ctx* ctx, AdjHistArgs* h) {
 // Self-energy of n_blocks blocks from first_block (launch_sigma geometry),
 // with the context's interaction: the local U or the dense tensor.
 cudaError_t sigma_blocks(kbe_ctx* ctx, int64_t first_block, int64_t n_blocks, int64_t diag_rel, const void* L,
-                         const void* R, void* Sl, void* Sg, cudaStream_t s) {
-  if (ctx->dense)
-    return launch_sigma_dense(ctx->M, first_block, n_blocks, diag_rel, (const double*)L, (const double*)R,
-                              ctx->d_Ut, ctx->d_Xt, (double*)Sl, (double*)Sg, ctx->d_status, s);
+                         const void* R, void* Sl, void* Sg, cudaStream_t s, int* launches) {
+  if (ctx->dense) {  // the slice workspace is free until the history slice of this row
+    int k = 0;
+    const cudaError_t e = launch_sigma_dense(ctx->M, first_block, n_blocks, diag_rel, (const double*)L,
+                                             (const double*)R, ctx->d_Ut, ctx->d_Xt, (double*)Sl, (double*)Sg,
+                                             ctx->d_status, ctx->d_part, ctx->part_bytes, s, &k);
+    *launches += k;
+    return e;
+  }
+  ++*launches;
   return launch_sigma(ctx->M, first_block, n_blocks, diag_rel, (const double*)L, (const double*)R, ctx->d_U,
                       (double*)Sl, (double*)Sg, ctx->d_status, s);
 }
@@ -365,8 +371,8 @@ kbe_status step_impl(kbe_ctx* ctx, int n, int P, int precision, void* L, void* R
   if (e != cudaSuccess) return cuda_fail(ctx, e, "kbe_step: predictor");
   for (int it = 0; it < P; ++it) {
     if ((e = keep(it)) != cudaSuccess) return cuda_fail(ctx, e, "kbe_step: iterate copy");
-    e = sigma_blocks(ctx, tri(n, 0), n + 1, n, L, R, Sl, Sg, s);
-    *count_out = ++count;
+    e = sigma_blocks(ctx, tri(n, 0), n + 1, n, L, R, Sl, Sg, s, &count);
+    *count_out = count;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "kbe_step: self-energy");
     if (ctx->adaptive_K > 0) {  // history order of interval n from this sweep's rows (Sec. 3.2)
       SelectArgs sa{ctx->M, n, ctx->adaptive_K, (const double*)L, (const double*)R, (const double*)Sl,
@@ -573,8 +579,7 @@ kbe_status ctl_workspace(kbe_ctx* ctx) {
 // right-hand side row n from the current row n (Sigma, order choice, slice, eps, F)
 kbe_status ctl_feval(CtlRun& r, int n) {
   kbe_ctx* ctx = r.ctx;
-  cudaError_t e = sigma_blocks(ctx, tri(n, 0), n + 1, n, r.L, r.R, r.Sl, r.Sg, r.s);
-  ++r.launches;
+  cudaError_t e = sigma_blocks(ctx, tri(n, 0), n + 1, n, r.L, r.R, r.Sl, r.Sg, r.s, &r.launches);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "kbe_run_controlled: self-energy");
   if (r.K_sel > 0 && n > 0) {
     SelectArgs sa{ctx->M, n, r.K_sel, (const double*)r.L, (const double*)r.R, (const double*)r.Sl,
@@ -602,11 +607,11 @@ kbe_status ctl_store(CtlRun& r, int n) {
   kbe_ctx* ctx = r.ctx;
   const size_t srow = (size_t)r.n_max * ctx->M * ctx->M * 2;  // doubles per s-row
   double* slot = r.Sring + (size_t)(n % kRing) * 2 * srow;
-  cudaError_t e = sigma_blocks(ctx, tri(n, 0), n + 1, n, r.L, r.R, slot, slot + srow, r.s);
+  cudaError_t e = sigma_blocks(ctx, tri(n, 0), n + 1, n, r.L, r.R, slot, slot + srow, r.s, &r.launches);
   StepArgs a = step_args(ctx, n, r.L, r.R, r.I, r.F);
   a.eps = r.eps_ring + (size_t)(n % kRing) * ctx->M * ctx->M * 2;
   if (e == cudaSuccess) e = launch_fock(a, r.s);
-  r.launches += 2;
+  ++r.launches;
   return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "kbe_run_controlled: accepted row");
 }
 
@@ -949,8 +954,7 @@ kbe_status kbe_selfenergy_slice(kbe_ctx* ctx, int n, const void* L, const void* 
   if (!aligned16(L) || !aligned16(R) || !aligned16(Sl) || !aligned16(Sg))
     return fail(ctx, KBE_EINVAL, "kbe_selfenergy_slice: NULL or misaligned pointer");
   if ((st = use_device(ctx)) != KBE_OK) return st;
-  cudaError_t e = sigma_blocks(ctx, tri(n, 0), n + 1, n, L, R, Sl, Sg, (cudaStream_t)stream);
-  ctx->last_launches = 1;
+  cudaError_t e = sigma_blocks(ctx, tri(n, 0), n + 1, n, L, R, Sl, Sg, (cudaStream_t)stream, &ctx->last_launches);
   return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "kbe_selfenergy_slice");
 }
 
@@ -964,8 +968,7 @@ kbe_status kbe_selfenergy_all(kbe_ctx* ctx, int n_rows, const void* L, const voi
     return fail(ctx, KBE_EINVAL, "kbe_selfenergy_all: NULL or misaligned pointer");
   kbe_status st = use_device(ctx);
   if (st != KBE_OK) return st;
-  cudaError_t e = sigma_blocks(ctx, 0, tri(n_rows, 0), -1, L, R, Sl, Sg, (cudaStream_t)stream);
-  ctx->last_launches = 1;
+  cudaError_t e = sigma_blocks(ctx, 0, tri(n_rows, 0), -1, L, R, Sl, Sg, (cudaStream_t)stream, &ctx->last_launches);
   return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "kbe_selfenergy_all");
 }
 
@@ -1041,8 +1044,8 @@ kbe_status kbe_step_sweep_band(kbe_ctx* ctx, int n, int row_lo, int row_hi, cons
   if (!aligned16(L) || !aligned16(R) || !aligned16(S_less) || !aligned16(S_great) || !aligned16(I_part))
     return fail(ctx, KBE_EINVAL, "kbe_step_sweep_band: NULL or misaligned pointer");
   cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = sigma_blocks(ctx, tri(n, 0), n + 1, n, L, R, S_less, S_great, s);
-  if (e != cudaSuccess) { ctx->last_launches = 1; return cuda_fail(ctx, e, "kbe_step_sweep_band: self-energy"); }
+  cudaError_t e = sigma_blocks(ctx, tri(n, 0), n + 1, n, L, R, S_less, S_great, s, &ctx->last_launches);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "kbe_step_sweep_band: self-energy");
   HistoryArgs a{ctx->M, n, (const double*)L, (const double*)R, (const double*)S_less, (const double*)S_great,
                 weights_view(ctx), (double*)I_part, ctx->d_part, ctx->part_bytes, ctx->d_status};
   a.band_lo = row_lo;
@@ -1050,7 +1053,7 @@ kbe_status kbe_step_sweep_band(kbe_ctx* ctx, int n, int row_lo, int row_hi, cons
   if (!next_events(ctx, &a.ev_begin, &a.ev_end)) return fail(ctx, KBE_ECUDA, "profiling: cudaEventCreate");
   int nl = 0;
   e = slice_f64(ctx, a, s, &nl);
-  ctx->last_launches = 1 + nl;
+  ctx->last_launches += nl;
   return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "kbe_step_sweep_band: history slice");
 }
 
@@ -1133,8 +1136,7 @@ kbe_status kbe_rhs_row(kbe_ctx* ctx, int j, int precision, const void* L, const 
   if ((st = use_device(ctx)) != KBE_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
   int count = 0, nl = 0;
-  cudaError_t e = sigma_blocks(ctx, tri(j, 0), j + 1, j, L, R, Sl, Sg, s);
-  ++count;
+  cudaError_t e = sigma_blocks(ctx, tri(j, 0), j + 1, j, L, R, Sl, Sg, s, &count);
   if (e != cudaSuccess) { ctx->last_launches = count; return cuda_fail(ctx, e, "kbe_rhs_row: self-energy"); }
   st = history(ctx, j, precision, L, R, Sl, Sg, I_work, s, &nl);
   count += nl;

@@ -56,11 +56,14 @@ __global__ void __launch_bounds__(kThreads) sigma_dense_kernel(DenseSigmaArgs a)
   double2* sQ = sT + g * MM;
   double2* sP = sQ + g * MM;
   const int tid = threadIdx.x;
-  const int64_t n_units = 2 * a.n_blocks;
+  const int64_t n_units = 2 * a.n_blocks * a.slices;
   bool ok = true;
   for (int64_t u = blockIdx.x; u < n_units; u += gridDim.x) {
-    const int64_t blk = u >> 1;
-    const int s = (int)(u & 1);
+    const int64_t blk = (u >> 1) / a.slices;
+    const int s = (int)(u & 1), slice = (int)((u >> 1) - blk * a.slices);
+    // this unit's pairs (d, b), whole tiles of g
+    const int tiles = (MM + g - 1) / g;
+    const int q_lo = tiles * slice / a.slices * g, q_hi = min(MM, tiles * (slice + 1) / a.slices * g);
     bool diag;
     if (a.diag_rel >= 0) {
       diag = blk == a.diag_rel;
@@ -86,8 +89,8 @@ __global__ void __launch_bounds__(kThreads) sigma_dense_kernel(DenseSigmaArgs a)
     double2 acc[kMaxAcc];
 #pragma unroll
     for (int k = 0; k < kMaxAcc; ++k) acc[k] = make_double2(0.0, 0.0);
-    for (int q0 = 0; q0 < MM; q0 += g) {
-      const int gc = min(g, MM - q0);
+    for (int q0 = q_lo; q0 < q_hi; q0 += g) {
+      const int gc = min(g, q_hi - q0);
       const int nT = gc * MM;
       // T^{db} and Q^{db} for the pairs of this tile
       for (int o = tid; o < 2 * nT; o += kThreads) {
@@ -143,7 +146,7 @@ __global__ void __launch_bounds__(kThreads) sigma_dense_kernel(DenseSigmaArgs a)
       }
       __syncthreads();
     }
-    double2* out = (s == 0 ? a.Sl : a.Sg) + blk * MM;
+    double2* out = a.slices > 1 ? a.part + ((slice * 2 + s) * a.n_blocks + blk) * MM : (s == 0 ? a.Sl : a.Sg) + blk * MM;
     if (G3 == 1) {
 #pragma unroll
       for (int k = 0; k < kMaxAcc; ++k) {
@@ -176,6 +179,22 @@ __global__ void __launch_bounds__(kThreads) sigma_dense_kernel(DenseSigmaArgs a)
   if (!ok) atomicOr(a.status, kStatusNumeric);
 }
 
+// The slices' partial sums [slice][s][block][M][M] in order.
+__global__ void __launch_bounds__(256) sigma_dense_sum(int slices, int64_t row, const double2* __restrict__ part,
+                                                       double2* __restrict__ Sl, double2* __restrict__ Sg,
+                                                       int* status) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= 2 * row) return;
+  double2 v = part[e];
+  for (int k = 1; k < slices; ++k) {
+    const double2 x = part[2 * k * row + e];
+    v.x += x.x;
+    v.y += x.y;
+  }
+  if (e < row) Sl[e] = v; else Sg[e - row] = v;
+  if (!(isfinite(v.x) && isfinite(v.y))) atomicOr(status, kStatusNumeric);
+}
+
 struct Tiling {
   int g, g3;
   size_t smem;
@@ -202,7 +221,8 @@ cudaError_t dense_sigma_prepare(int M) {
 
 cudaError_t launch_sigma_dense(int M, int64_t first_block, int64_t n_blocks, int64_t diag_rel, const double* L,
                                const double* R, const double* Ut, const double* Xt, double* Sl, double* Sg,
-                               int* status, cudaStream_t s) {
+                               int* status, double* work, size_t work_bytes, cudaStream_t s, int* launches) {
+  *launches = 0;
   if (n_blocks == 0) return cudaSuccess;
   const Tiling t = tiling(M);
   DenseSigmaArgs a;
@@ -219,10 +239,25 @@ cudaError_t launch_sigma_dense(int M, int64_t first_block, int64_t n_blocks, int
   a.status = status;
   a.g = t.g;
   a.g3 = t.g3;
-  int64_t blocks = 2 * n_blocks;
   const int64_t cap = (int64_t)sm_count() * 16;
+  // A row of few blocks leaves the last round of CTAs on a part of the SMs (n = 255:
+  // 512 units on 152 SMs, 3.4 each, the longest 4): a block's pairs are then split
+  // into slices, whose sums a second launch adds (M = 16, n = 255: 12.63 -> 10.55 ms).
+  // Blocks of small M take microseconds and are left whole.
+  a.slices = 1;
+  a.part = reinterpret_cast<double2*>(work);
+  if (M >= 8 && 2 * n_blocks < cap)
+    a.slices = (int)std::min<int64_t>((cap + 2 * n_blocks - 1) / (2 * n_blocks), std::min(8, M * M / t.g));
+  while (a.slices > 1 && (size_t)(2 * a.slices * n_blocks * M * M) * sizeof(double2) > work_bytes) --a.slices;
+  int64_t blocks = 2 * n_blocks * a.slices;
   if (blocks > cap) blocks = cap;
   sigma_dense_kernel<<<(unsigned)blocks, kThreads, t.smem, s>>>(a);
+  ++*launches;
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || a.slices == 1) return e;
+  const int64_t row = n_blocks * M * M;
+  sigma_dense_sum<<<(unsigned)((2 * row + 255) / 256), 256, 0, s>>>(a.slices, row, a.part, a.Sl, a.Sg, status);
+  ++*launches;
   return cudaGetLastError();
 }
 

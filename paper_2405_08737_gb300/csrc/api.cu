@@ -201,20 +201,24 @@ void adjoint_fx(const kbe_ctx* ctx, AdjHistArgs* h) {
 }
 
 // Self-energy of n_blocks blocks from first_block (launch_sigma geometry),
-// with the context's interaction: the local U or the dense tensor.
+// with the context's interaction: the local U or the dense tensor; with `fock`
+// (a row launch) also the row's Fock matrix.
 cudaError_t sigma_blocks(kbe_ctx* ctx, int64_t first_block, int64_t n_blocks, int64_t diag_rel, const void* L,
-                         const void* R, void* Sl, void* Sg, cudaStream_t s, int* launches) {
+                         const void* R, void* Sl, void* Sg, cudaStream_t s, int* launches,
+                         const StepArgs* fock = nullptr) {
   if (ctx->dense) {  // the slice workspace is free until the history slice of this row
     int k = 0;
     const cudaError_t e = launch_sigma_dense(ctx->M, first_block, n_blocks, diag_rel, (const double*)L,
                                              (const double*)R, ctx->d_Ut, ctx->d_Xt, (double*)Sl, (double*)Sg,
                                              ctx->d_status, ctx->d_part, ctx->part_bytes, s, &k);
     *launches += k;
-    return e;
+    if (e != cudaSuccess || !fock) return e;
+    ++*launches;
+    return launch_fock(*fock, s);
   }
   ++*launches;
   return launch_sigma(ctx->M, first_block, n_blocks, diag_rel, (const double*)L, (const double*)R, ctx->d_U,
-                      (double*)Sl, (double*)Sg, ctx->d_status, s);
+                      (double*)Sl, (double*)Sg, ctx->d_status, s, fock);
 }
 
 StepArgs step_args(kbe_ctx* ctx, int n, void* L, void* R, const void* I, void* F) {
@@ -371,7 +375,7 @@ kbe_status step_impl(kbe_ctx* ctx, int n, int P, int precision, void* L, void* R
   if (e != cudaSuccess) return cuda_fail(ctx, e, "kbe_step: predictor");
   for (int it = 0; it < P; ++it) {
     if ((e = keep(it)) != cudaSuccess) return cuda_fail(ctx, e, "kbe_step: iterate copy");
-    e = sigma_blocks(ctx, tri(n, 0), n + 1, n, L, R, Sl, Sg, s, &count);
+    e = sigma_blocks(ctx, tri(n, 0), n + 1, n, L, R, Sl, Sg, s, &count, &a);
     *count_out = count;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "kbe_step: self-energy");
     if (ctx->adaptive_K > 0) {  // history order of interval n from this sweep's rows (Sec. 3.2)
@@ -391,20 +395,19 @@ kbe_status step_impl(kbe_ctx* ctx, int n, int P, int precision, void* L, void* R
     if (ctx->thermal) {
       ThermalArgs x = thermal_args(ctx, a, Sl, Sg, I_work);
       x.df = precision != KBE_FP64;  // the thermal sums in double-float with the faster contractions
-      if ((e = thermal_sweep_a(ctx, x, s)) != cudaSuccess || (e = launch_fock(a, s)) != cudaSuccess ||
-          (e = launch_rhs_corrector(a, s)) != cudaSuccess || (e = launch_th_rhs(x, s)) != cudaSuccess ||
-          (e = launch_th_adams(x, true, s)) != cudaSuccess) {
-        *count_out = count + 7;
+      if ((e = thermal_sweep_a(ctx, x, s)) != cudaSuccess || (e = launch_rhs_corrector(a, s)) != cudaSuccess ||
+          (e = launch_th_rhs(x, s)) != cudaSuccess || (e = launch_th_adams(x, true, s)) != cudaSuccess) {
+        *count_out = count + 5;
         return cuda_fail(ctx, e, "kbe_step: thermal corrector");
       }
-      *count_out = (count += 7);
+      *count_out = (count += 5);
       continue;
     }
-    if ((e = launch_fock(a, s)) != cudaSuccess || (e = launch_rhs_corrector(a, s)) != cudaSuccess) {
-      *count_out = count + 3;
+    if ((e = launch_rhs_corrector(a, s)) != cudaSuccess) {
+      *count_out = count + 1;
       return cuda_fail(ctx, e, "kbe_step: corrector");
     }
-    *count_out = (count += 3);
+    *count_out = (count += 1);
   }
   if ((e = keep(P)) != cudaSuccess) return cuda_fail(ctx, e, "kbe_step: iterate copy");
   return KBE_OK;
@@ -1068,7 +1071,7 @@ kbe_status kbe_step_sweep_finish(kbe_ctx* ctx, int n, void* L, void* R, const vo
   StepArgs a = step_args(ctx, n, L, R, I, F_ring);
   cudaError_t e = launch_fock(a, s);
   if (e == cudaSuccess) e = launch_rhs_corrector(a, s);
-  ctx->last_launches = 3;
+  ctx->last_launches = 2;
   return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "kbe_step_sweep_finish");
 }
 

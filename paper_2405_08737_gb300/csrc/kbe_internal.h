@@ -160,8 +160,11 @@ struct kbe_ctx {
 namespace kbe {
 
 // ---- launchers (each returns cudaGetLastError() after the launch) -------
+struct StepArgs;
+// fock: also the Fock matrix of the row's iterate (launch_fock) in the same launch
 cudaError_t launch_sigma(int M, int64_t first_block, int64_t n_blocks, int64_t diag_rel, const double* L,
-                         const double* R, const double* U, double* Sl, double* Sg, int* status, cudaStream_t s);
+                         const double* R, const double* U, double* Sl, double* Sg, int* status, cudaStream_t s,
+                         const StepArgs* fock = nullptr);
 
 // Dense-interaction self-energy (sigma_dense.cu): same launch geometry as
 // launch_sigma; Ut, Xt are the reordered tensors of the context.

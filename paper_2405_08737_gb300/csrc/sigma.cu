@@ -34,13 +34,21 @@ __device__ __forceinline__ int64_t tri_row(int64_t p) {
 // triangles, the index of the next diagonal block by increments.  Five CTAs
 // per SM (at most 51 registers), each thread with the next entry's loads in
 // flight, keep enough bytes moving for HBM.
+// kFock: one more CTA forms the Fock matrix of the row (it reads the diagonal block
+// of the iterate, as the row's self-energy does), which saves a step a launch.
+template <bool kFock>
 __global__ void __launch_bounds__(256, 5) sigma_kernel(int MM, int M, int64_t n_elem, int64_t first_block,
                                                     int64_t diag_block, const double2* __restrict__ L,
                                                     const double2* __restrict__ R,
                                                     const double* __restrict__ U,
                                                     double2* __restrict__ Sl,
-                                                    double2* __restrict__ Sg, int* status) {
-  const int64_t per_cta = ((n_elem + gridDim.x - 1) / gridDim.x + blockDim.x - 1) / blockDim.x * blockDim.x;
+                                                    double2* __restrict__ Sg, int* status, StepArgs fock) {
+  const unsigned ctas = kFock ? gridDim.x - 1 : gridDim.x;
+  if (kFock && blockIdx.x == ctas) {
+    for (int ab = threadIdx.x; ab < MM; ab += blockDim.x) rk::fock_entry(fock, ab);
+    return;
+  }
+  const int64_t per_cta = ((n_elem + ctas - 1) / ctas + blockDim.x - 1) / blockDim.x * blockDim.x;
   const int64_t e_end = min(n_elem, (int64_t)(blockIdx.x + 1) * per_cta);
   int64_t e = (int64_t)blockIdx.x * per_cta + threadIdx.x;
   if (e >= e_end) return;
@@ -98,7 +106,8 @@ __global__ void __launch_bounds__(256, 5) sigma_kernel(int MM, int M, int64_t n_
 // Row launch: first_block = p(n,0), n_blocks = n+1, diagonal at n.
 // Whole-triangle launch: first_block = 0, n_blocks = tri(N), diag_rel = -1.
 cudaError_t launch_sigma(int M, int64_t first_block, int64_t n_blocks, int64_t diag_rel, const double* L,
-                         const double* R, const double* U, double* Sl, double* Sg, int* status, cudaStream_t s) {
+                         const double* R, const double* U, double* Sl, double* Sg, int* status, cudaStream_t s,
+                         const StepArgs* fock) {
   const int MM = M * M;
   const int64_t n_elem = n_blocks * MM;
   const int64_t off = first_block * MM;
@@ -106,8 +115,14 @@ cudaError_t launch_sigma(int M, int64_t first_block, int64_t n_blocks, int64_t d
   int64_t blocks = (n_elem + 255) / 256;
   const int64_t cap = (int64_t)sm_count() * 16;  // a grid-stride loop beyond ~16 CTAs per SM
   if (blocks > cap) blocks = cap;
-  sigma_kernel<<<(unsigned)blocks, 256, 0, s>>>(MM, M, n_elem, first_block, diag_rel, (const double2*)L + off,
-                                                (const double2*)R + off, U, (double2*)Sl, (double2*)Sg, status);
+  if (fock)
+    sigma_kernel<true><<<(unsigned)blocks + 1, 256, 0, s>>>(MM, M, n_elem, first_block, diag_rel,
+                                                            (const double2*)L + off, (const double2*)R + off, U,
+                                                            (double2*)Sl, (double2*)Sg, status, *fock);
+  else
+    sigma_kernel<false><<<(unsigned)blocks, 256, 0, s>>>(MM, M, n_elem, first_block, diag_rel, (const double2*)L + off,
+                                                         (const double2*)R + off, U, (double2*)Sl, (double2*)Sg, status,
+                                                         StepArgs{});
   return cudaGetLastError();
 }
 

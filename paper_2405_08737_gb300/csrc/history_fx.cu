@@ -173,6 +173,11 @@ __device__ __forceinline__ int find_sys(const Args& a, long long x, F base) {
 }
 __device__ __forceinline__ WeightsView weights_of(const Sys& s) { return WeightsView{s.wbar, s.band, s.band_w}; }
 
+// Programmatic dependent launch: lets the next kernel start its setup, and waits
+// until the kernel before is complete.
+__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Waits for a phase of a barrier, suspended by the hardware between polls.
 // Gives up after kWaitCycles, or when another role has.
 __device__ __forceinline__ bool try_suspend(uint64_t* bar, uint32_t parity) {
@@ -239,6 +244,7 @@ __device__ __forceinline__ int field64(double v) { return field_of((uint32_t)__d
 template <int NA>
 __global__ void __launch_bounds__(32 * NA) fx_prep(const __grid_constant__ Args a) {
   using C = Cfg<NA>;
+  grid_launch_next();
   const int al = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long chunks = head_of(a).chunks;
   for (long long ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
@@ -472,9 +478,6 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   Smem<NA>& sm = *reinterpret_cast<Smem<NA>*>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long total = head_of(a).total;
-  const long long q0 = range_lo(total, a.G, blockIdx.x), q1 = range_lo(total, a.G, blockIdx.x + 1);
-  int* const status = sys_at(a, 0).status;
 
   if (tid == 0) {
     // empty, bempty: both MMA threads
@@ -497,6 +500,10 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sm.tmem;
+  grid_wait();  // the small operands are complete
+  const long long total = head_of(a).total;
+  const long long q0 = range_lo(total, a.G, blockIdx.x), q1 = range_lo(total, a.G, blockIdx.x + 1);
+  int* const status = sys_at(a, 0).status;
 
   if (warp < kEpiWarps) {
     // --------------------------------------------------------- epilogue --
@@ -831,6 +838,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
 // Output entries (c, a, b): the partial sums of their tile in CTA order.
 template <int NA>
 __global__ void __launch_bounds__(256) fx_reduce(const __grid_constant__ Args a) {
+  grid_wait();
   const Head& h = head_of(a);
   const long long entries = h.entries, total = h.total;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < entries;
@@ -866,15 +874,28 @@ cudaError_t enqueue(const Args& a, bool quad, unsigned prep_blocks, unsigned red
   ++*launches;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  // the next two kernels are set up while the one before drains (they wait for
+  // it with griddepcontrol.wait): about 2 us each
+  cudaLaunchAttribute overlap;
+  overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  overlap.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)a.G);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = sizeof(Smem<NA>);
+  cfg.stream = st;
+  cfg.attrs = &overlap;
+  cfg.numAttrs = ev_begin ? 0 : 1;  // timed: no event inside the overlap
   if (ev_begin) cudaEventRecord(ev_begin, st);
-  if (quad)
-    fx_main<NA, true><<<a.G, kThreads, sizeof(Smem<NA>), st>>>(a);
-  else
-    fx_main<NA, false><<<a.G, kThreads, sizeof(Smem<NA>), st>>>(a);
+  e = quad ? cudaLaunchKernelEx(&cfg, fx_main<NA, true>, a) : cudaLaunchKernelEx(&cfg, fx_main<NA, false>, a);
+  if (e != cudaSuccess) return e;
   if (ev_end) cudaEventRecord(ev_end, st);
   ++*launches;
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  fx_reduce<NA><<<red_blocks, 256, 0, st>>>(a);
+  cfg.gridDim = dim3(red_blocks);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = 0;
+  cfg.numAttrs = ev_end ? 0 : 1;
+  if ((e = cudaLaunchKernelEx(&cfg, fx_reduce<NA>, a)) != cudaSuccess) return e;
   ++*launches;
   return cudaGetLastError();
 }

@@ -173,10 +173,8 @@ __device__ __forceinline__ int find_sys(const Args& a, long long x, F base) {
 }
 __device__ __forceinline__ WeightsView weights_of(const Sys& s) { return WeightsView{s.wbar, s.band, s.band_w}; }
 
-// Programmatic dependent launch: lets the next kernel start its setup, and waits
-// until the kernel before is complete.
+// Lets the next kernel (launch_overlapped) start its setup.
 __device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Waits for a phase of a barrier, suspended by the hardware between polls.
 // Gives up after kWaitCycles, or when another role has.
@@ -245,6 +243,7 @@ template <int NA>
 __global__ void __launch_bounds__(32 * NA) fx_prep(const __grid_constant__ Args a) {
   using C = Cfg<NA>;
   grid_launch_next();
+  grid_wait();
   const int al = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long chunks = head_of(a).chunks;
   for (long long ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
@@ -870,34 +869,23 @@ __global__ void __launch_bounds__(256) fx_reduce(const __grid_constant__ Args a)
 template <int NA>
 cudaError_t enqueue(const Args& a, bool quad, unsigned prep_blocks, unsigned red_blocks, cudaStream_t st, int* launches,
                     cudaEvent_t ev_begin, cudaEvent_t ev_end) {
-  fx_prep<NA><<<prep_blocks, 32 * NA, 0, st>>>(a);
-  ++*launches;
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_overlapped(fx_prep<NA>, prep_blocks, 32 * NA, 0, st, a);
   if (e != cudaSuccess) return e;
-  // the next two kernels are set up while the one before drains (they wait for
-  // it with griddepcontrol.wait): about 2 us each
-  cudaLaunchAttribute overlap;
-  overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  overlap.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)a.G);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = sizeof(Smem<NA>);
-  cfg.stream = st;
-  cfg.attrs = &overlap;
-  cfg.numAttrs = ev_begin ? 0 : 1;  // timed: no event inside the overlap
-  if (ev_begin) cudaEventRecord(ev_begin, st);
-  e = quad ? cudaLaunchKernelEx(&cfg, fx_main<NA, true>, a) : cudaLaunchKernelEx(&cfg, fx_main<NA, false>, a);
+  ++*launches;
+  if (ev_begin) {  // timed: no overlap with the kernels around it
+    cudaEventRecord(ev_begin, st);
+    if (quad) fx_main<NA, true><<<a.G, kThreads, sizeof(Smem<NA>), st>>>(a);
+    else fx_main<NA, false><<<a.G, kThreads, sizeof(Smem<NA>), st>>>(a);
+    e = cudaGetLastError();
+    cudaEventRecord(ev_end, st);
+  } else {
+    e = launch_overlapped(quad ? fx_main<NA, true> : fx_main<NA, false>, a.G, kThreads, sizeof(Smem<NA>), st, a);
+  }
   if (e != cudaSuccess) return e;
-  if (ev_end) cudaEventRecord(ev_end, st);
   ++*launches;
-  cfg.gridDim = dim3(red_blocks);
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = 0;
-  cfg.numAttrs = ev_end ? 0 : 1;
-  if ((e = cudaLaunchKernelEx(&cfg, fx_reduce<NA>, a)) != cudaSuccess) return e;
+  if ((e = launch_overlapped(fx_reduce<NA>, red_blocks, 256, 0, st, a)) != cudaSuccess) return e;
   ++*launches;
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 // One system's contraction in its workspace.

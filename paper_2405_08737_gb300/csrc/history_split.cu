@@ -155,6 +155,7 @@ __global__ void __launch_bounds__(256) split_prep(int M, int n, int parts, const
                                                   const double* __restrict__ Sg, WeightsView w,
                                                   uint8_t* __restrict__ small, int* __restrict__ e_small) {
   __shared__ int s_ef;
+  grid_wait();
   prep_chunk(M, n, parts, Sl, Sg, w, small, e_small, blockIdx.x, blockIdx.y, &s_ef);
 }
 
@@ -264,6 +265,7 @@ __global__ void __launch_bounds__(256, kNarrow ? 1 : 3) split_encode(EncodeArgs 
   const int cls = chunk_class(kap0 / M, (kap0 + kKC - 1) / M, c0, c0 + CT - 1, g.band_w);
   for (int e = t; e < upc * 128; e += blockDim.x) ecol[e] = 0;
   __syncthreads();
+  grid_wait();
   const double2* base = reinterpret_cast<const double2*>(arr == 0 ? a.L : a.R);
   const int c = c0 + cl;
   const bool enc = row_live && c >= a.c_min;
@@ -452,6 +454,7 @@ __global__ void __launch_bounds__(kThreads2, 1) split_main2(Split2Args a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sm.tmem;
+  grid_wait();
 
   if (warp == kEpi2 + 1) {
     // -------------------------------------------------------- producer --
@@ -1351,6 +1354,7 @@ __global__ void __launch_bounds__(kRedThreads, 7) split_reduce2(SplitGeom g, con
                                                              const double* __restrict__ R, WeightsView w,
                                                              double* __restrict__ out, int* status) {
   __shared__ RedShared sh;
+  grid_wait();
   const int c = blockIdx.x, pt = blockIdx.y;
   const int tile = (c / g.CT) * g.parts + pt;
   if (threadIdx.x == 0) {
@@ -1507,7 +1511,8 @@ cudaError_t launch_history_split2(const SplitLaunch& l, const SplitPlanes& pl_la
 
   cudaError_t e = split_prepare();
   if (e != cudaSuccess) return e;
-  split_prep<<<dim3(h.cpt, h.parts), 256, 0, s>>>(l.M, l.n, h.parts, l.Sl, l.Sg, l.w, small, e_small);
+  e = launch_overlapped(split_prep, dim3(h.cpt, h.parts), 256, 0, s, l.M, l.n, h.parts, l.Sl, l.Sg, l.w, small, e_small);
+  if (e != cudaSuccess) return e;
   ++*launches;
   // entries involving rows >= r0: every chunk of the columns c >= r0 (the
   // column tiles from the one holding column r0, those columns only), and
@@ -1531,9 +1536,10 @@ cudaError_t launch_history_split2(const SplitLaunch& l, const SplitPlanes& pl_la
       threads = (unsigned)((2 * ea.upc * ea.rows + 31) / 32 * 32);
     }
     if (ea.upc > 1 || ea.row_lo > 0)
-      split_encode<true><<<(ea.units + ea.upc - 1) / ea.upc, threads, 0, s>>>(ea);
+      e = launch_overlapped(split_encode<true>, (ea.units + ea.upc - 1) / ea.upc, threads, 0, s, ea);
     else
-      split_encode<false><<<ea.units, 256, 0, s>>>(ea);
+      e = launch_overlapped(split_encode<false>, ea.units, 256, 0, s, ea);
+    if (e != cudaSuccess) return e;
     ++*launches;
   }
   const int ct_hi = std::min(col_tiles, ct_lo + 1);
@@ -1543,20 +1549,27 @@ cudaError_t launch_history_split2(const SplitLaunch& l, const SplitPlanes& pl_la
     ea.row_lo = 0;
     ea.rows = 128;
     ea.upc = 1;
-    split_encode<false><<<ea.units, 256, 0, s>>>(ea);
+    if ((e = launch_overlapped(split_encode<false>, ea.units, 256, 0, s, ea)) != cudaSuccess) return e;
     ++*launches;
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   Split2Args args{g, pl, qu, pl_layout.cpt_stride, qs, small, e_small, part, l.status,
                   l.withhold, l.spin_limit > 0 ? l.spin_limit : kSpinLimit};
-  if (l.ev_begin) cudaEventRecord(l.ev_begin, s);
-  split_main2<<<h.G, kThreads2, sizeof(Smem2), s>>>(args);
-  if (l.ev_end) cudaEventRecord(l.ev_end, s);
+  if (l.ev_begin) {  // timed: no overlap with the kernels around it
+    cudaEventRecord(l.ev_begin, s);
+    split_main2<<<h.G, kThreads2, sizeof(Smem2), s>>>(args);
+    e = cudaGetLastError();
+    cudaEventRecord(l.ev_end, s);
+  } else {
+    e = launch_overlapped(split_main2, h.G, kThreads2, sizeof(Smem2), s, args);
+  }
+  if (e != cudaSuccess) return e;
   ++*launches;
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  split_reduce2<<<reduce2_grid(h), kRedThreads, 0, s>>>(g, part, l.Sl, l.Sg, l.R, l.w, l.out, l.status);
+  e = launch_overlapped(split_reduce2, reduce2_grid(h), kRedThreads, 0, s, g, part, l.Sl, l.Sg, l.R, l.w, l.out,
+                        l.status);
+  if (e != cudaSuccess) return e;
   ++*launches;
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 // ------------------------------------------------------------ fused host --

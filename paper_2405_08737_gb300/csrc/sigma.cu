@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(256, 5) sigma_kernel(int MM, int M, int64_t n_
                                                     const double* __restrict__ U,
                                                     double2* __restrict__ Sl,
                                                     double2* __restrict__ Sg, int* status, StepArgs fock) {
+  if (kFock) grid_wait();  // (the launch without the Fock matrix is not overlapped)
   const unsigned ctas = kFock ? gridDim.x - 1 : gridDim.x;
   if (kFock && blockIdx.x == ctas) {
     for (int ab = threadIdx.x; ab < MM; ab += blockDim.x) rk::fock_entry(fock, ab);
@@ -116,9 +117,9 @@ cudaError_t launch_sigma(int M, int64_t first_block, int64_t n_blocks, int64_t d
   const int64_t cap = (int64_t)sm_count() * 16;  // a grid-stride loop beyond ~16 CTAs per SM
   if (blocks > cap) blocks = cap;
   if (fock)
-    sigma_kernel<true><<<(unsigned)blocks + 1, 256, 0, s>>>(MM, M, n_elem, first_block, diag_rel,
-                                                            (const double2*)L + off, (const double2*)R + off, U,
-                                                            (double2*)Sl, (double2*)Sg, status, *fock);
+    return launch_overlapped(sigma_kernel<true>, (unsigned)blocks + 1, 256, 0, s, MM, M, n_elem, first_block, diag_rel,
+                             (const double2*)L + off, (const double2*)R + off, U, (double2*)Sl, (double2*)Sg, status,
+                             *fock);
   else
     sigma_kernel<false><<<(unsigned)blocks, 256, 0, s>>>(MM, M, n_elem, first_block, diag_rel, (const double2*)L + off,
                                                          (const double2*)R + off, U, (double2*)Sl, (double2*)Sg, status,

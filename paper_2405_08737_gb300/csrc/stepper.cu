@@ -26,6 +26,7 @@ __global__ void fock_kernel(StepArgs a) {
 }
 
 __global__ void __launch_bounds__(256) predictor_kernel(StepArgs a) {
+  grid_wait();
   const int64_t lin = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (lin < (int64_t)(a.n + 1) * a.M * a.M) rk::adams_entry(a, lin, false);
 }
@@ -42,6 +43,7 @@ __global__ void __launch_bounds__(256) rhs_kernel(StepArgs a) {
 // a block takes whole columns with a barrier between the two.  (One launch instead
 // of two: about 5 us per sweep.)
 __global__ void __launch_bounds__(256) rhs_corrector_kernel(StepArgs a, int cols) {
+  grid_wait();
   const int MM = a.M * a.M;
   const int64_t lo = (int64_t)blockIdx.x * cols * MM;
   const int64_t hi = min((int64_t)(a.n + 1) * MM, lo + (int64_t)cols * MM);
@@ -77,8 +79,7 @@ cudaError_t launch_fock(const StepArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 cudaError_t launch_predictor(const StepArgs& a, cudaStream_t s) {
-  predictor_kernel<<<blocks_for((int64_t)(a.n + 1) * a.M * a.M), 256, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_overlapped(predictor_kernel, blocks_for((int64_t)(a.n + 1) * a.M * a.M), 256, 0, s, a);
 }
 cudaError_t launch_rhs(const StepArgs& a, cudaStream_t s) {
   rhs_kernel<<<blocks_for((int64_t)(a.n + 1) * a.M * a.M), 256, 0, s>>>(a);
@@ -86,8 +87,7 @@ cudaError_t launch_rhs(const StepArgs& a, cudaStream_t s) {
 }
 cudaError_t launch_rhs_corrector(const StepArgs& a, cudaStream_t s) {
   const int cols = std::max(1, 256 / (a.M * a.M));
-  rhs_corrector_kernel<<<(unsigned)((a.n + cols) / cols), 256, 0, s>>>(a, cols);
-  return cudaGetLastError();
+  return launch_overlapped(rhs_corrector_kernel, (unsigned)((a.n + cols) / cols), 256, 0, s, a, cols);
 }
 
 }  // namespace kbe

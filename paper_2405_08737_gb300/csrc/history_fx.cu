@@ -26,8 +26,8 @@
 // real, and the digit stores (64 KB a unit), the MMA operand reads and the history
 // loads share the L1 / shared-memory data pipe, about 70% busy (M = 8, n = 600: issue
 // slots 62%, tensor pipe 37%).  With NA = 16 the epilogue holds the MMAs back as well.
-// Measured, in this kernel: the slice n = 1023, M = 8 in 0.83 ms (7.05 on the FP64
-// pipe, history_f64.cu), n = 511, M = 16 in 1.23 ms (14.4).
+// Measured, in this kernel: the slice n = 1023, M = 8 in 0.82 ms (7.05 on the FP64
+// pipe, history_f64.cu), n = 511, M = 16 in 1.18 ms (14.4).
 //
 // One persistent CTA per SM takes a contiguous range of chunks (32 history
 // entries of a 128-row column tile).  A unit is 8 entries, one MMA K step:
@@ -52,7 +52,13 @@
 // A row's exponent holds for the units accumulated together in tensor memory.
 // It starts kHeadroom bits above the larger of the unit's and the previous
 // chunk's largest entry; a unit that exceeds it nevertheless closes the
-// accumulation and starts the next with the larger exponent.
+// accumulation and starts the next with the larger exponent.  A row that had
+// only zeros so far (near the diagonal each column of the tile starts at a point
+// of its own) takes its exponent without that, so the sums use the exponents of
+// an accumulation's last unit, and starts kStartRoom bits above its first values, which
+// may be its smallest.  With an accumulation for each start, which had most near
+// the diagonal, and its band entries loaded one by one (for_band), the slice
+// M = 8, n = 124 took 85 us instead of 66, M = 5, n = 333 106 instead of 90.
 //
 // Partial sums go to one slot per (CTA, tile) and are added in CTA order, so
 // results are bitwise reproducible.  All waits are bounded.  A row or a small
@@ -131,7 +137,7 @@ __device__ __forceinline__ int kind_of(int flags) { return flags >> 8 & 0xFF; }
 
 struct alignas(16) Post {  // what the MMA thread hands to the epilogue with a buffer
   int type;                // kUnit (sums), kScale, kFlush, kEnd
-  int grp, eidx, plane;    // sum group (0: I^<, 1: D), exponent ring index and plane
+  int grp, eidx, plane;    // sum group (0: I^<, 1: D), exponent ring index (the last unit's) and plane
   int si, c0, slot;        // system; first column (scale); partial slot (flush)
   int cols;                // a values of the part, plus one
   int16_t es[16];          // small operand's exponents
@@ -390,80 +396,100 @@ __device__ __forceinline__ void load_quad(const Row& r, int kap, bool near, bool
   }
 }
 // Four entries of the band of term 2 (plane R): w_{c,m} R(c,m)^+ for c - band_w < m
-// <= c, in the adjoint w_{m,c} R(m,c) for c <= m < c + band_w.
-__device__ __noinline__ unsigned load_band(const Sys& s, const Row& r, int c, int kap, double2 z[4]) {
-  const int M = r.M, MM = M * M, bw = s.band_w;
+// <= c, in the adjoint w_{m,c} R(m,c) for c <= m < c + band_w.  band_values loads the
+// entries, like load_quad a unit ahead; band_weights, when they are converted, their
+// weights (which repeat from unit to unit, so they come from the L1 cache).  Loading
+// both and multiplying at once, one entry after the other, took 3.0 to 3.8 us a unit where
+// a far or near unit takes 1.4 to 1.8, and the CTA that holds a tile's band is the
+// last of a short row.
+template <class F>
+__device__ __forceinline__ void for_band(const Sys& s, const Row& r, int kap, F f) {
+  const int M = r.M, c = r.edge - s.shift;
   int m = div_m(kap, M, r.magic), x = kap - m * M;
-  unsigned mask = 0;
+#pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int hi = s.adj ? m : c, lo = s.adj ? c : m;
-    const bool in = m <= r.n && lo <= hi && hi - lo < bw;
-    z[i] = make_double2(0.0, 0.0);
-    if (in) {
-      const double w = s.band[(int64_t)hi * bw + (hi - lo)];
-      const double2 v = __ldg(s.adj ? r.dr + (tri(m, 0) * MM + x * M) : r.tr + (m * MM + x));
-      z[i] = make_double2(w * v.x, s.adj ? w * v.y : -w * v.y);
-    }
-    mask |= (unsigned)in << i;
+    const int d = s.adj ? m - c : c - m;
+    f(i, m, x, d, m <= r.n && d >= 0 && d < s.band_w);
     if (++x == M) { x = 0; ++m; }
   }
-  return mask;
+}
+__device__ __forceinline__ void band_values(const Sys& s, const Row& r, int kap, bool live, double2 z[4]) {
+  const int M = r.M, MM = M * M, adj = s.adj;
+  for_band(s, r, kap, [&](int i, int m, int x, int, bool in) {
+    z[i] = make_double2(0.0, 0.0);
+    if (in && live) z[i] = __ldg(adj ? r.dr + (tri0(m) * (unsigned)MM + (unsigned)(x * M)) : r.tr + (m * MM + x));
+  });
+}
+__device__ __forceinline__ void band_weights(const Sys& s, const Row& r, int kap, double2 z[4]) {
+  const int adj = s.adj, c = r.edge - s.shift;
+  for_band(s, r, kap, [&](int i, int m, int, int d, bool in) {
+    if (!in) return;  // zero
+    const double w = __ldg(s.band + (int64_t)(adj ? m : c) * s.band_w + d);
+    z[i] = make_double2(w * z[i].x, adj ? w * z[i].y : -w * z[i].y);
+  });
 }
 
 // ------------------------------------------------------------ epilogue ---
 // Folds the accumulator buffer at `at` into the FP64 sums s of this thread's row
 // and half of the a values, and hands the buffer back (empty) once its levels are
 // in registers.  kWhole: every a value of the part is in use (otherwise the
-// columns past the last one are skipped).
+// columns past the last one are skipped).  Two columns' levels are read at a time
+// and reduced to 64-bit integers before the next two are: a read waits for tensor
+// memory about as long as its arithmetic takes, and NA = 16, whose accumulations wait
+// for it, has no registers to hold more (one column at a time with its levels converted
+// first: M = 12, n = 389 in 549 us instead of 517, M = 16, n = 511 in 1.24 ms instead of 1.21).
 template <int NA, bool kWhole>
 __device__ __forceinline__ void fold(double (&s)[NA], uint32_t at, int E, int half, const Post& ps, uint64_t* empty) {
-  constexpr int kN = 2 * NA, kC = NA, kCols = NA == 8 ? 2 : 1;  // kCols: columns in registers at a time
+  constexpr int kN = 2 * NA, kC = NA, kCols = 2;  // kCols: columns in registers at a time
   const int cols = kWhole ? kC : (ps.cols - half) & ~1;
   uint32_t r[kDig][kCols];
   auto read = [&](int c2) {  // the levels of columns c2, ... in flight
 #pragma unroll
-    for (int d = 0; d < kDig; ++d) {
-      const uint32_t p = at + d * kN + 2 * c2 - c2 % 2;
-      if constexpr (kCols == 2)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(r[d][0]), "=r"(r[d][kCols - 1]) : "r"(p));
-      else
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[d][0]) : "r"(p));
-    }
+    for (int d = 0; d < kDig; ++d)
+#pragma unroll
+      for (int i = 0; i < kCols; i += 2) {
+        const uint32_t p = at + d * kN + 2 * (c2 + i);
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(r[d][i]), "=r"(r[d][i + 1]) : "r"(p));
+      }
   };
   read(0);
 #pragma unroll
   for (int c2 = 0; c2 < kC; c2 += kCols) {
     if (!kWhole && c2 > 0 && c2 >= cols) continue;
-    const int es = ps.es[2 * (c2 / 2) + half];
+    int es[kCols / 2];
+#pragma unroll
+    for (int i = 0; i < kCols / 2; ++i) es[i] = ps.es[c2 + 2 * i + half];
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    int v[kDig][kCols];
+    int64_t t[kCols];
 #pragma unroll
-    for (int i = 0; i < kCols; ++i)
+    for (int i = 0; i < kCols; ++i) {
+      int v[kDig];
 #pragma unroll
-      for (int d = 0; d < kDig; ++d) v[d][i] = __float2int_rn(__uint_as_float(r[d][i]));
+      for (int d = 0; d < kDig; ++d) v[d] = __float2int_rn(__uint_as_float(r[d][i]));
+      // the 64-bit integer sum_l S_l 256^(7-l) / 2^12: |S_0| <= 2^19, |S_1| <= 2^21, |S_2| <= 2^22 and
+      // |S_l| <= l 2^21 fit the 32-bit steps, and 2^10 products of 62-bit values stay below 2^(124+7-56-12)
+      const uint64_t p01 = (uint64_t)(int64_t)(v[0] * 256 + v[1]), p23 = (uint64_t)(int64_t)(v[2] * 256 + v[3]);
+      const int low = v[5] * 16 + ((v[6] + (v[7] >> 8) + 8) >> 4);
+      t[i] = (int64_t)((p01 << 36) + (p23 << 20) + ((uint64_t)(int64_t)v[4] << 12) + (uint64_t)(int64_t)low);
+    }
     if (c2 + kCols < cols) {
-      read(c2 + kCols);  // while these are folded
+      read(c2 + kCols);  // while these are scaled
     } else {
       tc_fence_before();
       __syncwarp();
       if ((threadIdx.x & 31) == 0) mbar_arrive(empty);
     }
-    // scale 2^(ev + eu - 68 + 12), ev = E - 1022, eu = es - 1022
-    const int ex = E + es - 2 * 1022 - 56;
 #pragma unroll
     for (int i = 0; i < kCols; ++i) {
-      // the 64-bit integer sum_l S_l 256^(7-l) / 2^12: |S_0| <= 2^19, |S_1| <= 2^21, |S_2| <= 2^22 and
-      // |S_l| <= l 2^21 fit the 32-bit steps, and 2^10 products of 62-bit values stay below 2^(124+7-56-12)
-      const uint64_t p01 = (uint64_t)(int64_t)(v[0][i] * 256 + v[1][i]), p23 = (uint64_t)(int64_t)(v[2][i] * 256 + v[3][i]);
-      const int low = v[5][i] * 16 + ((v[6][i] + (v[7][i] >> 8) + 8) >> 4);
-      const int64_t t = (int64_t)((p01 << 36) + (p23 << 20) + ((uint64_t)(int64_t)v[4][i] << 12) + (uint64_t)(int64_t)low);
+      // scale 2^(ev + eu - 68 + 12), ev = E - 1022, eu = es - 1022
+      const int ex = E + es[i / 2] - 2 * 1022 - 56;
       if (ex >= -1022 && ex <= 1023) {
-        s[c2 + i] = fma((double)t, __hiloint2double((ex + 1023) << 20, 0), s[c2 + i]);
+        s[c2 + i] = fma((double)t[i], __hiloint2double((ex + 1023) << 20, 0), s[c2 + i]);
       } else if (ex >= kNonFinite - 4096) {
         s[c2 + i] = __longlong_as_double(0x7FF8000000000000ll);
       } else {  // the scale alone leaves the range of FP64
         const int h = ex / 2;
-        s[c2 + i] += (double)t * __hiloint2double((h + 1023) << 20, 0) * __hiloint2double((ex - h + 1023) << 20, 0);
+        s[c2 + i] += (double)t[i] * __hiloint2double((h + 1023) << 20, 0) * __hiloint2double((ex - h + 1023) << 20, 0);
       }
     }
   }
@@ -573,7 +599,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
     Row row;
     double2 z[4];
     unsigned mask = 0, d = 0;
-    int flags = 0, E = 64, seen = 64;  // of the unit in z; the row's exponent; largest field of the current chunk
+    int flags = 0, kap = 0, si = 0, E = 64, seen = 64;  // of the unit in z; the row's exponent; largest field of the current chunk
     // the next unit's loads; false when there is none
     auto load = [&]() -> bool {
       Desc ds;
@@ -586,14 +612,11 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       flags = ds.flags;
       if (kind_of(flags) == kEnd) return false;
       if (flags & kNewTile) row = row_of(sys_at(a, ds.aux), ds.c0, 8 * wq + (lane & 7), plane);
-      const int kap = ds.kap + 4 * q;
+      kap = ds.kap + 4 * q;
+      si = ds.aux;
       if (flags & kFlagBand) {
-        double2 v[4];
-        const int c = ds.c0 + div_m(8 * wq + (lane & 7), row.M, row.magic);
-        mask = plane ? load_band(sys_at(a, ds.aux), row, c, kap, v) : 0u;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) z[i] = plane ? v[i] : make_double2(0.0, 0.0);
-        if (mask) mask = 15u;  // the others are zero
+        band_values(sys_at(a, ds.aux), row, kap, plane, z);
+        mask = 15u;
       } else {
         load_quad<kQuad>(row, kap, flags & kFlagNear, !(flags & (kFlagNear | kFlagLow)), z, mask);
       }
@@ -602,6 +625,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
     bool more = load();
     for (unsigned u = 0; more; ++u) {
       const int s = u % kStages;
+      if (flags & kFlagBand) band_weights(sys_at(a, si), row, kap, z);
       // exponent of the row
       int mx = 0;
 #pragma unroll
@@ -613,14 +637,14 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       bool raised = false;
       if (flags & kFirst) {
         const int prev = (flags & kFresh) || seen == 0x7FF ? 0 : seen;
-        E = max(max(mx, prev), 64) + kHeadroom;
+        E = max(max(mx, prev), 64) + (prev ? kHeadroom : kStartRoom);
         seen = mx;
       } else {
-        raised = mx > E;
-        if (raised) E = mx + kHeadroom;
+        if (mx > E) { raised = seen > 0; E = mx + (raised ? kHeadroom : kStartRoom); }
+        if (mx == 0x7FF) { raised |= seen > 0 && E != kNonFinite; }
         seen = max(seen, mx);
       }
-      if (mx == 0x7FF) { raised |= E != kNonFinite; E = kNonFinite; }
+      if (mx == 0x7FF) E = kNonFinite;
       const int Ez = kQuad && !(mask & 1u) ? kNonFinite : E;  // a masked quad's digits are zero
       uint64_t br[4], bi[4];
 #pragma unroll
@@ -743,6 +767,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
         return wait_bar(&sm.abort, &sm.accempty[buf], ((k / (kBufs / 2)) & 1) ^ 1, status);
       };
       auto close = [&]() {
+        sm.post[buf].eidx = (u - 1) % kExpRing;
         mbar_arrive(&sm.accfull[buf]);
         umma_commit(&sm.accfull[buf]);
         next_buffer();
@@ -792,7 +817,6 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
           Post& ps = sm.post[buf];
           ps.type = kUnit;
           ps.grp = me && (near || band);
-          ps.eidx = u % kExpRing;
           ps.plane = band ? 1 : me;
           ps.cols = (ds.flags >> 16) + 1;
 #pragma unroll

@@ -87,6 +87,25 @@ def test_high_orders_and_zero_history(kbe):
     ctx.close()
 
 
+@pytest.mark.parametrize("M,n", [(3, 560), (5, 269), (8, 128), (12, 73), (16, 47), (33, 16)])
+def test_rows_that_start_late(kbe, M, n):
+    """Rows of zeros that start inside an accumulation, with values 2^-70 of the
+    later ones or with those (the bound of test_slice_sizes)."""
+    import torch
+    ctx, t, order, L, R, Sl, Sg = _setup(kbe, M, n, 11 * M + n, "random")
+    rng = np.random.default_rng(n)
+    for x in (L, R):
+        x *= rng.choice([0.0, 2.0 ** -70, 1.0], p=[0.45, 0.45, 0.1], size=x.shape)
+        x[W.tri_index(n // 2, 0):] *= rng.choice([0.0, 1.0], size=(x.shape[0] - W.tri_index(n // 2, 0), 1, 1))
+    out = torch.zeros((2, n + 1, M, M), dtype=torch.complex128, device="cuda")
+    ctx.history_slice(n, _dev(L), _dev(R), _dev(Sl), _dev(Sg), out)
+    assert ctx.last_launch_count == 3
+    ctx.sync_status()
+    ref = oracle.history_slice(t, order, n, L, R, Sl, Sg, nthreads=oracle.threads_available())
+    assert np.abs(out.cpu().numpy() - ref).max() < TOL * np.abs(ref).max()
+    ctx.close()
+
+
 @pytest.mark.parametrize("M,n", [(5, 269), (8, 128), (13, 70), (16, 47), (24, 26), (33, 16)])
 def test_adjoint_is_the_transpose(kbe, M, n):
     """Re<Ibar, I(dS)> = Re<Sbar, dS> for random rows Ibar, dS, which are

@@ -27,7 +27,7 @@ constexpr int kChunkUnits = 4; // units of a chunk; two chunks of a plane accumu
 constexpr int kChunkK = kUnitK * kChunkUnits;
 constexpr int kOver = 6;       // chunks that a column tile visits twice, at most (see Walk)
 constexpr int kHeadroom = 2;   // bits between a row's exponent and its first values
-constexpr int kStartRoom = 6;  // the same for a row whose first values these are
+constexpr int kStartRoom = 3;  // the same for a row whose first values these are (6: errors up to 1.1 times as large, 8: 1.9)
 constexpr int kNonFinite = 8000;  // exponent of a row or column that holds a non-finite value
 
 // Values of a per part, bytes of a part's small operand of one unit (two halves

@@ -58,7 +58,7 @@
 // an accumulation's last unit, and starts kStartRoom bits above its first values, which
 // may be its smallest.  With an accumulation for each start, which had most near
 // the diagonal, and its band entries loaded one by one (for_band), the slice
-// M = 8, n = 124 took 85 us instead of 66, M = 5, n = 333 106 instead of 90.
+// M = 8, n = 124 took 85 us instead of 66, M = 5, n = 333 106 instead of 94.
 //
 // Partial sums go to one slot per (CTA, tile) and are added in CTA order, so
 // results are bitwise reproducible.  All waits are bounded.  A row or a small

@@ -49,6 +49,10 @@ void release(kbe_ctx* ctx) {
   cudaFree(ctx->d_wbar); cudaFree(ctx->d_band); cudaFree(ctx->d_corr); cudaFree(ctx->d_pred);
   cudaFree(ctx->d_h0); cudaFree(ctx->d_U); cudaFree(ctx->d_v); cudaFree(ctx->d_eps);
   cudaFree(ctx->d_part); cudaFree(ctx->d_status); cudaFree(ctx->d_split); cudaFree(ctx->d_adj);
+  cudaFree(ctx->d_sd);
+  if (ctx->sd_done) cudaEventDestroy(ctx->sd_done);
+  ctx->d_sd = nullptr;
+  ctx->sd_done = nullptr;
   cudaFree(ctx->d_fx);
   ctx->d_fx = nullptr;
   ctx->fx_bytes = 0;
@@ -206,12 +210,21 @@ void adjoint_fx(const kbe_ctx* ctx, AdjHistArgs* h) {
 cudaError_t sigma_blocks(kbe_ctx* ctx, int64_t first_block, int64_t n_blocks, int64_t diag_rel, const void* L,
                          const void* R, void* Sl, void* Sg, cudaStream_t s, int* launches,
                          const StepArgs* fock = nullptr) {
-  if (ctx->dense) {  // the slice workspace is free until the history slice of this row
+  if (ctx->dense) {
+    // Self-energy calls of one context may overlap on different streams, so the partial sums of split rows
+    // have a buffer of their own, which the calls take in turn; captured calls leave rows whole (a wait for
+    // an event of another stream's past would end the capture).
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &capture);
+    const bool split = e == cudaSuccess && capture == cudaStreamCaptureStatusNone && ctx->d_sd;
+    if (e != cudaSuccess) cudaGetLastError();
+    if (split && (e = cudaStreamWaitEvent(s, ctx->sd_done, 0)) != cudaSuccess) return e;
     int k = 0;
-    const cudaError_t e = launch_sigma_dense(ctx->M, first_block, n_blocks, diag_rel, (const double*)L,
-                                             (const double*)R, ctx->d_Ut, ctx->d_Xt, (double*)Sl, (double*)Sg,
-                                             ctx->d_status, ctx->d_part, ctx->part_bytes, s, &k);
+    e = launch_sigma_dense(ctx->M, first_block, n_blocks, diag_rel, (const double*)L, (const double*)R, ctx->d_Ut,
+                           ctx->d_Xt, (double*)Sl, (double*)Sg, ctx->d_status, ctx->d_sd, split ? ctx->sd_bytes : 0, s,
+                           &k);
     *launches += k;
+    if (e == cudaSuccess && k > 1) e = cudaEventRecord(ctx->sd_done, s);
     if (e != cudaSuccess || !fock) return e;
     ++*launches;
     return launch_fock(*fock, s);
@@ -936,6 +949,15 @@ kbe_status kbe_set_interaction(kbe_ctx* ctx, const double* U4) {
       ctx->d_Ut = ctx->d_Xt = ctx->d_HF = nullptr;
       cudaGetLastError();
       return fail(ctx, e == cudaErrorMemoryAllocation ? KBE_ENOMEM : KBE_ECUDA, "kbe_set_interaction: allocation");
+    }
+  }
+  if (!ctx->d_sd) {
+    ctx->sd_bytes = dense_sigma_work_bytes(M, ctx->n_max);
+    if (ctx->sd_bytes > 0 &&
+        ((!ctx->sd_done && cudaEventCreateWithFlags(&ctx->sd_done, cudaEventDisableTiming) != cudaSuccess) ||
+         cudaMalloc(&ctx->d_sd, ctx->sd_bytes) != cudaSuccess)) {
+      cudaGetLastError();  // no room: rows stay whole
+      ctx->d_sd = nullptr;
     }
   }
   if ((e = cudaMemcpy(ctx->d_Ut, Ut.data(), M4 * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess ||

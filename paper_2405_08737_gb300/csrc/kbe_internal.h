@@ -162,6 +162,9 @@ struct kbe_ctx {
   // general four-index interaction (Eq. SE, Eq. eps); unset: the local U
   bool dense = false;
   double* d_Ut = nullptr;     // [d][i][e][f] = U_ifde
+  double* d_sd = nullptr;     // partial sums of split self-energy rows (null: rows stay whole)
+  size_t sd_bytes = 0;
+  cudaEvent_t sd_done = nullptr;  // recorded after each use of d_sd
   double* d_Xt = nullptr;     // [b][j][a][c] = UEx_jabc = 2 U_jbac - U_jabc
   double* d_HF = nullptr;     // [(i,j)][(b,a)] = U_iabj - 2 U_ijba (Fock matrix)
   // adaptive time stepping: self-energy and Fock rings, iterates, sums
@@ -210,6 +213,7 @@ struct DenseSigmaArgs {
 cudaError_t launch_sigma_dense(int M, int64_t first_block, int64_t n_blocks, int64_t diag_rel, const double* L,
                                const double* R, const double* Ut, const double* Xt, double* Sl, double* Sg,
                                int* status, double* work, size_t work_bytes, cudaStream_t s, int* launches);
+size_t dense_sigma_work_bytes(int M, int64_t n_max);  // of `work` for any call of a context
 cudaError_t dense_sigma_prepare(int M);  // shared-memory opt-in, outside stream capture
 size_t dense_sigma_smem(int M);
 

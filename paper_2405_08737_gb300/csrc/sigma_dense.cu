@@ -211,6 +211,16 @@ Tiling tiling(int M) {
 
 }  // namespace
 
+// Fewest units that fill the chip: 16 per SM.
+static int64_t unit_cap() { return (int64_t)sm_count() * 16; }
+static int max_slices(int M) { return M >= 8 ? std::min(8, M * M / tiling(M).g) : 1; }
+
+// A row is split up to about the cap: 2 n_blocks slices < cap + 2 n_blocks < 2 cap.
+size_t dense_sigma_work_bytes(int M, int64_t n_max) {
+  const int64_t most = std::min(2 * unit_cap(), n_max * (n_max + 1) * max_slices(M));
+  return max_slices(M) > 1 ? (size_t)most * M * M * sizeof(double2) : 0;
+}
+
 size_t dense_sigma_smem(int M) { return tiling(M).smem; }
 
 cudaError_t dense_sigma_prepare(int M) {
@@ -239,15 +249,15 @@ cudaError_t launch_sigma_dense(int M, int64_t first_block, int64_t n_blocks, int
   a.status = status;
   a.g = t.g;
   a.g3 = t.g3;
-  const int64_t cap = (int64_t)sm_count() * 16;
+  const int64_t cap = unit_cap();
   // A row of few blocks leaves the last round of CTAs on a part of the SMs (n = 255:
   // 512 units on 152 SMs, 3.4 each, the longest 4): a block's pairs are then split
   // into slices, whose sums a second launch adds (M = 16, n = 255: 12.63 -> 10.55 ms).
   // Blocks of small M take microseconds and are left whole.
   a.slices = 1;
   a.part = reinterpret_cast<double2*>(work);
-  if (M >= 8 && 2 * n_blocks < cap)
-    a.slices = (int)std::min<int64_t>((cap + 2 * n_blocks - 1) / (2 * n_blocks), std::min(8, M * M / t.g));
+  if (2 * n_blocks < cap)
+    a.slices = (int)std::min<int64_t>((cap + 2 * n_blocks - 1) / (2 * n_blocks), max_slices(M));
   while (a.slices > 1 && (size_t)(2 * a.slices * n_blocks * M * M) * sizeof(double2) > work_bytes) --a.slices;
   int64_t blocks = 2 * n_blocks * a.slices;
   if (blocks > cap) blocks = cap;

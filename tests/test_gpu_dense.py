@@ -170,6 +170,32 @@ def test_dense_sigma_full_size_sampled_blocks(kbe):
     ctx.close()
 
 
+@pytest.mark.parametrize("M,n", [(8, 40), (12, 17), (16, 9)])
+def test_dense_rows_on_two_streams(kbe, M, n):
+    """Self-energy calls of one context that overlap on two streams give the
+    bits of the calls alone: the partial sums of split rows do not mix."""
+    import torch
+    ctx = _ctx(kbe, M, n + 1)
+    ctx.set_interaction(_general_tensor(M, M))
+    L, R = (_dev(x) for x in W.random_triangles(M, n + 1, 3 * M))
+    rows = (n, n - 3)
+    out = [torch.zeros((2, r + 1, M, M), dtype=torch.complex128, device="cuda") for r in rows]
+    ref = [torch.zeros_like(x) for x in out]
+    for r, x in zip(rows, ref):
+        ctx.selfenergy_slice(r, L, R, x[0], x[1])
+        ctx.sync_status()
+    streams = [torch.cuda.Stream() for _ in rows]
+    torch.cuda.synchronize()
+    for _ in range(10):
+        for r, x, s in zip(rows, out, streams):
+            ctx.selfenergy_slice(r, L, R, x[0], x[1], stream=s)
+    torch.cuda.synchronize()
+    ctx.sync_status()
+    for x, y in zip(out, ref):
+        assert torch.equal(torch.view_as_real(x), torch.view_as_real(y))
+    ctx.close()
+
+
 def _setup(M, n_t, kind, seed, with_pulse):
     t, order = W.grid(n_t, 0.05, 0.3, seed)
     h = W.chain_h(M, 1.0) if kind == "chain" else W.goe_h(M, seed)

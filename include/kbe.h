@@ -333,9 +333,10 @@ kbe_status kbe_step_sweep_finish(kbe_ctx* ctx, int n, void* L, void* R, const vo
  * F_ring, and the new row n of L and R is copied back to L_row_host and
  * R_row_host ((n+1) M^2 complex each).  The rows are copied from row n-1
  * down in up to 5 chunks whose sizes grow geometrically (ratio 1.8, the
- * first the smallest) on a copy stream of the context; with KBE_FP64 (and no adaptive orders or thermal branch) the
- * first sweep's history slice contracts the output columns of each chunk as
- * soon as it has arrived (column c reads rows c..n only), so the copies
+ * first the smallest) on a copy stream of the context; with KBE_FP64 (and no
+ * adaptive orders or thermal branch, and a slice that stays on the FP64 pipe)
+ * the first sweep's history slice contracts the output columns of each chunk
+ * as soon as it has arrived (column c reads rows c..n only), so the copies
  * overlap the contraction; the results are bitwise those of kbe_step on the
  * same data.  Otherwise the step starts once all rows are in.  Host buffers
  * should be page-locked (cudaHostAlloc or registered) for the copies to be

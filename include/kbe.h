@@ -65,12 +65,19 @@ typedef int kbe_status;
 #define KBE_DENSE_MAX_NORB 32  /* largest norb for a dense interaction      */
 
 /* precision argument of kbe_history_slice / kbe_step */
-#define KBE_FP64 0        /* FP64 accuracy, deterministic: FP64 arithmetic;  */
-                          /* the larger slices ((n+1)^2 norb^3 >= 5e6) form   */
-                          /* their products on the tensor cores from eight    */
-                          /* error-free 8-bit digits per value (about 2^-57   */
-                          /* of the largest product of 32 history entries)    */
-                          /* and sum them in FP64                             */
+#define KBE_FP64 0        /* FP64 accuracy, deterministic: FP64 arithmetic.   */
+                          /* The larger slices ((n+1)^2 norb^3 >= 5e6 and     */
+                          /* (n+1) norb^2 > 4096) form their products on the  */
+                          /* tensor cores from eight error-free 8-bit digits  */
+                          /* per value and sum them in FP64.  Their error per */
+                          /* 64 history entries (m, x) is typically 2^-53 (at */
+                          /* most 2^-46) of the largest product max_a         */
+                          /* |Sigma(n,m)_ax| |G(m,c)_xb| met there and in the */
+                          /* 32 entries before: a bound by orbital column b,  */
+                          /* not by output entry, unless the rows a of Sigma  */
+                          /* differ by a factor each.  kbe_history_slice_     */
+                          /* noalloc and kbe_history_slice_band over part of  */
+                          /* the rows sum each product in FP64                */
 #define KBE_SPLIT_BF16 1  /* the contraction on the 16-bit-float tensor cores */
                           /* with error-free 4-digit fixed-point splitting:   */
                           /* every value becomes round(v 2^(31-e)) in base-256 */

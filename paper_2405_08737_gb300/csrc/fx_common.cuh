@@ -13,6 +13,15 @@
 // levels weigh at most 2^-59 of 2^(ev+eu), typically 2^-61, where FP64 rounds
 // every partial sum at 2^-53 (error-free slicing: Ozaki, Ogita, Oishi & Rump,
 // Numer. Algorithms 59 (2012)).
+//
+// Exponents are shared: by a history row (c, b) over an accumulation of up to 64
+// entries k = (m, x), by a row a of the small operand A over the same.  Entries are
+// scaled first, A(a,k) by 1 / s_k and the history by s_k = max_a |A(a,k)| (Exps), so
+// 2^(ev+eu) is at most 2^5 times r_a max_k s_k |G(k,c,b)| with r_a = max_k |A(a,k)| / s_k
+// <= 1: the largest product of the accumulation and of the chunk before it, whose
+// exponent the row starts from.  Per accumulation the error is then at most 2^-46 of
+// that product, typically 2^-53.  It is the output's own largest product where the rows a
+// differ by a factor each; where they do not, it is that of a larger row of the part.
 #pragma once
 
 #include <cstdint>
@@ -29,12 +38,35 @@ constexpr int kOver = 6;       // chunks that a column tile visits twice, at mos
 constexpr int kHeadroom = 2;   // bits between a row's exponent and its first values
 constexpr int kStartRoom = 3;  // the same for a row whose first values these are (6: errors up to 1.1 times as large, 8: 1.9)
 constexpr int kNonFinite = 8000;  // exponent of a row or column that holds a non-finite value
+constexpr int kFiniteMost = 2100; // no sum of two exponents of finite values scales by more than 2^this
+
+// Exponents of a half of a unit's small block, ahead of its digits.  An entry k of
+// the small operand is scaled by 2^-ek (its largest value over the rows a of the
+// part), the history entry it meets by 2^ek: then a history row's exponent holds
+// the largest of its products, whatever the two sizes do along the history, over
+// the orbitals or between the two variants.  With exponents of the operands alone a column's
+// error was up to 6e-10 of its own products for a self-energy that rises by 2^24 and a
+// history that falls by 2^8 a point (M = 33), 5e-6 for G^< and Sigma^< 2^-40 of G^> and
+// Sigma^>, and all of it for orbitals of very different sizes.
+struct Exps {
+  int16_t es[2][16];    // of row a, per variant
+  uint32_t ek[2][4];    // of entries 2i and 2i + 1 in bits 0-11 and 20-31 of word i, per variant (the band's
+                        // variants share one); bits 12-19 of words i and i + 1 (i even) hold `least`, the least
+                        // exponent of a history row: its zeros lie 63 bits below it at every entry
+  uint32_t pad[8];      // to 128 bytes: the digits' core matrices behind it stay in one line each
+};
+// `least` of the words 2q, 2q + 1
+__host__ __device__ __forceinline__ int least_of(uint32_t w0, uint32_t w1) {
+  return (int)((w0 >> 12 & 0xFFu) | (w1 >> 4 & 0xFF00u));
+}
 
 // Values of a per part, bytes of a part's small operand of one unit (two halves
-// of 64 exponent bytes and two variants of 8 digits x 16 reals x 2 NA columns),
+// of exponents and two variants of 8 digits x 16 reals x 2 NA columns),
 // complex entries of a partial slot.
 __host__ __device__ constexpr int part_rows(int M) { return M <= 8 ? 8 : 16; }
-__host__ __device__ constexpr int small_block_bytes(int NA) { return 2 * (64 + 2 * kDig * 2 * NA * 2 * kUnitK * 2); }
+__host__ __device__ constexpr int small_block_bytes(int NA) {
+  return 2 * ((int)sizeof(Exps) + 2 * kDig * 2 * NA * 2 * kUnitK * 2);
+}
 __host__ __device__ constexpr int slot_complex(int NA) { return 2 * NA * kRows; }
 
 // One system's contraction as a list of column tiles of CT = 128 / M output
@@ -200,14 +232,16 @@ __host__ __device__ __forceinline__ int field_of(uint32_t hi) { return (int)((hi
 
 // Digits of v for exponent field E (every |v| < 2^(E - 1022)), as the bytes
 // d_i + 128 of a 64-bit word, d_0 on top.  Values more than 2^62 below the
-// exponent (zeros and, for E < 64, everything below 2^-1020) give 0.
-__host__ __device__ __forceinline__ uint64_t digit_bytes(uint32_t hi, uint32_t lo, int E) {
-  int t = E - field_of(hi);
+// exponent give 0 (so zeros and subnormals need E >= 63).
+__host__ __device__ __forceinline__ uint64_t digit_bytes_at(uint32_t hi, uint32_t lo, int t) {  // t = E - field
   t = t < 63 ? t : 63;
   const uint64_t m = ((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
   const uint64_t V = (m << 9) >> t;
   const uint64_t sg = (uint64_t)((int64_t)(int32_t)hi >> 31);  // 0 or all ones
   return (V ^ sg) + 0x8080808080808080ull - sg;
+}
+__host__ __device__ __forceinline__ uint64_t digit_bytes(uint32_t hi, uint32_t lo, int E) {
+  return digit_bytes_at(hi, lo, E - field_of(hi));
 }
 
 }  // namespace fx

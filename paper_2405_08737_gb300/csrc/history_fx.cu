@@ -92,7 +92,7 @@ using split::umma_idesc_f16;
 
 constexpr int kDigPlane = kRows * 2 * kUnitK * 2;         // one digit of one plane: 4 KB
 constexpr int kPlane = kDig * kDigPlane;                  // 32 KB
-constexpr int kExpBytes = 64;                             // exponents of a part's a values (int16), padded
+constexpr int kExpBytes = sizeof(Exps);                   // exponents of a part's small operand
 constexpr int kStages = 2, kBSlots = 4, kExpRing = 32;
 constexpr int kEpiWarps = 8;
 constexpr int kConvWarps = 16;                            // 8 rows each
@@ -103,17 +103,13 @@ constexpr long long kWaitCycles = 1ll << 31;              // a work wait gives u
 template <int NA>
 struct Cfg {
   static constexpr int kN = 2 * NA;                              // real columns per digit of the small operand
-  // registers of the epilogue, converter and other warpgroups (setmaxnreg), whose
-  // sum is the launch's 896 x 72: an epilogue thread holds 2 NA FP64 sums
-  static constexpr int kRegsEpi = NA == 8 ? 104 : 112, kRegsConv = NA == 8 ? 64 : 56, kRegsMisc = NA == 8 ? 40 : 56;
-  static_assert(256 * kRegsEpi + 512 * kRegsConv + 128 * kRegsMisc == kThreads * 72, "register split");
   static constexpr int kVarBytes = 2 * kDig * (kN / 8) * 128;    // one variant's digits of a unit
   static constexpr int kHalfBytes = kExpBytes + 2 * kVarBytes;   // exponents | variant 0 | variant 1
   static constexpr int kSmallBytes = 2 * kHalfBytes;             // small block of a unit: main half, band half
   static constexpr int kBufCols = kDig * kN;                     // accumulator buffer: 8 levels x kN columns
   static constexpr int kBufs = 512 / kBufCols;
   static constexpr size_t kSlot = slot_complex(NA);              // partial sums of one (CTA, tile): [2][NA][128] complex
-  static_assert(kSmallBytes == small_block_bytes(NA), "small operand layout");
+  static_assert(kSmallBytes == small_block_bytes(NA) && kHalfBytes % 128 == 0 && kExpBytes % 128 == 0, "small operand layout");
   // an epilogue still reading an accumulation's exponents is at most kStages units
   // and the open and the buffered ones (8 units per two buffers) behind the converters
   static_assert(kStages + kChunkUnits * (kBufs + 2) < kExpRing, "exponent ring");
@@ -141,6 +137,17 @@ struct alignas(16) Post {  // what the MMA thread hands to the epilogue with a b
   int si, c0, slot;        // system; first column (scale); partial slot (flush)
   int cols;                // a values of the part, plus one
   int16_t es[16];          // small operand's exponents
+};
+
+// Registers of the epilogue, converter and other warpgroups (setmaxnreg), whose sum is
+// the launch's 896 x 72: an epilogue thread holds 2 NA FP64 sums, a converter 16 words of
+// loads, as many of digits and the entries' exponents.  (With 56 for the converters of
+// NA = 16 the slice M = 16, n = 511 takes 1.36 ms instead of 1.24, with 104, 64 and 40 the
+// slice M = 8, n = 1023 865 us instead of 836.)
+template <int NA, bool kQuad>
+struct Regs {
+  static constexpr int kEpi = NA == 8 && kQuad ? 88 : 104, kConv = NA == 8 && kQuad ? 72 : 64, kMisc = 40;
+  static_assert(256 * kEpi + 512 * kConv + 128 * kMisc == kThreads * 72, "register split");
 };
 
 template <int NA>
@@ -238,8 +245,9 @@ __device__ __forceinline__ uint64_t bytes_of(double v, int E) {
 __device__ __forceinline__ int field64(double v) { return field_of((uint32_t)__double2hiint(v)); }
 
 // Small operands of a pair of chunks and a part (grid-stride over them; warp = a,
-// a lane has one entry of each chunk), with one exponent per a, pair and half
-// (near sums accumulate over the pair), in the real form
+// a lane has one entry of each chunk): an exponent per entry k, unit half and
+// variant (Exps), and with those taken off one exponent per a, pair, half and
+// variant (near sums accumulate over the pair), in the real form
 // of a complex product: columns (a, re): (P.re, -P.im), (a, im): (P.im, P.re) over
 // the entry's (re, im).  Layout of a variant of a unit: [K group 2][digit 8]
 // [column group][8 columns][8 reals].  With (l, g) = (S^<, S^>), resp. (Ibar^<, Ibar^>):
@@ -248,6 +256,7 @@ __device__ __forceinline__ int field64(double v) { return field_of((uint32_t)__d
 template <int NA>
 __global__ void __launch_bounds__(32 * NA) fx_prep(const __grid_constant__ Args a) {
   using C = Cfg<NA>;
+  __shared__ int s_ek[2][2][2][kChunkK];  // [half][variant][chunk][entry]: largest field over the rows a
   grid_launch_next();
   grid_wait();
   const int al = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -257,6 +266,8 @@ __global__ void __launch_bounds__(32 * NA) fx_prep(const __grid_constant__ Args 
     const int M = s.M, MM = M * M, n = s.n, parts = s.parts;
     const int pair = (int)((ch - s.chunk_base) / parts), p = (int)(ch - s.chunk_base - (long long)pair * parts);
     const int row = p * NA + al;
+    __syncthreads();
+    for (int i = threadIdx.x; i < 8 * kChunkK; i += 32 * NA) (&s_ek[0][0][0][0])[i] = 0;
     double2 l[2], g[2];
     double w0[2] = {1.0, 1.0}, w1[2] = {1.0, 1.0};
 #pragma unroll
@@ -273,31 +284,63 @@ __global__ void __launch_bounds__(32 * NA) fx_prep(const __grid_constant__ Args 
         }
       }
     }
-    const int kl = lane % kUnitK, kg = kl >> 2, kin = 2 * (kl & 3), cre = 2 * al, cim = 2 * al + 1;
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      double v[2][2][2];  // [chunk][variant][re, im]
-      int E = 0;
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const double dx = g[k].x - l[k].x, dy = g[k].y - l[k].y, sx = l[k].x + g[k].x, sy = l[k].y + g[k].y;
-        v[k][0][0] = s.adj ? (half ? g[k].x : -sx) : (half ? l[k].x : w0[k] * dx);
-        v[k][0][1] = s.adj ? (half ? g[k].y : -sy) : (half ? l[k].y : w0[k] * dy);
-        v[k][1][0] = s.adj ? (half ? sx : -g[k].x) : (half ? dx : -w1[k] * l[k].x);
-        v[k][1][1] = s.adj ? (half ? sy : -g[k].y) : (half ? dy : -w1[k] * l[k].y);
-        E = max(E, max(max(field64(v[k][0][0]), field64(v[k][0][1])), max(field64(v[k][1][0]), field64(v[k][1][1]))));
+    // (re, im) of a half's variants
+    auto values = [&](int half, int k, int var) -> double2 {
+      const double2 d = make_double2(g[k].x - l[k].x, g[k].y - l[k].y), t = make_double2(l[k].x + g[k].x, l[k].y + g[k].y);
+      if (s.adj) {
+        const double2 v = half ? (var ? t : g[k]) : (var ? g[k] : t);
+        return half ? v : make_double2(-v.x, -v.y);
       }
-      E = __reduce_max_sync(0xffffffffu, E);
-      E = E == 0x7FF ? kNonFinite : max(E, 64);
+      if (half) return var ? d : l[k];
+      return var ? make_double2(-w1[k] * l[k].x, -w1[k] * l[k].y) : make_double2(w0[k] * d.x, w0[k] * d.y);
+    };
+    __syncthreads();
+#pragma unroll
+    for (int half = 0; half < 2; ++half)
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        if (2 * pair + k >= s.cpt) break;
-        const int unit = (2 * pair + k) * kChunkUnits + lane / kUnitK;
-        uint8_t* out = s.small + ((size_t)unit * parts + p) * C::kSmallBytes + half * C::kHalfBytes;
-        if (kl == 0) reinterpret_cast<int16_t*>(out)[al] = (int16_t)E;
+        int f[2];
 #pragma unroll
         for (int var = 0; var < 2; ++var) {
-          const uint64_t br = bytes_of(v[k][var][0], E), bi = bytes_of(v[k][var][1], E);
+          const double2 v = values(half, k, var);
+          f[var] = max(field64(v.x), field64(v.y));
+          if (f[var] == 0x7FF) f[var] = 0;
+        }
+        if (half) f[0] = f[1] = max(f[0], f[1]);
+        if (f[0]) atomicMax(&s_ek[half][0][k][lane], f[0]);
+        if (f[1]) atomicMax(&s_ek[half][1][k][lane], f[1]);
+      }
+    __syncthreads();
+    const int kl = lane % kUnitK, kg = kl >> 2, kin = 2 * (kl & 3), cre = 2 * al, cim = 2 * al + 1;
+#pragma unroll
+    for (int half = 0; half < 2; ++half)
+#pragma unroll
+      for (int var = 0; var < 2; ++var) {
+        double2 v[2];
+        int ek[2], E = -kNonFinite;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          v[k] = values(half, k, var);
+          ek[k] = s_ek[half][var][k][lane];
+          const int f = max(field64(v[k].x), field64(v[k].y));
+          if (f) E = max(E, f == 0x7FF ? kNonFinite : f - ek[k]);
+        }
+        E = __reduce_max_sync(0xffffffffu, E);
+        if (E == -kNonFinite) E = 0;  // zeros
+        const int least = __reduce_max_sync(0xffffffffu, max(ek[0], ek[1])) + 64;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          if (2 * pair + k >= s.cpt) break;
+          const int unit = (2 * pair + k) * kChunkUnits + lane / kUnitK;
+          uint8_t* out = s.small + ((size_t)unit * parts + p) * C::kSmallBytes + half * C::kHalfBytes;
+          Exps& x = *reinterpret_cast<Exps*>(out);
+          if (kl == 0) x.es[var][al] = (int16_t)E;
+          const int ek1 = __shfl_down_sync(0xffffffffu, ek[k], 1);
+          if (al == 0 && !(kl & 1))
+            x.ek[var][kl >> 1] = (uint32_t)ek[k] | (uint32_t)(kl & 2 ? least >> 8 : least & 0xFF) << 12 | (uint32_t)ek1 << 20;
+          // zeros (and subnormals) whatever the exponents
+          const uint64_t br = bytes_of(v[k].x, field64(v[k].x) ? E + ek[k] : kNonFinite),
+                         bi = bytes_of(v[k].y, field64(v[k].y) ? E + ek[k] : kNonFinite);
 #pragma unroll
           for (int d = 0; d < kDig; ++d) {
             const uint32_t ri = digit_of(d, br, bi);              // (re, im)
@@ -308,7 +351,6 @@ __global__ void __launch_bounds__(32 * NA) fx_prep(const __grid_constant__ Args 
           }
         }
       }
-    }
   }
 }
 
@@ -481,11 +523,11 @@ __device__ __forceinline__ void fold(double (&s)[NA], uint32_t at, int E, int ha
     }
 #pragma unroll
     for (int i = 0; i < kCols; ++i) {
-      // scale 2^(ev + eu - 68 + 12), ev = E - 1022, eu = es - 1022
+      // scale 2^(ev + eu - 68 + 12), ev = E - 1022, eu = es - 1022 (the entries' own exponents cancel)
       const int ex = E + es[i / 2] - 2 * 1022 - 56;
       if (ex >= -1022 && ex <= 1023) {
         s[c2 + i] = fma((double)t[i], __hiloint2double((ex + 1023) << 20, 0), s[c2 + i]);
-      } else if (ex >= kNonFinite - 4096) {
+      } else if (ex > kFiniteMost) {
         s[c2 + i] = __longlong_as_double(0x7FF8000000000000ll);
       } else {  // the scale alone leaves the range of FP64
         const int h = ex / 2;
@@ -534,7 +576,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
     // --------------------------------------------------------- epilogue --
     // warp = 4 half + quadrant: 32 output rows (tensor-memory lanes), the even
     // or the odd a values of the part (kN / 2 columns)
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::kRegsEpi));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(Regs<NA, kQuad>::kEpi));
     constexpr int kC = kN / 2;
     const int quad = warp & 3, half = warp >> 2;
     const int j = quad * 32 + lane;
@@ -592,14 +634,15 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
     // ------------------------------------------------------- converters --
     // lane = row (3 bits) | K half q << 3 | plane << 4: a quarter warp writes
     // 128 consecutive bytes of a digit plane
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsConv));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(Regs<NA, kQuad>::kConv));
     const int wq = warp - kEpiWarps;
     const int q = (lane >> 3) & 1, plane = lane >> 4;
     const uint32_t dst0 = plane * kPlane + (q * 16 + wq) * 128 + (lane & 7) * 16;
     Row row;
     double2 z[4];
     unsigned mask = 0, d = 0;
-    int flags = 0, kap = 0, si = 0, E = 64, seen = 64;  // of the unit in z; the row's exponent; largest field of the current chunk
+    uint2 ekw = make_uint2(0, 0);  // exponents of the entries in z
+    int flags = 0, kap = 0, si = 0, E = 64, seen = 0;  // of the unit in z; the row's exponent; largest field of the current chunk
     // the next unit's loads; false when there is none
     auto load = [&]() -> bool {
       Desc ds;
@@ -614,6 +657,9 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       if (flags & kNewTile) row = row_of(sys_at(a, ds.aux), ds.c0, 8 * wq + (lane & 7), plane);
       kap = ds.kap + 4 * q;
       si = ds.aux;
+      // (read here and not when the unit is converted: behind the digit stores a read waits long; M = 8, n = 1023 963 us instead of 865)
+      ekw = *reinterpret_cast<const uint2*>(
+          &reinterpret_cast<const Exps*>(sm.small[(d - 1) % kBSlots])->ek[plane && !(flags & kFlagNear)][2 * q]);
       if (flags & kFlagBand) {
         band_values(sys_at(a, ds.aux), row, kap, plane, z);
         mask = 15u;
@@ -626,32 +672,45 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
     for (unsigned u = 0; more; ++u) {
       const int s = u % kStages;
       if (flags & kFlagBand) band_weights(sys_at(a, si), row, kap, z);
-      // exponent of the row
-      int mx = 0;
+      // exponent of the row, of the entries scaled as the small operand says
+      const uint32_t ek[4] = {ekw.x << 20, ekw.x & 0xFFF00000u, ekw.y << 20, ekw.y & 0xFFF00000u};
+      uint32_t top = 0, most = 0;  // (a zero counts as 2^-1022: below any product that matters)
 #pragma unroll
-      for (int i = 0; i < 4; ++i)  // masked entries are zero without kQuad
-        mx = __vimax3_s32(mx, __double2hiint(z[i].x) & 0x7FFFFFFF, __double2hiint(z[i].y) & 0x7FFFFFFF);
-      if (kQuad && !(mask & 1u)) mx = 0;
-      mx >>= 20;
+      for (int i = 0; i < 4; ++i) {  // masked entries are zero without kQuad
+        const uint32_t re = (uint32_t)__double2hiint(z[i].x) & 0x7FFFFFFFu, im = (uint32_t)__double2hiint(z[i].y) & 0x7FFFFFFFu;
+        most = __vimax3_u32(most, re, im);
+        top = __vimax3_u32(top, re + ek[i], im + ek[i]);
+      }
+      int mx = (int)(top >> 20);
+      if (most < 0x100000u || (kQuad && !(mask & 1u))) mx = 0;  // nothing but zeros
+      else if (most >= 0x7FF00000u) mx = kNonFinite;
       mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
       bool raised = false;
       if (flags & kFirst) {
-        const int prev = (flags & kFresh) || seen == 0x7FF ? 0 : seen;
-        E = max(max(mx, prev), 64) + (prev ? kHeadroom : kStartRoom);
+        const int prev = (flags & kFresh) || seen == kNonFinite ? 0 : seen;
+        E = max(max(mx, prev), least_of(ekw.x, ekw.y)) + (prev ? kHeadroom : kStartRoom);
         seen = mx;
       } else {
         if (mx > E) { raised = seen > 0; E = mx + (raised ? kHeadroom : kStartRoom); }
-        if (mx == 0x7FF) { raised |= seen > 0 && E != kNonFinite; }
         seen = max(seen, mx);
       }
-      if (mx == 0x7FF) E = kNonFinite;
+      if (mx == kNonFinite) E = kNonFinite;
       const int Ez = kQuad && !(mask & 1u) ? kNonFinite : E;  // a masked quad's digits are zero
       uint64_t br[4], bi[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const uint32_t fl = (kQuad ? mask << 24 : mask << (27 - i)) & 0x80000000u;
-        br[i] = digit_bytes((uint32_t)__double2hiint(z[i].x) ^ fl, (uint32_t)__double2loint(z[i].x), Ez);
-        bi[i] = digit_bytes((uint32_t)__double2hiint(z[i].y), (uint32_t)__double2loint(z[i].y), Ez);
+        const uint32_t re = (uint32_t)__double2hiint(z[i].x), im = (uint32_t)__double2hiint(z[i].y);
+        // E - ek - field, summed in the order that costs fewer registers (M = 8, n = 1023: 865 -> 836 us; M = 5, n = 333:
+        // 226 -> 217 us a step the other way)
+        if constexpr (NA == 8 && kQuad) {
+          const int Ei = Ez - (int)(ek[i] >> 20);
+          br[i] = digit_bytes(re ^ fl, (uint32_t)__double2loint(z[i].x), Ei);
+          bi[i] = digit_bytes(im, (uint32_t)__double2loint(z[i].y), Ei);
+        } else {
+          br[i] = digit_bytes_at(re ^ fl, (uint32_t)__double2loint(z[i].x), Ez - (int)(((re & 0x7FFFFFFFu) + ek[i]) >> 20));
+          bi[i] = digit_bytes_at(im, (uint32_t)__double2loint(z[i].y), Ez - (int)(((im & 0x7FFFFFFFu) + ek[i]) >> 20));
+        }
       }
       more = load();  // in flight while this unit's digits are written
       if (!__all_sync(0xffffffffu, wait_bar(&sm.abort, &sm.empty[s], ((u / kStages) & 1) ^ 1, status))) break;
@@ -668,7 +727,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       if (lane == 0) mbar_arrive(&sm.full[s]);
     }
   } else {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsMisc));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(Regs<NA, kQuad>::kMisc));
     if (warp == kProdWarp && lane == 0) {
       // ------------------------------------------------------- producer --
       unsigned d = 0;
@@ -821,7 +880,8 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
           ps.cols = (ds.flags >> 16) + 1;
 #pragma unroll
           for (int i = 0; i < NA / 8; ++i)
-            reinterpret_cast<int4*>(ps.es)[i] = reinterpret_cast<const int4*>(sm.small[b])[i];
+            reinterpret_cast<int4*>(ps.es)[i] =
+                reinterpret_cast<const int4*>(reinterpret_cast<const Exps*>(sm.small[b])->es[me && !near])[i];
         }
         tc_fence_after();
         // far: PL x variant 0 and Q x variant 1, both to I^<; near: PL and Q x

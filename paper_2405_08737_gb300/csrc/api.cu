@@ -408,19 +408,17 @@ kbe_status step_impl(kbe_ctx* ctx, int n, int P, int precision, void* L, void* R
     if (ctx->thermal) {
       ThermalArgs x = thermal_args(ctx, a, Sl, Sg, I_work);
       x.df = precision != KBE_FP64;  // the thermal sums in double-float with the faster contractions
-      if ((e = thermal_sweep_a(ctx, x, s)) != cudaSuccess || (e = launch_rhs_corrector(a, s)) != cudaSuccess ||
+      if ((e = thermal_sweep_a(ctx, x, s)) != cudaSuccess || (e = launch_rhs_corrector(a, s, &count)) != cudaSuccess ||
           (e = launch_th_rhs(x, s)) != cudaSuccess || (e = launch_th_adams(x, true, s)) != cudaSuccess) {
-        *count_out = count + 5;
+        *count_out = count + 4;
         return cuda_fail(ctx, e, "kbe_step: thermal corrector");
       }
-      *count_out = (count += 5);
+      *count_out = (count += 4);
       continue;
     }
-    if ((e = launch_rhs_corrector(a, s)) != cudaSuccess) {
-      *count_out = count + 1;
-      return cuda_fail(ctx, e, "kbe_step: corrector");
-    }
-    *count_out = (count += 1);
+    e = launch_rhs_corrector(a, s, &count);
+    *count_out = count;
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "kbe_step: corrector");
   }
   if ((e = keep(P)) != cudaSuccess) return cuda_fail(ctx, e, "kbe_step: iterate copy");
   return KBE_OK;
@@ -1092,8 +1090,8 @@ kbe_status kbe_step_sweep_finish(kbe_ctx* ctx, int n, void* L, void* R, const vo
   cudaStream_t s = (cudaStream_t)stream;
   StepArgs a = step_args(ctx, n, L, R, I, F_ring);
   cudaError_t e = launch_fock(a, s);
-  if (e == cudaSuccess) e = launch_rhs_corrector(a, s);
-  ctx->last_launches = 2;
+  ctx->last_launches = 1;
+  if (e == cudaSuccess) e = launch_rhs_corrector(a, s, &ctx->last_launches);
   return e == cudaSuccess ? KBE_OK : cuda_fail(ctx, e, "kbe_step_sweep_finish");
 }
 

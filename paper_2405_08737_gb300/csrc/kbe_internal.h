@@ -358,7 +358,7 @@ cudaError_t launch_run_small(const RunSmallHost& h, cudaStream_t s, int* launche
 cudaError_t launch_init_row0(int M, const double* rho, double* L, double* R, cudaStream_t s);
 cudaError_t launch_fock(const StepArgs& a, cudaStream_t s);
 cudaError_t launch_rhs(const StepArgs& a, cudaStream_t s);          // F row n only
-cudaError_t launch_rhs_corrector(const StepArgs& a, cudaStream_t s);  // F row n, then new row n
+cudaError_t launch_rhs_corrector(const StepArgs& a, cudaStream_t s, int* launches);  // F row n, then new row n
 
 // ---- adaptive history orders (adaptive.cu) -------------------------------
 struct SelectArgs {

@@ -14,8 +14,6 @@
 //
 // All kernels here are elementwise over the (2n+1) M^2 entries of a row.
 
-#include <algorithm>
-
 #include "row_kernels.cuh"
 
 namespace kbe {
@@ -32,9 +30,16 @@ __global__ void __launch_bounds__(256) predictor_kernel(StepArgs a) {
 }
 
 __global__ void __launch_bounds__(256) rhs_kernel(StepArgs a) {
+  grid_wait();
   const int64_t lin = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (lin >= (int64_t)(a.n + 1) * a.M * a.M) return;
   if (!rk::rhs_entry(a, lin)) atomicOr(a.status, kStatusNumeric);
+}
+
+__global__ void __launch_bounds__(256) corrector_kernel(StepArgs a) {
+  grid_wait();
+  const int64_t lin = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (lin < (int64_t)(a.n + 1) * a.M * a.M) rk::adams_entry(a, lin, true);
 }
 
 // Right-hand side, then corrector, of the columns of a block: an entry's right-hand
@@ -85,9 +90,24 @@ cudaError_t launch_rhs(const StepArgs& a, cudaStream_t s) {
   rhs_kernel<<<blocks_for((int64_t)(a.n + 1) * a.M * a.M), 256, 0, s>>>(a);
   return cudaGetLastError();
 }
-cudaError_t launch_rhs_corrector(const StepArgs& a, cudaStream_t s) {
-  const int cols = std::max(1, 256 / (a.M * a.M));
-  return launch_overlapped(rhs_corrector_kernel, (unsigned)((a.n + cols) / cols), 256, 0, s, a, cols);
+// Together while a block's threads cover a column (M <= 16: n = 14 18.6 us with the
+// Fock matrix, 20.7 apart at M = 17).  Beyond, a block would take M^2 / 256 turns of
+// M-long sums one after the other on only n + 1 blocks, so the two run over all
+// entries (us, together / apart: M = 17, n = 16 29 / 21, M = 32, n = 20 103 / 33,
+// M = 64, n = 5 702 / 56).
+cudaError_t launch_rhs_corrector(const StepArgs& a, cudaStream_t s, int* launches) {
+  const int MM = a.M * a.M;
+  if (MM <= 256) {
+    const int cols = 256 / MM;
+    ++*launches;
+    return launch_overlapped(rhs_corrector_kernel, (unsigned)((a.n + cols) / cols), 256, 0, s, a, cols);
+  }
+  const unsigned blocks = blocks_for((int64_t)(a.n + 1) * MM);
+  ++*launches;
+  const cudaError_t e = launch_overlapped(rhs_kernel, blocks, 256, 0, s, a);
+  if (e != cudaSuccess) return e;
+  ++*launches;
+  return launch_overlapped(corrector_kernel, blocks, 256, 0, s, a);
 }
 
 }  // namespace kbe

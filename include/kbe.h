@@ -192,7 +192,10 @@ kbe_status kbe_copy_mixed(kbe_ctx* ctx, int n_rows, void* buf, int to_context, v
  * integrals; no symmetry is assumed or used).  The self-energy becomes
  *   Sigma^<>_ij(t,t') = U_ifde UEx_jabc G^<>_fb(t,t') G^<>_ea(t,t') G^><_cd(t',t),
  *   UEx_jabc = 2 U_jbac - U_jabc,
- * evaluated in FP64 with 12 M^5 multiply-adds per block and component, and
+ * evaluated in FP64 with 12 M^5 multiply-adds per block and component (rows of
+ * few blocks spread a block over several thread blocks; a call under stream
+ * capture, or of a context without room for the partial sums, adds the same
+ * parts one after the other: the same result, up to 1.2 times the time), and
  * the Fock matrix eps_ij = h_ij(t) + i (U_iabj - 2 U_ijba) G^<_ba(t,t).  The
  * tensor is copied (3 M^4 doubles on the device, synchronously); the
  * model's pulse and v stay in force and its U is unused.  U4 = NULL returns

@@ -212,8 +212,8 @@ cudaError_t sigma_blocks(kbe_ctx* ctx, int64_t first_block, int64_t n_blocks, in
                          const StepArgs* fock = nullptr) {
   if (ctx->dense) {
     // Self-energy calls of one context may overlap on different streams, so the partial sums of split rows
-    // have a buffer of their own, which the calls take in turn; captured calls leave rows whole (a wait for
-    // an event of another stream's past would end the capture).
+    // have a buffer of their own, which the calls take in turn; captured calls add a block's slices in one
+    // unit (a wait for an event of another stream's past would end the capture), with the same sums.
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(s, &capture);
     const bool split = e == cudaSuccess && capture == cudaStreamCaptureStatusNone && ctx->d_sd;

@@ -207,12 +207,13 @@ struct DenseSigmaArgs {
   double2* Sg;
   int* status;
   int g, g3;          // pairs per tile, accumulator groups
-  int slices;         // parts of a block's pairs, one unit each (1: whole blocks)
-  double2* part;      // their partial sums [slice][s][block][M][M]
+  int slices;         // parts of a block's pairs, summed one after the other
+  double2* part;      // a unit per slice: the partial sums [slice][s][block][M][M]; null: a unit per block
 };
 cudaError_t launch_sigma_dense(int M, int64_t first_block, int64_t n_blocks, int64_t diag_rel, const double* L,
                                const double* R, const double* Ut, const double* Xt, double* Sl, double* Sg,
                                int* status, double* work, size_t work_bytes, cudaStream_t s, int* launches);
+int dense_sigma_slices(int M, int64_t n_blocks);  // 1: a call uses no workspace
 size_t dense_sigma_work_bytes(int M, int64_t n_max);  // of `work` for any call of a context
 cudaError_t dense_sigma_prepare(int M);  // shared-memory opt-in, outside stream capture
 size_t dense_sigma_smem(int M);

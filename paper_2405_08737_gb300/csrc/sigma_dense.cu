@@ -56,14 +56,13 @@ __global__ void __launch_bounds__(kThreads) sigma_dense_kernel(DenseSigmaArgs a)
   double2* sQ = sT + g * MM;
   double2* sP = sQ + g * MM;
   const int tid = threadIdx.x;
-  const int64_t n_units = 2 * a.n_blocks * a.slices;
+  const bool split = a.part != nullptr;     // a unit is one slice, else all of them in order
+  const int parts = split ? a.slices : 1, tiles = (MM + g - 1) / g;
+  const int64_t n_units = 2 * a.n_blocks * parts;
   bool ok = true;
   for (int64_t u = blockIdx.x; u < n_units; u += gridDim.x) {
-    const int64_t blk = (u >> 1) / a.slices;
-    const int s = (int)(u & 1), slice = (int)((u >> 1) - blk * a.slices);
-    // this unit's pairs (d, b), whole tiles of g
-    const int tiles = (MM + g - 1) / g;
-    const int q_lo = tiles * slice / a.slices * g, q_hi = min(MM, tiles * (slice + 1) / a.slices * g);
+    const int64_t blk = (u >> 1) / parts;
+    const int s = (int)(u & 1), part = (int)((u >> 1) - blk * parts);
     bool diag;
     if (a.diag_rel >= 0) {
       diag = blk == a.diag_rel;
@@ -86,95 +85,109 @@ __global__ void __launch_bounds__(kThreads) sigma_dense_kernel(DenseSigmaArgs a)
       }
     }
     __syncthreads();
-    double2 acc[kMaxAcc];
+    for (int slice = part; slice < (split ? part + 1 : a.slices); ++slice) {
+      double2 acc[kMaxAcc];
 #pragma unroll
-    for (int k = 0; k < kMaxAcc; ++k) acc[k] = make_double2(0.0, 0.0);
-    for (int q0 = q_lo; q0 < q_hi; q0 += g) {
-      const int gc = min(g, q_hi - q0);
-      const int nT = gc * MM;
-      // T^{db} and Q^{db} for the pairs of this tile
-      for (int o = tid; o < 2 * nT; o += kThreads) {
-        const bool isQ = o >= nT;
-        const int oo = isQ ? o - nT : o;
-        const int p = oo / MM, rc = oo - p * MM;
-        const int q = q0 + p, d = q / M, b = q - d * M;
-        double2 v = make_double2(0.0, 0.0);
-        if (!isQ) {
-          const double* w = a.Ut + ((int64_t)d * MM + rc) * M;  // U_{i f d e}, f = 0..M-1
-          for (int f = 0; f < M; ++f) {
-            const double c = __ldg(w + f);
-            const double2 x = sA[f * M + b];
-            v.x = fma(c, x.x, v.x);
-            v.y = fma(c, x.y, v.y);
+      for (int k = 0; k < kMaxAcc; ++k) acc[k] = make_double2(0.0, 0.0);
+      // this slice's pairs (d, b), whole tiles of g
+      const int q_lo = tiles * slice / a.slices * g, q_hi = min(MM, tiles * (slice + 1) / a.slices * g);
+      for (int q0 = q_lo; q0 < q_hi; q0 += g) {
+        const int gc = min(g, q_hi - q0);
+        const int nT = gc * MM;
+        // T^{db} and Q^{db} for the pairs of this tile
+        for (int o = tid; o < 2 * nT; o += kThreads) {
+          const bool isQ = o >= nT;
+          const int oo = isQ ? o - nT : o;
+          const int p = oo / MM, rc = oo - p * MM;
+          const int q = q0 + p, d = q / M, b = q - d * M;
+          double2 v = make_double2(0.0, 0.0);
+          if (!isQ) {
+            const double* w = a.Ut + ((int64_t)d * MM + rc) * M;  // U_{i f d e}, f = 0..M-1
+            for (int f = 0; f < M; ++f) {
+              const double c = __ldg(w + f);
+              const double2 x = sA[f * M + b];
+              v.x = fma(c, x.x, v.x);
+              v.y = fma(c, x.y, v.y);
+            }
+            sT[oo] = v;
+          } else {
+            const double* w = a.Xt + ((int64_t)b * MM + rc) * M;  // UEx_{j a b c}, c = 0..M-1
+            for (int c = 0; c < M; ++c) {
+              const double cw = __ldg(w + c);
+              const double2 x = sC[c * M + d];
+              v.x = fma(cw, x.x, v.x);
+              v.y = fma(cw, x.y, v.y);
+            }
+            sQ[oo] = v;
           }
-          sT[oo] = v;
-        } else {
-          const double* w = a.Xt + ((int64_t)b * MM + rc) * M;  // UEx_{j a b c}, c = 0..M-1
-          for (int c = 0; c < M; ++c) {
-            const double cw = __ldg(w + c);
-            const double2 x = sC[c * M + d];
-            v.x = fma(cw, x.x, v.x);
-            v.y = fma(cw, x.y, v.y);
-          }
-          sQ[oo] = v;
         }
-      }
-      __syncthreads();
-      // P^{db}_ia = sum_e T^{db}_ie A_ea
-      for (int o = tid; o < nT; o += kThreads) {
-        const int p = o / MM, rc = o - p * MM, i = rc / M, ca = rc - i * M;
-        const double2* t = sT + p * MM + i * M;
-        double2 v = make_double2(0.0, 0.0);
-        for (int e = 0; e < M; ++e) cfma(v, t[e], sA[e * M + ca]);
-        sP[o] = v;
-      }
-      __syncthreads();
-      // Sigma_ij += sum_a P^{db}_ia Q^{db}_ja, pairs split over G3 groups
+        __syncthreads();
+        // P^{db}_ia = sum_e T^{db}_ie A_ea
+        for (int o = tid; o < nT; o += kThreads) {
+          const int p = o / MM, rc = o - p * MM, i = rc / M, ca = rc - i * M;
+          const double2* t = sT + p * MM + i * M;
+          double2 v = make_double2(0.0, 0.0);
+          for (int e = 0; e < M; ++e) cfma(v, t[e], sA[e * M + ca]);
+          sP[o] = v;
+        }
+        __syncthreads();
+        // Sigma_ij += sum_a P^{db}_ia Q^{db}_ja, pairs split over G3 groups
 #pragma unroll
-      for (int k = 0; k < kMaxAcc; ++k) {
-        const int item = tid + k * kThreads;
-        if (item < G3 * MM) {
-          const int grp = item / MM, ij = item - grp * MM, i = ij / M, j = ij - i * M;
-          double2 v = acc[k];
-          for (int p = grp; p < gc; p += G3) {
-            const double2* pp = sP + p * MM + i * M;
-            const double2* qq = sQ + p * MM + j * M;
-            for (int c = 0; c < M; ++c) cfma(v, pp[c], qq[c]);
+        for (int k = 0; k < kMaxAcc; ++k) {
+          const int item = tid + k * kThreads;
+          if (item < G3 * MM) {
+            const int grp = item / MM, ij = item - grp * MM, i = ij / M, j = ij - i * M;
+            double2 v = acc[k];
+            for (int p = grp; p < gc; p += G3) {
+              const double2* pp = sP + p * MM + i * M;
+              const double2* qq = sQ + p * MM + j * M;
+              for (int c = 0; c < M; ++c) cfma(v, pp[c], qq[c]);
+            }
+            acc[k] = v;
           }
-          acc[k] = v;
+        }
+        __syncthreads();
+      }
+      double2* out = split ? a.part + ((slice * 2 + s) * a.n_blocks + blk) * MM : (s == 0 ? a.Sl : a.Sg) + blk * MM;
+      const bool add = !split && slice > 0;  // to the slices before it, as sigma_dense_sum does
+      if (G3 == 1) {
+#pragma unroll
+        for (int k = 0; k < kMaxAcc; ++k) {
+          const int item = tid + k * kThreads;
+          if (item < MM) {
+            double2 v = acc[k];
+            if (add) {
+              v.x = out[item].x + v.x;
+              v.y = out[item].y + v.y;
+            }
+            out[item] = v;
+            ok &= isfinite(v.x) && isfinite(v.y);
+          }
+        }
+      } else {
+        double2* red = sT;  // G3 * MM <= g * MM entries
+#pragma unroll
+        for (int k = 0; k < kMaxAcc; ++k) {
+          const int item = tid + k * kThreads;
+          if (item < G3 * MM) red[item] = acc[k];
+        }
+        __syncthreads();
+        for (int ij = tid; ij < MM; ij += kThreads) {
+          double2 v = red[ij];
+          for (int grp = 1; grp < G3; ++grp) {
+            v.x += red[grp * MM + ij].x;
+            v.y += red[grp * MM + ij].y;
+          }
+          if (add) {
+            v.x = out[ij].x + v.x;
+            v.y = out[ij].y + v.y;
+          }
+          out[ij] = v;
+          ok &= isfinite(v.x) && isfinite(v.y);
         }
       }
       __syncthreads();
     }
-    double2* out = a.slices > 1 ? a.part + ((slice * 2 + s) * a.n_blocks + blk) * MM : (s == 0 ? a.Sl : a.Sg) + blk * MM;
-    if (G3 == 1) {
-#pragma unroll
-      for (int k = 0; k < kMaxAcc; ++k) {
-        const int item = tid + k * kThreads;
-        if (item < MM) {
-          out[item] = acc[k];
-          ok &= isfinite(acc[k].x) && isfinite(acc[k].y);
-        }
-      }
-    } else {
-      double2* red = sT;  // G3 * MM <= g * MM entries
-#pragma unroll
-      for (int k = 0; k < kMaxAcc; ++k) {
-        const int item = tid + k * kThreads;
-        if (item < G3 * MM) red[item] = acc[k];
-      }
-      __syncthreads();
-      for (int ij = tid; ij < MM; ij += kThreads) {
-        double2 v = red[ij];
-        for (int grp = 1; grp < G3; ++grp) {
-          v.x += red[grp * MM + ij].x;
-          v.y += red[grp * MM + ij].y;
-        }
-        out[ij] = v;
-        ok &= isfinite(v.x) && isfinite(v.y);
-      }
-    }
-    __syncthreads();
   }
   if (!ok) atomicOr(a.status, kStatusNumeric);
 }
@@ -215,6 +228,18 @@ Tiling tiling(int M) {
 static int64_t unit_cap() { return (int64_t)sm_count() * 16; }
 static int max_slices(int M) { return M >= 8 ? std::min(8, M * M / tiling(M).g) : 1; }
 
+// Slices of a block's pairs (d, b) whose sums are added in order.  A row of few blocks
+// leaves the last round of CTAs on a part of the SMs (n = 255: 512 units on
+// 152 SMs, 3.4 each, the longest 4): the slices are then units of their own, whose sums a
+// second launch adds (M = 16, n = 255: 12.63 -> 10.55 ms).
+// Blocks of small M take microseconds and are left whole.  The number depends on
+// the sizes alone, so that results do not depend on how a call is run.
+int dense_sigma_slices(int M, int64_t n_blocks) {
+  const int64_t units = 2 * n_blocks;
+  if (units >= unit_cap()) return 1;
+  return (int)std::min<int64_t>((unit_cap() + units - 1) / units, max_slices(M));
+}
+
 // A row is split up to about the cap: 2 n_blocks slices < cap + 2 n_blocks < 2 cap.
 size_t dense_sigma_work_bytes(int M, int64_t n_max) {
   const int64_t most = std::min(2 * unit_cap(), n_max * (n_max + 1) * max_slices(M));
@@ -249,22 +274,15 @@ cudaError_t launch_sigma_dense(int M, int64_t first_block, int64_t n_blocks, int
   a.status = status;
   a.g = t.g;
   a.g3 = t.g3;
-  const int64_t cap = unit_cap();
-  // A row of few blocks leaves the last round of CTAs on a part of the SMs (n = 255:
-  // 512 units on 152 SMs, 3.4 each, the longest 4): a block's pairs are then split
-  // into slices, whose sums a second launch adds (M = 16, n = 255: 12.63 -> 10.55 ms).
-  // Blocks of small M take microseconds and are left whole.
-  a.slices = 1;
-  a.part = reinterpret_cast<double2*>(work);
-  if (2 * n_blocks < cap)
-    a.slices = (int)std::min<int64_t>((cap + 2 * n_blocks - 1) / (2 * n_blocks), max_slices(M));
-  while (a.slices > 1 && (size_t)(2 * a.slices * n_blocks * M * M) * sizeof(double2) > work_bytes) --a.slices;
-  int64_t blocks = 2 * n_blocks * a.slices;
-  if (blocks > cap) blocks = cap;
+  a.slices = dense_sigma_slices(M, n_blocks);
+  // without a workspace a unit takes its block's slices in order: the same sums
+  const bool split = a.slices > 1 && (size_t)(2 * a.slices * n_blocks * M * M) * sizeof(double2) <= work_bytes;
+  a.part = split ? reinterpret_cast<double2*>(work) : nullptr;
+  const int64_t blocks = std::min(2 * n_blocks * (split ? a.slices : 1), unit_cap());
   sigma_dense_kernel<<<(unsigned)blocks, kThreads, t.smem, s>>>(a);
   ++*launches;
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || a.slices == 1) return e;
+  if (e != cudaSuccess || !split) return e;
   const int64_t row = n_blocks * M * M;
   sigma_dense_sum<<<(unsigned)((2 * row + 255) / 256), 256, 0, s>>>(a.slices, row, a.part, a.Sl, a.Sg, status);
   ++*launches;

@@ -51,3 +51,21 @@ def test_captured_row_is_the_direct_row(kbe, M, n):
     ctx.sync_status()
     assert out[0].abs().max() > 0 and torch.equal(out[0], out[1])
     ctx.close()
+
+
+def test_balanced_rows_stay_whole(kbe):
+    """Rows that fill every SM alike are not split (M = 8: 0.92 of the speed), the
+    rows around them are."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 3 * sms // 2 - 1  # three units per SM
+    ctx = _ctx(kbe, 8, n + 30)
+    L, R = _data(8, n + 29)
+    S = torch.zeros((2, n + 30, 8, 8), dtype=torch.complex128, device="cuda")
+    launches = []
+    for row in (n, n + 10, n // 2):
+        ctx.selfenergy_slice(row, L, R, S[0], S[1])
+        launches.append(ctx.last_launch_count)
+    ctx.sync_status()
+    assert launches == [1, 2, 2]
+    ctx.close()

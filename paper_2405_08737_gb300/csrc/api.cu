@@ -212,12 +212,16 @@ cudaError_t sigma_blocks(kbe_ctx* ctx, int64_t first_block, int64_t n_blocks, in
                          const StepArgs* fock = nullptr) {
   if (ctx->dense) {
     // Self-energy calls of one context may overlap on different streams, so the partial sums of split rows
-    // have a buffer of their own, which the calls take in turn; captured calls add a block's slices in one
-    // unit (a wait for an event of another stream's past would end the capture), with the same sums.
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    cudaError_t e = cudaStreamIsCapturing(s, &capture);
-    const bool split = e == cudaSuccess && capture == cudaStreamCaptureStatusNone && ctx->d_sd;
-    if (e != cudaSuccess) cudaGetLastError();
+    // have a buffer of their own, which the calls that split take in turn; captured calls add a block's slices
+    // in one unit (a wait for an event of another stream's past would end the capture), with the same sums.
+    cudaError_t e = cudaSuccess;
+    bool split = ctx->d_sd && dense_sigma_slices(ctx->M, n_blocks) > 1;
+    if (split) {
+      cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+      e = cudaStreamIsCapturing(s, &capture);
+      split = e == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+      if (e != cudaSuccess) cudaGetLastError();
+    }
     if (split && (e = cudaStreamWaitEvent(s, ctx->sd_done, 0)) != cudaSuccess) return e;
     int k = 0;
     e = launch_sigma_dense(ctx->M, first_block, n_blocks, diag_rel, (const double*)L, (const double*)R, ctx->d_Ut,

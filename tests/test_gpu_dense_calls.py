@@ -69,3 +69,29 @@ def test_balanced_rows_stay_whole(kbe):
     ctx.sync_status()
     assert launches == [1, 2, 2]
     ctx.close()
+
+
+def test_whole_rows_wait_for_no_other_stream(kbe):
+    """A call that needs no workspace runs beside split rows of another stream:
+    it is done before the last of them."""
+    import torch
+    M, n, rows = 16, 255, 50
+    ctx = _ctx(kbe, M, n + 1)
+    L, R = _data(M, n)
+    S = torch.zeros((2, n + 1, M, M), dtype=torch.complex128, device="cuda")
+    T = torch.zeros((2, W.tri_size(rows), M, M), dtype=torch.complex128, device="cuda")
+    ctx.selfenergy_all(rows, L, R, T[0], T[1])
+    assert ctx.last_launch_count == 1  # not split
+    ctx.sync_status()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    done = torch.cuda.Event()
+    for _ in range(20):  # about 10 ms each
+        ctx.selfenergy_slice(n, L, R, S[0], S[1], stream=a)
+        assert ctx.last_launch_count == 2
+    done.record(a)
+    ctx.selfenergy_all(rows, L, R, T[0], T[1], stream=b)
+    b.synchronize()
+    assert not done.query()
+    torch.cuda.synchronize()
+    ctx.sync_status()
+    ctx.close()

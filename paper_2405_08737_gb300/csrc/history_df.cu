@@ -114,7 +114,9 @@ __device__ __forceinline__ void point(const DfArgs& p, Sums& t, int m, int c, in
     }
   }
   if (m > c) return;
-  // term 2 in the band, with the exact weight: w_{c,m} S^s G^A
+  // term 2 in the band, with the exact weight: w_{c,m} S^s G^A.  Four FP64 operations per a, as many
+  // as two weighted values take: they bound the short slices, most of which are band (with S^> - S^< formed
+  // first, which takes two more, M = 16, n = 13 took 44 us instead of 41, M = 64, n = 3 157 instead of 146).
   const int M = p.M;
   const double wcm = p.w.at(c, m);
   float4 ga = cneg(q);
@@ -126,8 +128,9 @@ __device__ __forceinline__ void point(const DfArgs& p, Sums& t, int m, int c, in
   for (int k = 0; k < kNA; ++k) {
     if (k < na) {
       const double2 vl = sl[(int64_t)k * M], vg = sg[(int64_t)k * M];
-      cmac(t.lr[k], t.li[k], c2f(make_double2(wcm * vl.x, wcm * vl.y)), ga);
-      cmac(t.dr[k], t.di[k], c2f(make_double2(wcm * (vg.x - vl.x), wcm * (vg.y - vl.y))), ga);
+      const double2 wl = make_double2(wcm * vl.x, wcm * vl.y);
+      cmac(t.lr[k], t.li[k], c2f(wl), ga);
+      cmac(t.dr[k], t.di[k], c2f(make_double2(fma(wcm, vg.x, -wl.x), fma(wcm, vg.y, -wl.y))), ga);
     }
   }
 }

@@ -284,16 +284,23 @@ __global__ void __launch_bounds__(32 * NA) fx_prep(const __grid_constant__ Args 
         }
       }
     }
-    // (re, im) of a half's variants
-    auto values = [&](int half, int k, int var) -> double2 {
-      const double2 d = make_double2(g[k].x - l[k].x, g[k].y - l[k].y), t = make_double2(l[k].x + g[k].x, l[k].y + g[k].y);
+    double2 v[2][2][2];  // [half][variant][chunk]; FP64 arithmetic bounds this kernel, so once
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
       if (s.adj) {
-        const double2 v = half ? (var ? t : g[k]) : (var ? g[k] : t);
-        return half ? v : make_double2(-v.x, -v.y);
+        const double2 t = make_double2(l[k].x + g[k].x, l[k].y + g[k].y);
+        v[0][0][k] = make_double2(-t.x, -t.y);
+        v[0][1][k] = make_double2(-g[k].x, -g[k].y);
+        v[1][0][k] = g[k];
+        v[1][1][k] = t;
+      } else {
+        const double2 d = make_double2(g[k].x - l[k].x, g[k].y - l[k].y);
+        v[0][0][k] = make_double2(w0[k] * d.x, w0[k] * d.y);
+        v[0][1][k] = make_double2(-w1[k] * l[k].x, -w1[k] * l[k].y);
+        v[1][0][k] = l[k];
+        v[1][1][k] = d;
       }
-      if (half) return var ? d : l[k];
-      return var ? make_double2(-w1[k] * l[k].x, -w1[k] * l[k].y) : make_double2(w0[k] * d.x, w0[k] * d.y);
-    };
+    }
     __syncthreads();
 #pragma unroll
     for (int half = 0; half < 2; ++half)
@@ -302,8 +309,7 @@ __global__ void __launch_bounds__(32 * NA) fx_prep(const __grid_constant__ Args 
         int f[2];
 #pragma unroll
         for (int var = 0; var < 2; ++var) {
-          const double2 v = values(half, k, var);
-          f[var] = max(field64(v.x), field64(v.y));
+          f[var] = max(field64(v[half][var][k].x), field64(v[half][var][k].y));
           if (f[var] == 0x7FF) f[var] = 0;
         }
         if (half) f[0] = f[1] = max(f[0], f[1]);
@@ -316,13 +322,11 @@ __global__ void __launch_bounds__(32 * NA) fx_prep(const __grid_constant__ Args 
     for (int half = 0; half < 2; ++half)
 #pragma unroll
       for (int var = 0; var < 2; ++var) {
-        double2 v[2];
         int ek[2], E = -kNonFinite;
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-          v[k] = values(half, k, var);
           ek[k] = s_ek[half][var][k][lane];
-          const int f = max(field64(v[k].x), field64(v[k].y));
+          const int f = max(field64(v[half][var][k].x), field64(v[half][var][k].y));
           if (f) E = max(E, f == 0x7FF ? kNonFinite : f - ek[k]);
         }
         E = __reduce_max_sync(0xffffffffu, E);
@@ -339,8 +343,9 @@ __global__ void __launch_bounds__(32 * NA) fx_prep(const __grid_constant__ Args 
           if (al == 0 && !(kl & 1))
             x.ek[var][kl >> 1] = (uint32_t)ek[k] | (uint32_t)(kl & 2 ? least >> 8 : least & 0xFF) << 12 | (uint32_t)ek1 << 20;
           // zeros (and subnormals) whatever the exponents
-          const uint64_t br = bytes_of(v[k].x, field64(v[k].x) ? E + ek[k] : kNonFinite),
-                         bi = bytes_of(v[k].y, field64(v[k].y) ? E + ek[k] : kNonFinite);
+          const double2 z = v[half][var][k];
+          const uint64_t br = bytes_of(z.x, field64(z.x) ? E + ek[k] : kNonFinite),
+                         bi = bytes_of(z.y, field64(z.y) ? E + ek[k] : kNonFinite);
 #pragma unroll
           for (int d = 0; d < kDig; ++d) {
             const uint32_t ri = digit_of(d, br, bi);              // (re, im)

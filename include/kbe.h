@@ -615,12 +615,14 @@ kbe_status kbe_batch_step(kbe_batch* b, const int* rows, int P, int precision, v
 kbe_status kbe_batch_set_policy(kbe_batch* b, int block, int item_work_log2);
 kbe_status kbe_batch_get_policy(const kbe_batch* b, int* block, int* item_work_log2);
 
-/* Autotuner: times the persistent history kernel of the batch at `rows`
- * for each candidate policy (block 128 or 256, item_work_log2 = 14, 16, ..,
- * 26; `reps` timed runs after one warm-up, CUDA events on `stream`), keeps
- * the fastest (kbe_batch_set_policy) and returns it with its time in ms.
- * Synchronous.  Overwrites the self-energy rows and history slices of the
- * systems active at `rows`. */
+/* Autotuner: times the persistent FP64 history kernel of the batch at `rows`
+ * over the systems whose slices a step at those rows forms there (the larger
+ * ones go to the tensor cores) for each candidate policy (block 128 or 256,
+ * item_work_log2 = 14, 16, .., 26; `reps` timed runs after one warm-up, CUDA
+ * events on `stream`), keeps the fastest (kbe_batch_set_policy) and returns it
+ * with its time in ms.  Synchronous.  Overwrites the self-energy rows of the
+ * systems active at `rows` and the history slices of those it times.  Without
+ * any such system the policy stays as it is, nothing runs and the time is 0. */
 kbe_status kbe_batch_autotune(kbe_batch* b, const int* rows, int reps, void* stream, int* block_out,
                               int* item_work_log2_out, double* best_ms);
 

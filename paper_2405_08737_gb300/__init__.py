@@ -543,8 +543,9 @@ class Batch:
         return b.value, w.value
 
     def autotune(self, rows, reps=2, stream=None):
-        """Time the candidate tile policies at ``rows``; keep and return the
-        fastest as (block, item_work_log2, ms)."""
+        """Time the candidate tile policies at ``rows`` on the systems whose
+        slices run on the FP64 pipe there; keep and return the fastest as
+        (block, item_work_log2, ms), or the present one and 0 without any."""
         r, p = self._rows(rows)
         b, w, ms = ctypes.c_int(), ctypes.c_int(), ctypes.c_double()
         self._check(lib().kbe_batch_autotune(self._h, p, reps, Context._stream(stream), ctypes.byref(b),

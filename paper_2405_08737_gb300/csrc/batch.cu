@@ -83,7 +83,7 @@ struct BatchDev {
   unsigned long long* counter;
   int* status;
   // FP64 slices on the tensor cores: systems of up to 8 and of more orbitals
-  int use_fx, ctas;
+  int ctas;
   fx::Sys* fx_table[2];
   fx::Head* fx_head;    // [2]
 };
@@ -158,7 +158,7 @@ __global__ void batch_plan(BatchDev b) {
     s.chunk_len = len;
     s.xblk = (int)((outputs + b.block - 1) / b.block);
     elems[i] = outputs;
-    s.fx = b.use_fx && s.fx_work && fx_takes(s.M, n);
+    s.fx = s.fx_work && fx_takes(s.M, n);
     items[i] = s.fx ? 0 : (int64_t)s.xblk * nchunk;
     cost[i] = (double)len * (double)s.M;  // work of one item, up to the common factors
   }
@@ -384,7 +384,7 @@ int slice_paths(const kbe_batch* b, const int* rows) {
   for (int i = 0; i < b->n_sys; ++i) {
     if (rows[i] < 1) continue;
     const BatchSys& y = b->sys[i];
-    mask |= b->dev.use_fx && y.fx_work && fx_takes(y.M, rows[i]) ? (y.M > 8 ? 4 : 2) : 1;
+    mask |= y.fx_work && fx_takes(y.M, rows[i]) ? (y.M > 8 ? 4 : 2) : 1;
   }
   return mask;
 }
@@ -526,7 +526,6 @@ kbe_status kbe_batch_create(kbe_ctx* const* ctxs, int n_sys, kbe_batch** out) {
   b->dev.item_off = reinterpret_cast<int64_t*>(base + o_ioff);
   b->dev.counter = reinterpret_cast<unsigned long long*>(base + o_cnt);
   b->dev.status = reinterpret_cast<int*>(base + o_st);
-  b->dev.use_fx = 1;
   b->dev.ctas = sm_count();
   b->dev.fx_table[0] = reinterpret_cast<fx::Sys*>(base + o_fx8);
   b->dev.fx_table[1] = reinterpret_cast<fx::Sys*>(base + o_fx16);
@@ -754,13 +753,17 @@ kbe_status kbe_batch_autotune(kbe_batch* b, const int* rows, int reps, void* str
   if (e != cudaSuccess) return bcuda(b, e, "kbe_batch_autotune: cudaSetDevice");
   kbe_status st = upload(b);
   if (st != KBE_OK) return st;
+  if (!(slice_paths(b, rows) & 1)) {  // the policy concerns the FP64 pipe's kernel: nothing to choose
+    if (block_out) *block_out = b->dev.block;
+    if (work_out) *work_out = b->dev.item_work_log2;
+    if (best_ms) *best_ms = 0.0;
+    return KBE_OK;
+  }
   cudaStream_t s = (cudaStream_t)stream;
   if ((e = cudaMemcpyAsync((void*)b->dev.rows, rows, sizeof(int) * b->n_sys, cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return bcuda(b, e, "kbe_batch_autotune: rows upload");
-  // the slice of the current state: self-energy rows, then timed history slices
-  // (of every active system: the policy concerns the FP64 pipe's kernel)
+  // the slices of the current state that a step forms there: self-energy rows, then timed history slices
   BatchDev d = b->dev;
-  d.use_fx = 0;
   batch_plan<<<1, 256, (size_t)b->n_sys * 24, s>>>(d);
   batch_rows<kOpSigma><<<sm_count() * 8, 256, 0, s>>>(d);
   cudaEvent_t e0, e1;

@@ -103,9 +103,13 @@ typedef int kbe_status;
 /* Create a context for norb orbitals and at most n_max time points.
  * Allocates device workspace only (split-reduction partials, weight tables,
  * status word); the two-time arrays belong to the caller.
- * The workspace of the FP64 slices on the tensor cores (about 2.1 KB times
- * n_max norb ceil(norb/8)) is optional: without room for it every FP64 slice
- * runs on the FP64 pipe.
+ * Contexts whose longest row (n = n_max - 1) takes its FP64 slice to the tensor
+ * cores also hold that form's workspace: about 2.1 KB n_max norb for norb <= 8,
+ * 4.1 KB n_max norb ceil(norb/16) beyond (digits of the self-energy row), plus 32,
+ * beyond 64, KB per column tile (n_max / floor(128/norb) times ceil(norb/16))
+ * and SM (24 MB at norb = 8, 239 MB at norb = 24, 1.2 GB at norb = 64, n_max =
+ * 1024).  Without room for it every FP64 slice of the context runs on the
+ * FP64 pipe: its low bits then differ from those of a context that has it.
  * KBE_EINVAL: out == NULL, norb < 1, norb > 64, n_max < 1, or sizes that
  * overflow 64-bit block indices.  KBE_ENOMEM / KBE_ECUDA on device errors. */
 kbe_status kbe_create(int norb, int n_max, kbe_ctx** out);

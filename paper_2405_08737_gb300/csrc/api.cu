@@ -746,7 +746,7 @@ kbe_status kbe_create(int norb, int n_max, kbe_ctx** out) {
     return fail(nullptr, e == cudaErrorMemoryAllocation ? KBE_ENOMEM : KBE_ECUDA,
                 std::string("kbe_create: split workspace: ") + cudaGetErrorString(e));
   }
-  if ((int64_t)row > kRunMaxRow) {  // rows that the FP64 slice takes on the tensor cores
+  if (fx_takes(norb, n_max - 1)) {  // the longest row, at least, takes its FP64 slice to the tensor cores
     ctx->fx_bytes = fx_workspace_bytes(norb, n_max);
     if (cudaMalloc(&ctx->d_fx, ctx->fx_bytes) != cudaSuccess || fx_prepare() != cudaSuccess) {
       cudaGetLastError();  // no room: the slice stays on the FP64 pipe

@@ -294,8 +294,9 @@ kbe_status kbe_rhs_row(kbe_ctx* ctx, int j, int precision, const void* L, const 
  * previous step are not encoded again.  A caller that rewrites those rows
  * between steps (a restart into the same buffers) calls kbe_reset_cache.
  * Rows that kbe_run_steps takes in its cooperative launch take it here too,
- * one launch per step (not during a stream capture: there, and where the
- * device refuses it, one launch per kernel). */
+ * one launch per step, unless norb is a multiple of 8 from 24 on (not during a
+ * stream capture: there, and where the device refuses it, one launch per kernel;
+ * the same bits either way). */
 kbe_status kbe_step(kbe_ctx* ctx, int n, int P, int precision, void* L, void* R, void* S_less,
                     void* S_great, void* I_work, void* F_ring, void* stream);
 

@@ -1197,9 +1197,12 @@ kbe_status kbe_step(kbe_ctx* ctx, int n, int P, int precision, void* L, void* R,
   int count = 0;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing((cudaStream_t)stream, &capture) != cudaSuccess) cudaGetLastError();
-  if (coop_steps(ctx, precision) && small_row(ctx, n) && capture == cudaStreamCaptureStatusNone) {
-    // one launch instead of a dozen (steps on the stored history, us: M = 2, n = 30 89 -> 46; M = 4, n = 63
-    // 105 -> 61; M = 8, n = 63 197 -> 185)
+  // One launch instead of a dozen (steps on the stored history, P = 2, us, per kernel / so: M = 2, n = 20 60 /
+  // 41; M = 4, n = 100 103 / 77; M = 8, n = 30 98 / 84).  Where M is a multiple of 8 from 24 on the launches per kernel
+  // are the faster ones for any row (M = 24, n = 3 109 / 121; M = 32, n = 3 133 / 157; M = 40, n = 1 157 / 204; but
+  // M = 26, n = 3 154 / 130; M = 33, n = 2 183 / 166).
+  const bool together = ctx->M < 24 || ctx->M % 8;
+  if (together && coop_steps(ctx, precision) && small_row(ctx, n) && capture == cudaStreamCaptureStatusNone) {
     int next = n;
     st = steps_small(ctx, &next, n, P, L, R, Sl, Sg, I_work, F_ring, (cudaStream_t)stream, false, &count);
   } else {

@@ -147,7 +147,7 @@ def test_df64_of_more_than_32_orbitals(kbe, M, n):
 # first ones), on the FP64 pipe and on the tensor cores
 @pytest.mark.parametrize("M,n,P", [(1, 30, 2), (2, 5, 1), (2, 200, 2), (2, 1023, 2), (3, 60, 3), (4, 63, 2), (4, 255, 2),
                                    (5, 100, 2), (7, 50, 2), (8, 1, 2), (8, 40, 2), (8, 63, 2), (13, 20, 2), (16, 9, 1),
-                                   (16, 15, 2), (32, 3, 2), (45, 1, 2), (8, 64, 2), (8, 140, 2), (17, 20, 2), (24, 30, 1)])
+                                   (16, 15, 2), (24, 5, 2), (26, 3, 2), (32, 3, 1), (32, 3, 2), (45, 1, 2), (8, 64, 2), (8, 140, 2), (17, 20, 2), (24, 30, 1)])
 @pytest.mark.parametrize("precision", ["fp64", "df64"])
 def test_captured_step_is_the_direct_step(kbe, M, n, P, precision):
     """Bitwise: row n, its right-hand side, the self-energy row and the slice.  (FP64:
@@ -174,7 +174,7 @@ def test_captured_step_is_the_direct_step(kbe, M, n, P, precision):
 
     start()
     run.step(n, P=P, precision=precision)
-    small = precision == "fp64" and (n + 1) * M * M <= 4096
+    small = precision == "fp64" and (n + 1) * M * M <= 4096 and (M < 24 or M % 8 != 0)
     assert (ctx.last_launch_count == 1) == small
     direct = result()
     start()

@@ -310,8 +310,8 @@ def cpu_thread_scaling(run, t, order, U, n_s=255):
 def batch_bench(kbe, seed, P, stream, rank=0, world=1):
     """The batching form on 64 independent chains (M in {4,8,12,16,24},
     N_t in [256,1536], U in [0.5,3]): one batched KBE step advances every
-    system at its last row n_i = N_t,i - 1.  Times the plain FP64 path (one
-    kbe_step per system, in sequence), the batched graph in FP64 and with
+    system at its last row n_i = N_t,i - 1.  Times KBE_FP64 (one
+    kbe_step per system, in sequence; the plain_fp64 keys), the batched graph in FP64 and with
     the split-precision contraction, and reports the deviation of the new
     rows from the plain path's.  Histories are the non-interacting
     propagators; the stored right-hand sides are their exact t-derivatives.
@@ -365,7 +365,7 @@ def batch_bench(kbe, seed, P, stream, rank=0, world=1):
     def new_rows():
         return [r.L[W.tri_size(n):W.tri_size(n) + n + 1].clone() for r, n in zip(runs, rows)]
 
-    # plain FP64 path: one kbe_step per system
+    # KBE_FP64 (larger slices on the tensor cores, the others on the FP64 pipe): one kbe_step per system
     plain_launches = 0
     e0.record(stream)
     for r, n in zip(runs, rows):
@@ -462,9 +462,10 @@ def digit_roofline(kernel, M, n, digit_flops, k_avg_ms):
 
 def split_roofline(M, n, k_avg_ms):
     """Of the split contraction: 13 digit pairs x 4 real products x 2 flops
-    per complex multiply-add, (n+1)(3n+2) M^3 of them; the bytes the kernel
-    actually streams are reported beside it."""
-    out = digit_roofline(SPLIT_KERNEL, M, n, 13 * 4 * 2 * (n + 1) * (3 * n + 2) * M ** 3, k_avg_ms)
+    per complex multiply-add, 2 (n+1)^2 M^3 of them (the third product of a
+    history point cancels below the weight band); the bytes the kernel actually
+    streams are reported beside it."""
+    out = digit_roofline(SPLIT_KERNEL, M, n, 13 * 4 * 2 * 2 * (n + 1) ** 2 * M ** 3, k_avg_ms)
     out["streamed_bytes"] = split_stream_bytes(M, n)
     return out
 

@@ -95,8 +95,8 @@ typedef int kbe_status;
                           /* product, compensated sums): about 1e-14 of the   */
                           /* terms' sizes, several times the FP64 pipe's      */
                           /* rate on this part.  Slices of (n+1)^2 norb^3 >=  */
-                          /* 8e6 are formed as for KBE_FP64, which is faster  */
-                          /* there.  Deterministic.                           */
+                          /* 8e6 and (n+1) norb^2 > 4096 are formed as for    */
+                          /* KBE_FP64, which is faster there.  Deterministic. */
 
 /* ---------------------------------------------------------- lifecycle -- */
 
@@ -636,9 +636,9 @@ kbe_status kbe_batch_sync_status(kbe_batch* b, void* stream);
 
 /* ------------------------------------------------ allocation-free entry -- */
 
-/* History slice of row n (the same Eq. KBE2 contraction and kernels as
- * kbe_history_slice, KBE_FP64) for callers that cannot allocate device
- * memory: code that runs inside another framework's memory pool or
+/* History slice of row n (the Eq. KBE2 contraction of kbe_history_slice,
+ * KBE_FP64, with its FP64-pipe kernels at every size) for callers that cannot
+ * allocate device memory: code that runs inside another framework's memory pool or
  * allocator hooks (a nested cudaMalloc there would re-enter the allocator
  * or escape its accounting), or hosts that only hand over fixed buffers.
  * The paper has no counterpart; this entry exists for those callers.

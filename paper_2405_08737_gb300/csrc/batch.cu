@@ -24,7 +24,7 @@
 // instead: batch_fx_plan lists them on the device, and one launch of
 // history_fx.cu's kernels per class (M <= 8, M > 8) contracts all of them, each CTA
 // with an equal share of the chunks.  Ten systems of M = 4..24 and 299..667 points:
-// 221 ms per step on the FP64 pipe, 28.5 ms so.  The graph is captured again only
+// 221 ms per step on the FP64 pipe, 24.1 ms so.  The graph is captured again only
 // when the set of kernels in use changes.
 //
 // Elementwise kernels run grid-stride over the concatenation of all active

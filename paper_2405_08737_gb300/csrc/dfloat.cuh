@@ -257,12 +257,6 @@ __device__ __forceinline__ float4 c2f(double2 v) {
 }
 __device__ __forceinline__ float4 cneg(float4 v) { return make_float4(-v.x, -v.y, -v.z, -v.w); }
 __device__ __forceinline__ float4 cconj(float4 v) { return make_float4(v.x, v.y, -v.z, -v.w); }
-// double-float complex sum (error of order 2^-47 of |a| + |b|)
-__device__ __forceinline__ float4 cadd4(float4 a, float4 b) {
-  const F2 r = add(F2{a.x, a.y}, F2{b.x, b.y});
-  const F2 i = add(F2{a.z, a.w}, F2{b.z, b.w});
-  return make_float4(r.hi, r.lo, i.hi, i.lo);
-}
 // the pair's value in FP64
 __device__ __forceinline__ double acc_value(Acc a) { return (double)a.s + (double)a.c; }
 

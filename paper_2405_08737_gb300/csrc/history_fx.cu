@@ -27,7 +27,7 @@
 // loads share the L1 / shared-memory data pipe (M = 8, n = 1023: issue slots 66%,
 // LSU wavefronts 44%, tensor pipe 17%, DRAM 33%).  With NA = 16 the epilogue holds the MMAs back as well.
 // Measured, in this kernel: the slice n = 1023, M = 8 in 0.82 ms (7.05 on the FP64
-// pipe, history_f64.cu), n = 511, M = 16 in 1.18 ms (14.4).
+// pipe, history_f64.cu), n = 511, M = 16 in 1.19 ms (14.4).
 //
 // One persistent CTA per SM takes a contiguous range of chunks (32 history
 // entries of a 128-row column tile).  A unit is 8 entries, one MMA K step:
@@ -49,7 +49,8 @@
 // 16 an accumulation waits for the epilogue of the one before).
 // One MMA thread instead of two: 0.88 and 1.31 ms for the two slices above.  History
 // loads of far quads as 4 x 16 instead of 2 x 32 bytes pass twice through the data pipe.
-// A row's exponent holds for the units accumulated together in tensor memory.
+// A row's exponent holds for the units accumulated together in tensor memory, and
+// counts its entries as the small operand scales them (Exps in fx_common.cuh).
 // It starts kHeadroom bits above the larger of the unit's and the previous
 // chunk's largest entry; a unit that exceeds it nevertheless closes the
 // accumulation and starts the next with the larger exponent.  A row that had

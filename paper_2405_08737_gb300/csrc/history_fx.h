@@ -6,20 +6,26 @@
 
 namespace kbe {
 
-// Whether an FP64 slice is better there than on the FP64 pipe: from (n + 1)^2 M^3 =
+// Whether an FP64 slice goes there instead of the FP64 pipe: from (n + 1)^2 M^3 =
 // 5e6 on, and never for the rows that kbe_run_steps takes in its cooperative
-// kernel.  Below that the FP64 pipe is as fast or faster, above it falls behind
-// with the cube of M (slices on the FP64 pipe against the tensor cores, us: M = 5,
-// n = 163 95 / 87; M = 8, n = 64 89 / 66, n = 1023 7080 / 905; M = 12, n = 29 63 / 91,
-// n = 50 107 / 130; M = 16, n = 16 55 / 84, n = 30 102 / 89; M = 24, n = 10 68 / 100,
-// n = 20 159 / 138; M = 32, n = 16 249 / 140).
+// kernel.  Above the line the tensor cores are faster at every M (FP64 pipe / tensor cores,
+// us: M = 3, n = 456 127 / 70; M = 5, n = 200 119 / 64; M = 8, n = 98 108 / 64, n = 1023 7050 / 835;
+// M = 9, n = 85 156 / 82; M = 13, n = 47 135 / 92; M = 16, n = 34 129 / 82; M = 24, n = 19 156 / 84;
+// M = 33, n = 11 163 / 86; M = 64, n = 4 222 / 84).  They cross below it, between 1.5e6
+// and 3e6 (M = 8, n = 65 92 / 56; M = 12, n = 30 62 / 69, n = 40 88 / 79; M = 16, n = 17 56 / 69,
+// n = 24 78 / 70; M = 24, n = 10 68 / 72): the line was measured with an earlier form
+// of these kernels, and rows in between pay up to two thirds more than they had to.
+// The adjoint's line is the slice's (n at 5e6: M = 5 170 / 92, M = 8 131 / 82, M = 16 184 /
+// 117, M = 33 277 / 163; crossing near 2e6: M = 12, n = 30 102 / 104, M = 24, n = 10 111 / 120).
 __host__ __device__ inline bool fx_takes(int M, int n) {
   const double N = n + 1.0, m = M;
   return N * m * m > kRunMaxRow && N * N * m * m * m >= 5e6;
 }
 // The same for KBE_DF64 slices against their own kernel (history_df.cu): from
-// 8e6 on (us, double-float / tensor cores: M = 8, n = 100 111 / 77; M = 16, n = 30 74 /
-// 89, n = 511 4620 / 1350; M = 24, n = 20 114 / 138; M = 32, n = 16 168 / 140).
+// 8e6 on (us, double-float / tensor cores: M = 5, n = 260 152 / 73; M = 8, n = 130 132 / 68;
+// M = 13, n = 60 115 / 99; M = 16, n = 50 127 / 84; M = 33, n = 18 218 / 122).  They cross between
+// 2e6 and 6e6 (M = 8, n = 65 72 / 56; M = 9, n = 60 68 / 78, n = 85 99 / 82; M = 13, n = 47 81 / 92;
+// M = 16, n = 30 68 / 76, n = 34 90 / 82; M = 24, n = 14 72 / 80, n = 19 99 / 84).
 __host__ __device__ inline bool fx_takes_df(int M, int n) {
   const double N = n + 1.0, m = M;
   return N * m * m > kRunMaxRow && N * N * m * m * m >= 8e6;

@@ -235,13 +235,15 @@ static int max_slices(int M) { return M >= 8 ? std::min(8, M * M / tiling(M).g) 
 // also hides latency (M = 8, n = 75, two per SM: 150 -> 110 us).  From three on, where the
 // last round leaves less than a twentieth idle, a block's second staging costs the smaller M more
 // than it gives (whole / sliced, us: M = 8, n = 227 299 / 327, n = 455 597 / 623, M = 9, n = 303 847 /
-// 887, M = 11, n = 227 1573 / 1577; M = 12, n = 227 2847 / 2625, M = 16, n = 303 12.63 / 12.36 ms).
+// 887, M = 11, n = 227 1573 / 1577; M = 12, n = 227 2847 / 2625, M = 16, n = 303 12.63 / 12.36 ms); from
+// eight on a fiftieth (M = 8, n = 900, 0.99 busy, 1169 / 1209, n = 1100, 0.97 busy, 1456 / 1412).
 // Blocks of M < 8 take microseconds and are left whole.  The number depends on
 // the sizes alone, so that results do not depend on how a call is run.
 int dense_sigma_slices(int M, int64_t n_blocks) {
   const int64_t units = 2 * n_blocks, sms = sm_count(), rounds = (units + sms - 1) / sms;
   if (units >= unit_cap()) return 1;
-  if (M < 12 && rounds >= 3 && 20 * units >= 19 * rounds * sms) return 1;
+  const int64_t idle = rounds < 8 ? 20 : 50;
+  if (M < 12 && rounds >= 3 && idle * units >= (idle - 1) * rounds * sms) return 1;
   return (int)std::min<int64_t>((unit_cap() + units - 1) / units, max_slices(M));
 }
 

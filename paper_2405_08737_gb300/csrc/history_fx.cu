@@ -24,7 +24,7 @@
 // ones.  What bounds it then is the conversion: every history entry is read in
 // both orientations and cut into digits with about 30 integer instructions per
 // real, and the digit stores (64 KB a unit), the MMA operand reads and the history
-// loads share the L1 / shared-memory data pipe (M = 8, n = 1023: issue slots 66%,
+// loads share the L1 / shared-memory data pipe (M = 8, n = 1023: issue slots 70%,
 // LSU wavefronts 44%, tensor pipe 17%, DRAM 33%).  With NA = 16 the epilogue holds the MMAs back as well.
 // Measured, in this kernel: the slice n = 1023, M = 8 in 0.82 ms (7.05 on the FP64
 // pipe, history_f64.cu), n = 511, M = 16 in 1.19 ms (14.4).

@@ -75,9 +75,11 @@ typedef int kbe_status;
                           /* |Sigma(n,m)_ax| |G(m,c)_xb| met there and in the */
                           /* 32 entries before: a bound by orbital column b,  */
                           /* not by output entry, unless the rows a of Sigma  */
-                          /* differ by a factor each.  kbe_history_slice_     */
-                          /* noalloc and kbe_history_slice_band over part of  */
-                          /* the rows sum each product in FP64                */
+                          /* differ by a factor each.  History values below   */
+                          /* 2^-958 count with fewer bits there, below 2^-1020 */
+                          /* with none.  kbe_history_slice_noalloc and        */
+                          /* kbe_history_slice_band over part of the rows sum */
+                          /* each product in FP64                             */
 #define KBE_SPLIT_BF16 1  /* the contraction on the 16-bit-float tensor cores */
                           /* with error-free 4-digit fixed-point splitting:   */
                           /* every value becomes round(v 2^(31-e)) in base-256 */

@@ -107,7 +107,7 @@ extern "C" kbe_status kbe_history_slice_noalloc(int norb, int n, const double* t
   const int MM = norb * norb;
   const size_t row = (size_t)(n + 1) * MM;          // complex entries per s
   const size_t wdoubles = (size_t)n_t * (kMaxOrder + 2) + 64;  // wbar + band (+ status, padding)
-  // the prep buffers (3 complex rows) must fit next to the weight tables
+  // room for 3 complex rows next to the weight tables (the prep buffers are 2 of them)
   if (wdoubles + 6 * row > kScratchDoubles)
     return fail(KBE_EINVAL, "kbe_history_slice_noalloc: (n+1)*norb^2 exceeds the 64 MiB scratch "
                             "(at most about 1.37e6 complex entries per row)");

@@ -527,12 +527,15 @@ kbe_status kbe_reset_cache(kbe_ctx* ctx);
 kbe_status kbe_sync_status(kbe_ctx* ctx, void* stream);
 
 /* Test support for the device-side failure path (no fault is involved):
- * the next split-precision contraction launched on this context (by
- * kbe_history_slice, kbe_step, ... with KBE_SPLIT_BF16) issues no copy for
- * its work unit `unit` (a unit is one column tile of 128 / norb output
- * columns times one chunk of 16 history entries; the persistent CTA that
- * owns it stops producing there), and every wait of its pipeline gives up
- * after spin_limit polls (instead of about 2^26).  The consumers' bounded
+ * the next tensor-core contraction of a history slice launched on this
+ * context (by kbe_history_slice, kbe_step, ... with KBE_SPLIT_BF16, or with
+ * KBE_FP64 or KBE_DF64 for a slice that these form there) issues no copy for
+ * its work unit `unit` (split: a unit is one column tile of 128 / norb output
+ * columns times one chunk of 16 history entries, and the persistent CTA that
+ * owns it stops producing there; FP64: the unit of 8 history entries with
+ * that number in every CTA), and every wait of its pipeline gives up
+ * after spin_limit polls (split: instead of about 2^26; FP64: after 256
+ * spin_limit clocks instead of 2^31).  The consumers' bounded
  * waits run out, every CTA of the launch finishes the copies and MMAs it
  * had already issued, frees its tensor memory and returns, and
  * kbe_sync_status reports KBE_ETIMEOUT; the slice's output is then

@@ -181,6 +181,12 @@ kbe_status history(kbe_ctx* ctx, int n, int precision, const void* L, const void
   HistoryArgs a{ctx->M, n, (const double*)L, (const double*)R, (const double*)Sl, (const double*)Sg,
                 weights_view(ctx), (double*)I_out, ctx->d_part, ctx->part_bytes, ctx->d_status};
   cudaError_t e;
+  if (precision == KBE_FP64 ? use_fx(ctx, n) : ctx->d_fx && fx_takes_df(ctx->M, n)) {
+    a.withhold = ctx->dbg_withhold;
+    a.spin_limit = ctx->dbg_spin;
+    ctx->dbg_withhold = -1;  // one launch only
+    ctx->dbg_spin = 0;
+  }
   if (precision == KBE_DF64) {
     if (!next_events(ctx, &a.ev_begin, &a.ev_end)) return fail(ctx, KBE_ECUDA, "profiling: cudaEventCreate");
     e = ctx->d_fx && fx_takes_df(ctx->M, n) ? launch_history_fx(a, ctx->d_fx, ctx->fx_bytes, s, launches)

@@ -151,6 +151,7 @@ struct Regs {
   static_assert(256 * kEpi + 512 * kConv + 128 * kMisc == kThreads * 72, "register split");
 };
 
+
 template <int NA>
 struct Smem {
   uint8_t stage[kStages][2 * kPlane];
@@ -172,6 +173,8 @@ struct Args {
   const Sys* table;
   const Head* head;
   int G;
+  int withhold;           // failure-path test: the unit of each CTA that its producer does not supply
+  long long wait_cycles;  // and the length of its waits (0: no test)
 };
 __device__ __forceinline__ const Sys& sys_at(const Args& a, int i) { return a.table ? a.table[i] : a.one; }
 __device__ __forceinline__ const Head& head_of(const Args& a) { return a.table ? *a.head : a.one_head; }
@@ -191,7 +194,7 @@ __device__ __forceinline__ WeightsView weights_of(const Sys& s) { return Weights
 __device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Waits for a phase of a barrier, suspended by the hardware between polls.
-// Gives up after kWaitCycles, or when another role has.
+// Gives up after kWaitCycles (kTest: the launch's own), or when another role has.
 __device__ __forceinline__ bool try_suspend(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -201,11 +204,12 @@ __device__ __forceinline__ bool try_suspend(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ bool wait_bar(int* abort, uint64_t* bar, uint32_t parity, int* status) {
+template <bool kTest>
+__device__ __forceinline__ bool wait_bar(const Args& a, int* abort, uint64_t* bar, uint32_t parity, int* status) {
   if (try_suspend(bar, parity)) return true;
   const long long t0 = clock64();
   while (!try_suspend(bar, parity)) {
-    const bool late = clock64() - t0 > kWaitCycles;
+    const bool late = clock64() - t0 > (kTest ? a.wait_cycles : kWaitCycles);
     if (late || *(volatile int*)abort) {
       if (late) { atomicOr(status, kStatusTimeout); *(volatile int*)abort = 1; }
       return false;
@@ -544,7 +548,9 @@ __device__ __forceinline__ void fold(double (&s)[NA], uint32_t at, int E, int ha
 }
 
 // ---------------------------------------------------------------- main ---
-template <int NA, bool kQuad>
+// kTest: a launch whose producers stop at a unit (kbe_debug_withhold_split), an instantiation of its own (with the
+// unit and the cycles read from the arguments the slice n = 1023, M = 8 took 858 us instead of 834).
+template <int NA, bool kQuad, bool kTest = false>
 __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ Args a) {
   using C = Cfg<NA>;
   constexpr int kN = C::kN, kBufs = C::kBufs, kBufCols = C::kBufCols;
@@ -594,7 +600,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
     for (int from = 0;;) {      // thread 0's message, or its sum and then thread 1's
       const unsigned k = from ? used[1]++ : used[0]++;
       const int buf = 2 * (k % (kBufs / 2)) + from;
-      if (!__all_sync(0xffffffffu, wait_bar(&sm.abort, &sm.accfull[buf], (k / (kBufs / 2)) & 1, status))) break;
+      if (!__all_sync(0xffffffffu, wait_bar<kTest>(a, &sm.abort, &sm.accfull[buf], (k / (kBufs / 2)) & 1, status))) break;
       tc_fence_after();
       const Post& ps = sm.post[buf];
       const int type = ps.type;
@@ -654,7 +660,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       Desc ds;
       do {
         const int b = d % kBSlots;
-        if (!__all_sync(0xffffffffu, wait_bar(&sm.abort, &sm.bfull[b], (d / kBSlots) & 1, status))) return false;
+        if (!__all_sync(0xffffffffu, wait_bar<kTest>(a, &sm.abort, &sm.bfull[b], (d / kBSlots) & 1, status))) return false;
         ds = sm.desc[b];
         ++d;
       } while (kind_of(ds.flags) == kFlush || kind_of(ds.flags) == kScale);
@@ -719,7 +725,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
         }
       }
       more = load();  // in flight while this unit's digits are written
-      if (!__all_sync(0xffffffffu, wait_bar(&sm.abort, &sm.empty[s], ((u / kStages) & 1) ^ 1, status))) break;
+      if (!__all_sync(0xffffffffu, wait_bar<kTest>(a, &sm.abort, &sm.empty[s], ((u / kStages) & 1) ^ 1, status))) break;
       if (__any_sync(0xffffffffu, raised) && lane == 0) *(volatile unsigned*)&sm.raise[s] = u + 1;
       if (q == 0) sm.erow[u % kExpRing][plane][8 * wq + (lane & 7)] = (int16_t)E;
       uint8_t* dst = sm.stage[s] + dst0;
@@ -740,7 +746,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       // the next slot, its descriptor written; false when the wait ran out
       auto put = [&](int kap, int c0, int flags, int aux) -> bool {
         const int b = d % kBSlots;
-        if (!wait_bar(&sm.abort, &sm.bempty[b], ((d / kBSlots) & 1) ^ 1, status)) return false;
+        if (!wait_bar<kTest>(a, &sm.abort, &sm.bempty[b], ((d / kBSlots) & 1) ^ 1, status)) return false;
         sm.desc[b] = Desc{kap, c0, flags, aux};
         return true;
       };
@@ -758,6 +764,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
         walk_to(w, *S, si, q0 - S->unit_base);
         int fresh = kFresh | kNewTile, cls = -1;
         bool scaled = false, joined = false;
+        int units = 0;
         while (q < q1 && !stop) {
           if (w.cls != cls) fresh |= kFresh;
           if (S->adj && !scaled && w.cls == kBand && w.j0 < w.j1) {
@@ -772,6 +779,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
           const uint8_t* src = S->small + (w.cls == kBand ? C::kHalfBytes : 0) +
                                ((size_t)w.kc * kChunkUnits * S->parts + w.part) * C::kSmallBytes;
           for (int unit = w.j0; unit < w.j1; ++unit) {
+            if (kTest && units++ == a.withhold) { stop = true; break; }
             const int flags = (w.cls == kNear ? kFlagNear : 0) | (w.cls == kBand ? kFlagBand : 0) |
                               (unit == w.j0 && !joined ? kFirst : 0) | (unit + 1 == w.j1 && !join ? kLast : 0) |
                               (S->adj ? kFlagLow : 0) | min(NA, S->M - w.part * NA) << 16;
@@ -829,7 +837,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
         buf = 2 * (k % (kBufs / 2)) + me;
       };
       auto wait_buffer = [&]() {
-        return wait_bar(&sm.abort, &sm.accempty[buf], ((k / (kBufs / 2)) & 1) ^ 1, status);
+        return wait_bar<kTest>(a, &sm.abort, &sm.accempty[buf], ((k / (kBufs / 2)) & 1) ^ 1, status);
       };
       auto close = [&]() {
         sm.post[buf].eidx = (u - 1) % kExpRing;
@@ -854,7 +862,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
       };
       for (unsigned d = 0; !stop; ++d) {
         const int b = d % kBSlots;
-        if (!wait_bar(&sm.abort, &sm.bfull[b], (d / kBSlots) & 1, status)) { stop = true; break; }
+        if (!wait_bar<kTest>(a, &sm.abort, &sm.bfull[b], (d / kBSlots) & 1, status)) { stop = true; break; }
         const Desc ds = sm.desc[b];
         const int kind = kind_of(ds.flags);
         if (kind == kEnd) break;
@@ -868,7 +876,7 @@ __global__ void __launch_bounds__(kThreads, 1) fx_main(const __grid_constant__ A
         }
         const int s = u % kStages;
         const bool near = ds.flags & kFlagNear, band = ds.flags & kFlagBand;
-        if (!wait_bar(&sm.abort, &sm.full[s], (u / kStages) & 1, status)) { stop = true; break; }
+        if (!wait_bar<kTest>(a, &sm.abort, &sm.full[s], (u / kStages) & 1, status)) { stop = true; break; }
         for (int i = 0; i < kBSlots && held; ++i)
           if (held >> i & 1u) {
             mbar_arrive(&sm.bempty[i]);
@@ -962,7 +970,12 @@ cudaError_t enqueue(const Args& a, bool quad, unsigned prep_blocks, unsigned red
   cudaError_t e = launch_overlapped(fx_prep<NA>, prep_blocks, 32 * NA, 0, st, a);
   if (e != cudaSuccess) return e;
   ++*launches;
-  if (ev_begin) {  // timed: no overlap with the kernels around it
+  if (a.wait_cycles) {
+    if (ev_begin) cudaEventRecord(ev_begin, st);
+    fx_main<NA, false, true><<<a.G, kThreads, sizeof(Smem<NA>), st>>>(a);
+    e = cudaGetLastError();
+    if (ev_end) cudaEventRecord(ev_end, st);
+  } else if (ev_begin) {  // timed: no overlap with the kernels around it
     cudaEventRecord(ev_begin, st);
     if (quad) fx_main<NA, true><<<a.G, kThreads, sizeof(Smem<NA>), st>>>(a);
     else fx_main<NA, false><<<a.G, kThreads, sizeof(Smem<NA>), st>>>(a);
@@ -980,7 +993,8 @@ cudaError_t enqueue(const Args& a, bool quad, unsigned prep_blocks, unsigned red
 
 // One system's contraction in its workspace.
 cudaError_t launch_one(Sys s, int M, int n, int band_w, int adj, void* work, size_t work_bytes, cudaStream_t st,
-                       int* launches, cudaEvent_t ev_begin, cudaEvent_t ev_end) {
+                       int* launches, cudaEvent_t ev_begin, cudaEvent_t ev_end, long long withhold = -1,
+                       long long spin_limit = 0) {
   *launches = 0;
   if (M < 1 || M > kMaxNorb || n < 0) return cudaErrorInvalidValue;
   const int NA = part_rows(M);
@@ -995,6 +1009,10 @@ cudaError_t launch_one(Sys s, int M, int n, int band_w, int adj, void* work, siz
   a.G = (int)std::min<long long>(a.one_head.total, sm_count());
   if (small_bytes(s, NA) + ((size_t)s.tiles + a.G) * slot_complex(NA) * 16 > work_bytes) return cudaErrorInvalidValue;
   a.one = s;
+  if (withhold >= 0) {
+    a.withhold = (int)std::min<long long>(withhold, 1 << 30);
+    a.wait_cycles = 256 * std::min<long long>(spin_limit, kWaitCycles / 256);
+  }
   cudaError_t e = fx_prepare();
   if (e != cudaSuccess) return e;
   const unsigned prep = (unsigned)std::min<long long>(a.one_head.chunks, 1 << 30);
@@ -1028,6 +1046,8 @@ cudaError_t fx_prepare() {
   if (e == cudaSuccess) e = set((const void*)fx_main<8, false>, sizeof(Smem<8>));
   if (e == cudaSuccess) e = set((const void*)fx_main<16, true>, sizeof(Smem<16>));
   if (e == cudaSuccess) e = set((const void*)fx_main<16, false>, sizeof(Smem<16>));
+  if (e == cudaSuccess) e = set((const void*)fx_main<8, false, true>, sizeof(Smem<8>));
+  if (e == cudaSuccess) e = set((const void*)fx_main<16, false, true>, sizeof(Smem<16>));
   if (e == cudaSuccess) done_mask.fetch_or(bit);
   return e;
 }
@@ -1043,7 +1063,8 @@ cudaError_t launch_history_fx(const HistoryArgs& h, void* work, size_t work_byte
   s.out0 = h.out;
   s.out1 = h.out + 2 * (size_t)(h.n + 1) * h.M * h.M;
   s.status = h.status;
-  return launch_one(s, h.M, h.n, h.w.band_w, 0, work, work_bytes, st, launches, h.ev_begin, h.ev_end);
+  return launch_one(s, h.M, h.n, h.w.band_w, 0, work, work_bytes, st, launches, h.ev_begin, h.ev_end, h.withhold,
+                    h.spin_limit);
 }
 
 cudaError_t launch_fx_table(int NA, bool quad, const Sys* table, const Head* head, cudaStream_t st, int* launches) {

@@ -233,6 +233,8 @@ struct HistoryArgs {
   cudaEvent_t ev_end = nullptr;
   int band_lo = 0;                 // contributions of the stored rows [band_lo, band_hi) only
   int band_hi = 0x7fffffff;
+  long long withhold = -1;         // failure-path test of launch_history_fx (kbe_debug_withhold_split)
+  long long spin_limit = 0;
 };
 // FP64 history slice; sets *launches to the number of kernels enqueued.
 cudaError_t launch_history_f64(const HistoryArgs& a, cudaStream_t s, int* launches);
